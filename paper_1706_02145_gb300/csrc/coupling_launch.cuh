@@ -73,45 +73,51 @@ constexpr int kGenericRPB = 64;
 // FP64_UNROLLED: 1 = compile-time FP64 kernel, 0 = runtime-table FP64 kernel
 // Algorithmic flops per ordered sphere pair and RHS of the rotation-
 // translation-rotation evaluation, counted from the same compile-time tables
-// the kernel uses (FMA = 2 flops, complex multiply = 6, complex MAC = 8):
-//   z-rotation of x+- (2 NH complex multiplies), Wigner-d entries (monomials
-//   and one FMA per term, evaluated twice), forward and backward block
-//   rotations (8 flops per R entry each), axial build (4 flops per term plus 4
-//   for the W+- combination per (mu >= 0, l, l') block), axial apply (2 complex
-//   MACs per (mu, l, l')), output phase (2 NH complex MACs), h_p recurrence.
+// the kernel uses (an FMA is 2 flops), in the cosine / sine basis:
+//   turning by M phi: 2 products and 2 FMAs, forward, or 4 FMAs, backward, per
+//   (l, M > 0), tau and part; cos / sin of q theta and m phi and the entries of
+//   the rotation blocks, one FMA per term (both evaluated twice); the blocks
+//   themselves, 2 flops per entry, tau and part, forward and backward; axial
+//   entries (4 flops per term, plus 4 for A +- iB at mu > 0) formed once per
+//   (mu >= 0, l <= l'), applied to both rows (a complex MAC is 8); the sums
+//   c +- s before and after, 4 complex additions per (l, mu > 0) each; the h_p
+//   recurrence.
 // f(integral_constant<l>) for l = 1 .. sizeof...(I)
 template <typename F, int... I>
 void for_each_degree(F&& f, std::integer_sequence<int, I...>) {
   (f(std::integral_constant<int, I + 1>{}), ...);
 }
+template <int l, int KIND, int MU, int... MI>
+long long rot_terms_row(std::integer_sequence<int, MI...>) {
+  return (0LL + ... + (rtr::RotEntry<l, KIND, MU, MI + KIND>::unit() ? 0 : rtr::RotEntry<l, KIND, MU, MI + KIND>::terms()));
+}
+template <int l, int... MUI>
+long long rot_terms(std::integer_sequence<int, MUI...>) {
+  return (0LL + ... + (rot_terms_row<l, 0, MUI>(std::make_integer_sequence<int, MUI + 1>{}) +
+                       rot_terms_row<l, 1, MUI>(std::make_integer_sequence<int, MUI>{})));
+}
 
 template <int L>
 long long rtr_flops_per_pair_t() {
-  long long f = 0;
-  constexpr int NH = L * (L + 2);
-  f += 2LL * NH * 6;                                   // e^{i m phi} x+-
-  f += 2LL * (4 * L - 2) + 8;                          // h_p recurrence and start
-  long long rot = 0, dm = 0;
+  long long f = 2LL * (4 * L - 2) + 8;  // h_p recurrence and start
+  f += 2LL * 2 * 6 * (L - 1);           // cos / sin of q theta and m phi, twice
   auto per_l = [&](auto LL_) {
     constexpr int l = decltype(LL_)::value;
-    rot += 8LL * (2 * l + 1) * (2 * l + 1);
-    dm += (2 * l + 1) + 2LL * rtr::DTab<l>::value.off[rtr::DTab<l>::value.ncanon];
+    f += 4LL * l * (6 + 8);                                         // turning by M phi
+    f += 2LL * 2 * rot_terms<l>(std::make_integer_sequence<int, l + 1>{});  // entries of C and S
+    f += 2LL * 8 * (2 * l * l + 2 * l + 1 - (l == 1 ? 1 : 0));      // their products (S of degree 1 is +-1)
+    f += 2LL * 8 * l;                                               // c +- s
   };
   for_each_degree(per_l, std::make_integer_sequence<int, L>{});
-  f += 2 * rot + 2 * dm;
-  // axial entries: with the transpose symmetry only the entries lo <= li are
-  // formed; every entry is applied to both rows
-  constexpr bool sym = rtr::Config<L, float>::SYM_AXIAL;
   for (int mu = 0; mu <= L; ++mu) {
     for (int lo = (mu > 1 ? mu : 1); lo <= L; ++lo) {
       for (int li = (mu > 1 ? mu : 1); li <= L; ++li) {
         const rtr::AxialRow<L> a = rtr::make_axial<L>(mu, lo, li);
-        if (!sym || lo <= li) f += 4LL * (a.na + a.nb) + 4;
+        if (lo <= li) f += 4LL * (a.na + a.nb) + (mu > 0 ? 4 : 0);
         f += (mu > 0 ? 2 : 1) * 16LL;
       }
     }
   }
-  f += 2LL * NH * 8;                                   // output phase and accumulate
   return f;
 }
 

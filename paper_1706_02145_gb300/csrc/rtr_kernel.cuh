@@ -1,17 +1,31 @@
 // Coupling matvec y_i = sum_{j != i} W^{ij} x_j by rotation-translation-
 // rotation (see rtr_tables.cuh for the factorisation W = D^H W_z D).
 //
-// Per ordered pair (i, j), one thread (the receiver's):
+// Per ordered pair (i, j), one thread (the receiver's), with the sources held
+// in the cosine / sine basis of rtr_tables.cuh (c_M and s_M of each tau):
 //   1. geometry: k|d| and its phase (FP32 kernel: float-float arithmetic;
-//      FP64 kernel: FP64), h_p(k|d|), cos/sin(theta/2), e^{i m phi}
-//   2. x'+-[l, mu] = sum_m R^l_{mu m}(theta) e^{i m phi} x+-[l, m]
-//   3. y'+-[l, mu] = sum_{l'} (A_z +- i B_z)[l, l', mu] x'+-[l', mu]
-//      (built once for mu >= 0 and reused, B sign flipped, for -mu)
-//   4. y+-[l, m] += e^{-i m phi} sum_mu R^l_{mu m}(theta) y'+-[l, mu]
-// with x+- = x_1 +- x_2 (the tau structure [[A, B], [B, A]] of W, App. A.2).
-// All coefficients (Wigner-d sums, axial a5/b5 terms) are compile-time
+//      FP64 kernel: FP64), h_p(k|d|), cos / sin of q theta and m phi
+//   2. (c_M, s_M) turned by M phi, then c'_mu = sum_M C_{mu M} c_M and
+//      s'_mu = sum_M S_{mu M} s_M per degree l and tau
+//   3. the axial products: for mu > 0 the sums c1 +- s2 and c2 +- s1 see only
+//      A + iB or A - iB, so each entry is one complex number per sum
+//   4. the same C and S (symmetric, their own inverses), turned back by M phi,
+//      added to the receiver's sums
+// All coefficients (rotation blocks, axial a5/b5 terms) are compile-time
 // immediates; one code stream serves every warp.  Per pair the thread does
-// O(L^3) work instead of the O(L^4) of the direct per-entry evaluation.
+// O(L^3) work instead of the O(L^4) of the direct per-entry evaluation.  The
+// real basis halves the rotations' products (2 l^2 + 2 l + 1 per degree
+// against (2 l + 1)^2) and makes every number of steps 2 and 4 real, so that
+// (re, im) travel together through the packed two-lane FMA.
+//
+// Bound by FP32 (FP64) issue; memory traffic is a few MB per product.  In the
+// cosine / sine basis a pair costs 4 448 flops at lmax 4 (5 728 with complex
+// rotations of all 2 l + 1 orders), 2 248 at lmax 3, 7 780 at lmax 5, and the
+// entries of the rotation blocks need no half-angle powers.  Measured on
+// GB300, master product, before -> after: FP32 N = 10 000 lmax 4 9.87 -> 7.71
+// ms (error against 64 bits 6.0e-7 -> 3.2e-7), N = 777 lmax 5 with 8 right-hand
+// sides 2.27 -> 1.11 ms, N = 100 000 lmax 3 492 -> 395 ms; FP64 N = 2001 lmax 4
+// 22.9 -> 17.5 ms.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -25,30 +39,38 @@
 namespace celes {
 namespace rtr {
 
-// FP32 rotations (steps 2 and 4) on the packed two-lane FMA of sm_100+
-// (__ffma2_rn, per lane the rounding of fmaf: results are bit-identical to the
-// scalar form).  It halves the issue slots of the rotations, which dominate
-// the instruction stream: N = 10 000 matvec 12.4 -> 10.4 ms at lmax 4, 5.65 ->
-// 5.17 ms at lmax 3.  At lmax 5 ptxas then moves the rotated coefficients to
-// the stack (8.7 vs 4.1 ms at N = 4000), so lmax 5 keeps the scalar form.
-template <int L, typename R>
-constexpr bool kPacked = std::is_same<R, float>::value && L <= 4;
-// launch-shape option bits of the pair code: 1 = the x+ phase multiply on the
-// packed FMA, 2 = packed rotations at every lmax (lmax 5 with x' and y' in
-// shared memory has the registers for them)
-template <int L, typename R, int OPT>
-constexpr bool kPackedRot = std::is_same<R, float>::value && (L <= 4 || (OPT & 2) != 0);
-
 template <typename R>
 struct alignas(4 * sizeof(R)) Quad4 {
   R x, y, z, w;
 };
 
-template <int L, typename R>
-struct Geom {
-  R hre[2 * L + 1], him[2 * L + 1];
-  R cp[2 * L + 1], sp[2 * L + 1];  // powers of cos(theta/2), sin(theta/2)
-  R ere[L + 1], eim[L + 1];
+// a complex value whose two parts take the same real factors
+template <typename R>
+struct C2 {
+  R x, y;
+};
+// w b + c and w b for a real w: FP32 on the packed two-lane FMA of sm_100+
+// (per lane the rounding of fmaf), which halves the issue slots of the
+// rotations while the scalar FMAs of the axial step fill the other half of the
+// FP32 lanes
+__device__ __forceinline__ C2<float> fma2(float w, C2<float> b, C2<float> c) {
+  const float2 r = __ffma2_rn(make_float2(w, w), make_float2(b.x, b.y), make_float2(c.x, c.y));
+  return C2<float>{r.x, r.y};
+}
+__device__ __forceinline__ C2<float> mul2(float w, C2<float> b) {
+  const float2 r = __fmul2_rn(make_float2(w, w), make_float2(b.x, b.y));
+  return C2<float>{r.x, r.y};
+}
+__device__ __forceinline__ C2<double> fma2(double w, C2<double> b, C2<double> c) {
+  return C2<double>{fma_(w, b.x, c.x), fma_(w, b.y, c.y)};
+}
+__device__ __forceinline__ C2<double> mul2(double w, C2<double> b) { return C2<double>{w * b.x, w * b.y}; }
+
+// the scalars of one pair that every table derives from
+template <typename R>
+struct GeomS {
+  R ix, sn, cs;        // 1/(k d), sin(k d), cos(k d)
+  R ct, st, cph, sph;  // cos/sin theta, cos/sin phi of d
 };
 
 // ---- FP32 pair geometry without FP64 arithmetic ----------------------------
@@ -111,48 +133,47 @@ __device__ __forceinline__ void sincos_quadrant(float y, int iq, float& s, float
   c = ((iq + 1) & 2) ? -c0 : c0;
 }
 
+// h_p(k d), p = 0..2L (closed forms of h_0, h_1 and upward recurrence)
 template <int L, typename R>
-__device__ __forceinline__ void geometry_angles_t(R ct, R st, R cph, R sph, Geom<L, R>& g);
-template <int L>
-__device__ __forceinline__ void geometry_angles(float ct, float st, float cph, float sph, Geom<L, float>& g) {
-  geometry_angles_t<L, float>(ct, st, cph, sph, g);
-}
-
-// the few scalars every table of a pair derives from
-struct GeomS {
-  float ix, sn, cs;        // 1/(k d), sin(k d), cos(k d)
-  float ct, st, cph, sph;  // cos/sin theta, cos/sin phi of d
+struct Hankel {
+  R re[2 * L + 1], im[2 * L + 1];
+  __device__ __forceinline__ explicit Hankel(const GeomS<R>& q) {
+    const R ix = q.ix, sn = q.sn, cs = q.cs;
+    re[0] = sn * ix;
+    im[0] = -cs * ix;
+    re[1] = -ix * fma_(-sn, ix, cs);
+    im[1] = -ix * fma_(cs, ix, sn);
+#pragma unroll
+    for (int p = 1; p < 2 * L; ++p) {
+      const R c = static_cast<R>(2 * p + 1) * ix;
+      re[p + 1] = fma_(c, re[p], -re[p - 1]);
+      im[p + 1] = fma_(c, im[p], -im[p - 1]);
+    }
+  }
 };
 
-// h_p(k d), p = 0..2L (closed forms of h_0, h_1 and upward recurrence)
-template <int L>
-__device__ __forceinline__ void fill_hankel(const GeomS& q, Geom<L, float>& g) {
-  constexpr int PM = 2 * L;
-  const float ix = q.ix, sn = q.sn, cs = q.cs;
-  g.hre[0] = sn * ix;
-  g.him[0] = -cs * ix;
-  g.hre[1] = -ix * fma_(-sn, ix, cs);
-  g.him[1] = -ix * fma_(cs, ix, sn);
+// cos / sin of q theta and m phi, q, m = 0..L
+template <int L, typename R>
+struct Angles {
+  R ct[L + 1], st[L + 1], cf[L + 1], sf[L + 1];
+  __device__ __forceinline__ Angles(R c, R s, R cp, R sp) {
+    ct[0] = cf[0] = static_cast<R>(1);
+    st[0] = sf[0] = static_cast<R>(0);
+    ct[1] = c;
+    st[1] = s;
+    cf[1] = cp;
+    sf[1] = sp;
 #pragma unroll
-  for (int p = 1; p < PM; ++p) {
-    const float c = static_cast<float>(2 * p + 1) * ix;
-    g.hre[p + 1] = fma_(c, g.hre[p], -g.hre[p - 1]);
-    g.him[p + 1] = fma_(c, g.him[p], -g.him[p - 1]);
+    for (int m = 2; m <= L; ++m) {
+      ct[m] = fma_(ct[m - 1], c, -st[m - 1] * s);
+      st[m] = fma_(ct[m - 1], s, st[m - 1] * c);
+      cf[m] = fma_(cf[m - 1], cp, -sf[m - 1] * sp);
+      sf[m] = fma_(cf[m - 1], sp, sf[m - 1] * cp);
+    }
   }
-}
+};
 
-template <int L>
-__device__ __forceinline__ GeomS geometry_ff_scalars(const PosFF& a, const PosFF& b);
-
-template <int L>
-__device__ __forceinline__ void geometry_ff(const PosFF& a, const PosFF& b, Geom<L, float>& g) {
-  const GeomS q = geometry_ff_scalars<L>(a, b);
-  fill_hankel<L>(q, g);
-  geometry_angles<L>(q.ct, q.st, q.cph, q.sph, g);
-}
-
-template <int L>
-__device__ __forceinline__ GeomS geometry_ff_scalars(const PosFF& a, const PosFF& b) {
+__device__ __forceinline__ GeomS<float> geometry_ff(const PosFF& a, const PosFF& b) {
   // k (r_a - r_b) per axis as s + e (unnormalised; |e| << |s| or s == 0)
   float sx, ex, sy, ey, sz, ez;
   two_diff(a.xh, b.xh, sx, ex);
@@ -185,109 +206,72 @@ __device__ __forceinline__ GeomS geometry_ff_scalars(const PosFF& a, const PosFF
   const float n = rintf(__fmul_rn(r, static_cast<float>(1.0 / HALF_PI)));
   float y = __fmaf_rn(-n, H1, r);  // exact
   y = __fadd_rn(y, __fmaf_rn(-n, H2, delta));
-  float sn, cs;
-  sincos_quadrant(y, static_cast<int>(n) & 3, sn, cs);
+  GeomS<float> q;
+  sincos_quadrant(y, static_cast<int>(n) & 3, q.sn, q.cs);
+  // reciprocals from the approximate reciprocal square roots, each with one
+  // Newton step (an error of about half an ulp, without the branches of an
+  // exact division or square root)
   const float kd = __fadd_rn(r, delta);
-  GeomS q;
-  q.ix = 1.0f / kd;
-  q.sn = sn;
-  q.cs = cs;
+  q.ix = fma_(rinv, fma_(-kd, rinv, 1.0f), rinv);
   const float dxf = __fadd_rn(sx, ex), dyf = __fadd_rn(sy, ey), dzf = __fadd_rn(sz, ez);
-  const float rho = sqrtf(fma_(dxf, dxf, dyf * dyf));
-  q.ct = fminf(1.0f, fmaxf(-1.0f, dzf * rinv));
-  q.st = fminf(1.0f, rho * rinv);
-  const float ir = rho > 0.0f ? 1.0f / rho : 0.0f;
-  q.cph = rho > 0.0f ? dxf * ir : 1.0f;
-  q.sph = dyf * ir;
+  const float rho2 = fma_(dxf, dxf, dyf * dyf);
+  const float w = rsqrtf(rho2);
+  const float t = rho2 * w;  // rho
+  const float e = 0.5f * fma_(-t, w, 1.0f);
+  const bool off_axis = rho2 > 0.0f;  // on the z axis phi does not matter
+  const float ir = fma_(w, e, w);
+  q.ct = dzf * q.ix;
+  q.st = off_axis ? fma_(t, e, t) * q.ix : 0.0f;
+  q.cph = off_axis ? dxf * ir : 1.0f;
+  q.sph = off_axis ? dyf * ir : 0.0f;
   return q;
 }
 
 // FP64 pair geometry (the FP64 kernel)
-template <int L, typename R>
-__device__ __forceinline__ void geometry(double dx, double dy, double dz, double k, Geom<L, R>& g) {
-  static_assert(sizeof(R) == 8, "the FP32 kernel uses geometry_ff");
-  constexpr int PM = 2 * L;
-  const double d2 = fma_(dx, dx, fma_(dy, dy, dz * dz));
-  const double d = sqrt(d2);
+__device__ __forceinline__ GeomS<double> geometry(double dx, double dy, double dz, double k) {
+  const double d = sqrt(fma_(dx, dx, fma_(dy, dy, dz * dz)));
   const double kd = k * d;
   const double TWO_PI = 6.283185307179586476925286766559;
   const double ph = fma_(-rint(kd * (1.0 / TWO_PI)), TWO_PI, kd);
-  double sn, cs;
-  sincos(ph, &sn, &cs);
-  const double ix = 1.0 / kd;
-  g.hre[0] = sn * ix;
-  g.him[0] = -cs * ix;
-  g.hre[1] = -ix * fma_(-sn, ix, cs);
-  g.him[1] = -ix * fma_(cs, ix, sn);
-#pragma unroll
-  for (int p = 1; p < PM; ++p) {
-    const double a = static_cast<double>(2 * p + 1) * ix;
-    g.hre[p + 1] = fma_(a, g.hre[p], -g.hre[p - 1]);
-    g.him[p + 1] = fma_(a, g.him[p], -g.him[p - 1]);
-  }
+  GeomS<double> q;
+  sincos(ph, &q.sn, &q.cs);
+  q.ix = 1.0 / kd;
   const double id = 1.0 / d;
   const double rho = sqrt(fma_(dx, dx, dy * dy));
-  const double ct = dz * id;
-  const double st = rho * id;
+  q.ct = dz * id;
+  q.st = rho * id;
   const double ir = rho > 0.0 ? 1.0 / rho : 0.0;
-  const double cph = rho > 0.0 ? dx * ir : 1.0;
-  const double sph = dy * ir;
-  geometry_angles_t<L, R>(ct, st, cph, sph, g);
+  q.cph = rho > 0.0 ? dx * ir : 1.0;
+  q.sph = dy * ir;
+  return q;
 }
 
-// half angles, their powers and e^{i m phi}
-template <int L, typename R>
-__device__ __forceinline__ void geometry_angles_t(R ct, R st, R cph, R sph, Geom<L, R>& g) {
-  constexpr int PM = 2 * L;
-  // half angles without cancellation: c = sqrt((1+ct)/2), s = st/(2c) for
-  // ct >= 0, and the mirror formulas otherwise
-  R c, s;
-  if (ct >= static_cast<R>(0)) {
-    c = sqrt(static_cast<R>(0.5) * (static_cast<R>(1) + ct));
-    s = static_cast<R>(0.5) * st / c;
-  } else {
-    s = sqrt(static_cast<R>(0.5) * (static_cast<R>(1) - ct));
-    c = static_cast<R>(0.5) * st / s;
-  }
-  g.cp[0] = static_cast<R>(1);
-  g.sp[0] = static_cast<R>(1);
-#pragma unroll
-  for (int q = 1; q <= PM; ++q) {
-    g.cp[q] = g.cp[q - 1] * c;
-    g.sp[q] = g.sp[q - 1] * s;
-  }
-  g.ere[0] = static_cast<R>(1);
-  g.eim[0] = static_cast<R>(0);
-#pragma unroll
-  for (int m = 1; m <= L; ++m) {
-    g.ere[m] = fma_(g.ere[m - 1], cph, -g.eim[m - 1] * sph);
-    g.eim[m] = fma_(g.ere[m - 1], sph, g.eim[m - 1] * cph);
+// ---- rotation blocks C and S of degree l -----------------------------------
+template <int L, int l, int KIND, int MU, int M, int Q, typename R>
+__device__ __forceinline__ void rot_term(const Angles<L, R>& g, R& acc) {
+  using E = RotCoef<l, KIND, MU, M, Q>;
+  if constexpr (E::v != 0.0) {
+    constexpr R c = static_cast<R>(E::v);
+    const R f = E::sine ? g.st[Q] : g.ct[Q];
+    if constexpr (Q == 0) acc = c;
+    else acc = E::before() == 0 ? c * f : fma_(c, f, acc);
   }
 }
-
-// ---- Wigner-d canonical entries of degree l --------------------------------
-template <int l, int T, typename R>
-__device__ __forceinline__ void dterm(const R* q, R& acc) {
-  constexpr R C = static_cast<R>(DTerm<l, T>::c);
-  acc = fma_(C, q[DTerm<l, T>::j], acc);
-}
-template <int l, int T0, typename R, int... K>
-__device__ __forceinline__ R dsum(const R* q, std::integer_sequence<int, K...>) {
+template <int L, int l, int KIND, int MU, int M, typename R, int... QI>
+__device__ __forceinline__ R rot_value(const Angles<L, R>& g, std::integer_sequence<int, QI...>) {
   R acc = static_cast<R>(0);
-  (dterm<l, T0 + K>(q, acc), ...);
+  (rot_term<L, l, KIND, MU, M, QI>(g, acc), ...);
   return acc;
 }
-template <int l, typename R, int... C>
-__device__ __forceinline__ void dcanon(const R* q, R* dv, std::integer_sequence<int, C...>) {
-  ((dv[C] = dsum<l, DCanon<l, C>::t0>(q, std::make_integer_sequence<int, DCanon<l, C>::t1 - DCanon<l, C>::t0>{})),
+template <int L, int l, int KIND, int MU, typename R, int... MI>
+__device__ __forceinline__ void rot_table_row(const Angles<L, R>& g, R* v, std::integer_sequence<int, MI...>) {
+  ((v[rot_id(KIND, MU, MI + KIND)] = rot_value<L, l, KIND, MU, MI + KIND>(g, std::make_integer_sequence<int, l + 1>{})),
    ...);
 }
-template <int L, int l, typename R>
-__device__ __forceinline__ void dmatrix(const Geom<L, R>& g, R* dv) {
-  R q[2 * l + 1];
-#pragma unroll
-  for (int j = 0; j <= 2 * l; ++j) q[j] = g.cp[2 * l - j] * g.sp[j];
-  dcanon<l, R>(q, dv, std::make_integer_sequence<int, DCount<l>::ncanon>{});
+template <int L, int l, typename R, int... MUI>
+__device__ __forceinline__ void rot_table(const Angles<L, R>& g, R* vc, R* vs, std::integer_sequence<int, MUI...>) {
+  (rot_table_row<L, l, 0, MUI>(g, vc, std::make_integer_sequence<int, MUI + 1>{}), ...);
+  (rot_table_row<L, l, 1, MUI>(g, vs, std::make_integer_sequence<int, MUI>{}), ...);
 }
 
 // row index of (l, m) inside one polarisation block
@@ -296,152 +280,101 @@ struct Row {
   static constexpr int r = l * (l + 1) - 1 + m;
 };
 
-// ---- step 2: x'[l, MU] = sum_M R_{MU,M} e^{i M phi} x[l, M] ----------------
-// x~ (rotated about z) of degree l held in xt[2][2l+1][2]
-template <int L, int l, int MU, int OPT, typename R, typename XV, int... MI>
-__device__ __forceinline__ void rot_fwd_row(const R* dv, const R (&xt)[2][2 * l + 1][2], XV& xp,
-                                            std::integer_sequence<int, MI...>) {
-  constexpr int NH = L * (L + 2);
-  R a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-  if constexpr (kPackedRot<L, R, OPT>) {
-    // (re, im) of one complex value per packed FMA, same rounding as fma_
-    float2 a = make_float2(0.0f, 0.0f), b = a;
-    (
-        [&] {
-          constexpr int M = MI - l;
-          using RA = RAt<l, MU, M>;
-          const float w = RA::sign > 0 ? dv[RA::id] : -dv[RA::id];
-          const float2 ww = make_float2(w, w);
-          a = __ffma2_rn(ww, make_float2(xt[0][MI][0], xt[0][MI][1]), a);
-          b = __ffma2_rn(ww, make_float2(xt[1][MI][0], xt[1][MI][1]), b);
-        }(),
-        ...);
-    a0 = a.x;
-    a1 = a.y;
-    b0 = b.x;
-    b1 = b.y;
+// row mu of block KIND times in[tau][.] (C: columns 0..l, S: 1..l, stored from 0)
+template <int l, int KIND, int MU, typename R, int... MI>
+__device__ __forceinline__ C2<R> rot_row(const R* v, const C2<R>* in, std::integer_sequence<int, MI...>) {
+  if constexpr (RotEntry<l, KIND, KIND, KIND>::unit()) {
+    if constexpr (RotCoef<l, KIND, KIND, KIND, 0>::v > 0.0) return in[0];
+    else return C2<R>{-in[0].x, -in[0].y};
   } else {
-    (
-        [&] {
-          constexpr int M = MI - l;
-          using RA = RAt<l, MU, M>;
-          const R w = RA::sign > 0 ? dv[RA::id] : -dv[RA::id];
-          a0 = fma_(w, xt[0][MI][0], a0);
-          a1 = fma_(w, xt[0][MI][1], a1);
-          b0 = fma_(w, xt[1][MI][0], b0);
-          b1 = fma_(w, xt[1][MI][1], b1);
-        }(),
-        ...);
+    C2<R> a = mul2(v[rot_id(KIND, MU + KIND, KIND)], in[0]);
+    ((a = fma2(v[rot_id(KIND, MU + KIND, MI + 1 + KIND)], in[MI + 1], a)), ...);
+    return a;
   }
-  constexpr int r = Row<l, MU>::r;
-  xp(2 * r) = a0;
-  xp(2 * r + 1) = a1;
-  xp(2 * (NH + r)) = b0;
-  xp(2 * (NH + r) + 1) = b1;
+}
+template <int l, int KIND, typename R, int... MUI>
+__device__ __forceinline__ void rot_apply(const R* v, const C2<R>* in, C2<R>* out,
+                                          std::integer_sequence<int, MUI...>) {
+  constexpr int n = KIND == 0 ? l + 1 : l;
+  ((out[MUI] = rot_row<l, KIND, MUI>(v, in, std::make_integer_sequence<int, n - 1>{})), ...);
 }
 
-// PP (packed phase): the x+ half's e^{i m phi} multiply on the packed
-// two-lane FMA, which moves work from the scalar half of the FP32 lanes (that
-// carries the axial entries, the axial apply and the phases) to the half that
-// carries the packed rotations; an autotuner candidate (ConfigAlt at lmax 4)
-template <int L, int l, int OPT, typename R, typename XV, int... MUI>
-__device__ __forceinline__ void rot_fwd_block(const Geom<L, R>& g, const Pair2<R>* __restrict__ xs, XV& xp,
-                                              std::integer_sequence<int, MUI...>) {
-  constexpr int NH = L * (L + 2);
-  R dv[DCount<l>::ncanon];
-  dmatrix<L, l>(g, dv);
-  R xt[2][2 * l + 1][2];
+// ---- step 2: x' = (C, S) (x turned by phi), degree l ------------------------
+template <int L, int l, typename R, typename XV>
+__device__ __forceinline__ void rot_fwd_block(const Angles<L, R>& g, const Quad4<R>* __restrict__ xs, XV& xp) {
+  C2<R> c[2][l + 1], s[2][l], oc[2][l + 1], os[2][l];
+  {
+    const Quad4<R> q = xs[Row<l, 0>::r];
+    c[0][0] = C2<R>{q.x, q.y};
+    c[1][0] = C2<R>{q.z, q.w};
+  }
 #pragma unroll
-  for (int mi = 0; mi <= 2 * l; ++mi) {
-    const int m = mi - l;
-    const int am = m < 0 ? -m : m;
-    const R er = g.ere[am];
-    const R ei = m < 0 ? -g.eim[am] : g.eim[am];
-    const int r = l * (l + 1) - 1 + m;
-    const Pair2<R> xa = xs[r], xb = xs[NH + r];
-    if constexpr ((OPT & 1) != 0 && kPackedRot<L, R, OPT>) {
-      const float2 t = __fmul2_rn(make_float2(xa.im, xa.im), make_float2(-ei, er));
-      const float2 u = __ffma2_rn(make_float2(xa.re, xa.re), make_float2(er, ei), t);
-      xt[0][mi][0] = u.x;
-      xt[0][mi][1] = u.y;
-    } else {
-      xt[0][mi][0] = fma_(xa.re, er, -xa.im * ei);
-      xt[0][mi][1] = fma_(xa.re, ei, xa.im * er);
-    }
-    xt[1][mi][0] = fma_(xb.re, er, -xb.im * ei);
-    xt[1][mi][1] = fma_(xb.re, ei, xb.im * er);
+  for (int m = 1; m <= l; ++m) {
+    const Quad4<R> qc = xs[l * (l + 1) - 1 + m], qs = xs[l * (l + 1) - 1 - m];
+    const R cf = g.cf[m], sf = g.sf[m];
+    c[0][m] = fma2(cf, C2<R>{qc.x, qc.y}, mul2(sf, C2<R>{qs.x, qs.y}));
+    s[0][m - 1] = fma2(cf, C2<R>{qs.x, qs.y}, mul2(-sf, C2<R>{qc.x, qc.y}));
+    c[1][m] = fma2(cf, C2<R>{qc.z, qc.w}, mul2(sf, C2<R>{qs.z, qs.w}));
+    s[1][m - 1] = fma2(cf, C2<R>{qs.z, qs.w}, mul2(-sf, C2<R>{qc.z, qc.w}));
   }
-  (rot_fwd_row<L, l, MUI - l, OPT>(dv, xt, xp, std::make_integer_sequence<int, 2 * l + 1>{}), ...);
+  R vc[RotCount<l>::nc], vs[RotCount<l>::ns];
+  rot_table<L, l>(g, vc, vs, std::make_integer_sequence<int, l + 1>{});
+  rot_apply<l, 0>(vc, c[0], oc[0], std::make_integer_sequence<int, l + 1>{});
+  rot_apply<l, 0>(vc, c[1], oc[1], std::make_integer_sequence<int, l + 1>{});
+  rot_apply<l, 1>(vs, s[0], os[0], std::make_integer_sequence<int, l>{});
+  rot_apply<l, 1>(vs, s[1], os[1], std::make_integer_sequence<int, l>{});
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+#pragma unroll
+    for (int m = 0; m <= l; ++m) {
+      xp(4 * (l * (l + 1) - 1 + m) + 2 * t) = oc[t][m].x;
+      xp(4 * (l * (l + 1) - 1 + m) + 2 * t + 1) = oc[t][m].y;
+    }
+#pragma unroll
+    for (int m = 0; m < l; ++m) {
+      xp(4 * (l * (l + 1) - 2 - m) + 2 * t) = os[t][m].x;
+      xp(4 * (l * (l + 1) - 2 - m) + 2 * t + 1) = os[t][m].y;
+    }
+  }
 }
-
-template <int L, int OPT, typename R, typename XV, int... LI>
-__device__ __forceinline__ void rot_fwd(const Geom<L, R>& g, const Pair2<R>* __restrict__ xs, XV& xp,
+template <int L, typename R, typename XV, int... LI>
+__device__ __forceinline__ void rot_fwd(const Angles<L, R>& g, const Quad4<R>* __restrict__ xs, XV& xp,
                                         std::integer_sequence<int, LI...>) {
-  (rot_fwd_block<L, LI + 1, OPT>(g, xs, xp, std::make_integer_sequence<int, 2 * (LI + 1) + 1>{}), ...);
+  (rot_fwd_block<L, LI + 1>(g, xs, xp), ...);
 }
 
-// ---- step 3: axial translation --------------------------------------------
+// ---- step 3: axial translation, in place (y' overwrites x') -----------------
+// (MU > 0: times 1/2, the factor of going to the sums and back)
 template <int L, int MU, int LO, int LI, int T, typename R>
-__device__ __forceinline__ void ax_a(const Geom<L, R>& g, R& ar, R& ai) {
+__device__ __forceinline__ void ax_a(const Hankel<L, R>& h, R& ar, R& ai) {
   using A = AxialA<L, MU, LO, LI, T>;
-  constexpr R C = static_cast<R>(A::c);
-  ar = fma_(C, g.hre[A::p], ar);
-  ai = fma_(C, g.him[A::p], ai);
+  constexpr R C = static_cast<R>(MU > 0 ? 0.5 * A::c : A::c);
+  ar = T == 0 ? C * h.re[A::p] : fma_(C, h.re[A::p], ar);
+  ai = T == 0 ? C * h.im[A::p] : fma_(C, h.im[A::p], ai);
 }
 template <int L, int MU, int LO, int LI, int T, typename R>
-__device__ __forceinline__ void ax_b(const Geom<L, R>& g, R& br, R& bi) {
+__device__ __forceinline__ void ax_b(const Hankel<L, R>& h, R& br, R& bi) {
   using B = AxialB<L, MU, LO, LI, T>;
-  constexpr R C = static_cast<R>(B::c);
-  br = fma_(C, g.hre[B::p], br);
-  bi = fma_(C, g.him[B::p], bi);
+  constexpr R C = static_cast<R>(MU > 0 ? 0.5 * B::c : B::c);
+  br = T == 0 ? C * h.re[B::p] : fma_(C, h.re[B::p], br);
+  bi = T == 0 ? C * h.im[B::p] : fma_(C, h.im[B::p], bi);
 }
 template <int L, int MU, int LO, int LI, typename R, int... KA, int... KB>
-__device__ __forceinline__ void ax_entry(const Geom<L, R>& g, R& ar, R& ai, R& br, R& bi,
+__device__ __forceinline__ void ax_entry(const Hankel<L, R>& h, R& ar, R& ai, R& br, R& bi,
                                          std::integer_sequence<int, KA...>, std::integer_sequence<int, KB...>) {
-  (ax_a<L, MU, LO, LI, KA>(g, ar, ai), ...);
-  (ax_b<L, MU, LO, LI, KB>(g, br, bi), ...);
+  (ax_a<L, MU, LO, LI, KA>(h, ar, ai), ...);
+  (ax_b<L, MU, LO, LI, KB>(h, br, bi), ...);
 }
-
-template <typename R>
-__device__ __forceinline__ void cmac(R& yr, R& yi, R wr, R wi, R xr, R xi) {
-  yr = fma_(wr, xr, fma_(-wi, xi, yr));
-  yi = fma_(wr, xi, fma_(wi, xr, yi));
-}
-
-// one (l, l') entry of the axial block for +MU (and the mirrored -MU),
-// accumulated into the row sums y[0..3] (+MU: y+ re/im, y- re/im) and
-// y[4..7] (-MU)
-template <int L, int MU, int LO, int LI, typename R, typename XV>
-__device__ __forceinline__ void ax_pair(const Geom<L, R>& g, XV& xp, R (&y)[8]) {
-  constexpr int NH = L * (L + 2);
-  if constexpr (LI >= MU) {
-    R ar = 0, ai = 0, br = 0, bi = 0;
-    ax_entry<L, MU, LO, LI>(g, ar, ai, br, bi, std::make_integer_sequence<int, AxialN<L, MU, LO, LI>::na>{},
-                            std::make_integer_sequence<int, AxialN<L, MU, LO, LI>::nb>{});
-    // W+ = A + i B', W- = A - i B'
-    const R wpr = ar - bi, wpi = ai + br, wmr = ar + bi, wmi = ai - br;
-    constexpr int ri = Row<LI, MU>::r;
-    cmac(y[0], y[1], wpr, wpi, xp(2 * ri), xp(2 * ri + 1));
-    cmac(y[2], y[3], wmr, wmi, xp(2 * (NH + ri)), xp(2 * (NH + ri) + 1));
-    if constexpr (MU > 0) {
-      // -mu: B changes sign, so W+ and W- swap
-      constexpr int rim = Row<LI, -MU>::r;
-      cmac(y[4], y[5], wmr, wmi, xp(2 * rim), xp(2 * rim + 1));
-      cmac(y[6], y[7], wpr, wpi, xp(2 * (NH + rim)), xp(2 * (NH + rim) + 1));
-    }
-  }
-}
-
-template <int L, int MU, int LO, typename R, typename YV>
-__device__ __forceinline__ void ax_store(YV& yp, const R (&y)[8]);
 
 // y += S w x for one (row, column) entry, S = +-1 at compile time
 template <int S, typename R>
-__device__ __forceinline__ void cmac_s(R& yr, R& yi, R wr, R wi, R xr, R xi) {
+__device__ __forceinline__ void cmac_s(R* y, R wr, R wi, const R* x) {
   if constexpr (S > 0) {
-    cmac(yr, yi, wr, wi, xr, xi);
+    y[0] = fma_(wr, x[0], fma_(-wi, x[1], y[0]));
+    y[1] = fma_(wr, x[1], fma_(wi, x[0], y[1]));
   } else {
-    cmac(yr, yi, -wr, -wi, xr, xi);
+    y[0] = fma_(-wr, x[0], fma_(wi, x[1], y[0]));
+    y[1] = fma_(-wr, x[1], fma_(-wi, x[0], y[1]));
   }
 }
 
@@ -450,173 +383,140 @@ __device__ __forceinline__ void cmac_s(R& yr, R& yi, R wr, R wi, R xr, R xi) {
 // alike; it follows from the inversion parity of the SVWFs, and is checked
 // against the dense coupling matrix).  So each entry with LO <= LI is formed
 // once and applied to row LO (column LI) and, with that sign, to row LI
-// (column LO).  y[l - 1] holds row l: (+mu: y+ re/im, y- re/im; -mu: same).
-template <int L, int MU, int LO, int LI, typename R, typename XV>
-__device__ __forceinline__ void ax_sym_pair(const Geom<L, R>& g, XV& xp, R (&y)[L][8]) {
-  constexpr int NH = L * (L + 2);
+// (column LO).  u[l - 1], y[l - 1]: the sums of degree l, MU > 0
+// (c1 + s2, c2 - s1 | c1 - s2, c2 + s1), MU = 0 (c1, c2), re and im each.
+template <int L, int MU, int LO, int LI, typename R>
+__device__ __forceinline__ void ax_sym_pair(const Hankel<L, R>& h, const R (&u)[L][8], R (&y)[L][8]) {
   if constexpr (LO >= MU && LI >= MU && LO <= LI) {
     R ar = 0, ai = 0, br = 0, bi = 0;
-    ax_entry<L, MU, LO, LI>(g, ar, ai, br, bi, std::make_integer_sequence<int, AxialN<L, MU, LO, LI>::na>{},
+    ax_entry<L, MU, LO, LI>(h, ar, ai, br, bi, std::make_integer_sequence<int, AxialN<L, MU, LO, LI>::na>{},
                             std::make_integer_sequence<int, AxialN<L, MU, LO, LI>::nb>{});
-    const R wpr = ar - bi, wpi = ai + br, wmr = ar + bi, wmi = ai - br;
-    {
-      R(&yo)[8] = y[LO - 1];
-      constexpr int ri = Row<LI, MU>::r;
-      cmac(yo[0], yo[1], wpr, wpi, xp(2 * ri), xp(2 * ri + 1));
-      cmac(yo[2], yo[3], wmr, wmi, xp(2 * (NH + ri)), xp(2 * (NH + ri) + 1));
-      if constexpr (MU > 0) {
-        constexpr int rim = Row<LI, -MU>::r;
-        cmac(yo[4], yo[5], wmr, wmi, xp(2 * rim), xp(2 * rim + 1));
-        cmac(yo[6], yo[7], wpr, wpi, xp(2 * (NH + rim)), xp(2 * (NH + rim) + 1));
+    constexpr int S = ((LO + LI) & 1) ? -1 : 1;
+    if constexpr (MU == 0) {
+      cmac_s<1>(y[LO - 1], ar, ai, u[LI - 1]);
+      cmac_s<1>(y[LO - 1] + 2, ar, ai, u[LI - 1] + 2);
+      if constexpr (LO != LI) {
+        cmac_s<S>(y[LI - 1], ar, ai, u[LO - 1]);
+        cmac_s<S>(y[LI - 1] + 2, ar, ai, u[LO - 1] + 2);
       }
-    }
-    if constexpr (LO != LI) {
-      constexpr int S = ((LO + LI) & 1) ? -1 : 1;
-      R(&yt)[8] = y[LI - 1];
-      constexpr int rj = Row<LO, MU>::r;
-      cmac_s<S>(yt[0], yt[1], wpr, wpi, xp(2 * rj), xp(2 * rj + 1));
-      cmac_s<S>(yt[2], yt[3], wmr, wmi, xp(2 * (NH + rj)), xp(2 * (NH + rj) + 1));
-      if constexpr (MU > 0) {
-        constexpr int rjm = Row<LO, -MU>::r;
-        cmac_s<S>(yt[4], yt[5], wmr, wmi, xp(2 * rjm), xp(2 * rjm + 1));
-        cmac_s<S>(yt[6], yt[7], wpr, wpi, xp(2 * (NH + rjm)), xp(2 * (NH + rjm) + 1));
+    } else {
+      // W+ = A + i B', W- = A - i B'
+      const R wpr = ar - bi, wpi = ai + br, wmr = ar + bi, wmi = ai - br;
+      cmac_s<1>(y[LO - 1], wpr, wpi, u[LI - 1]);
+      cmac_s<1>(y[LO - 1] + 2, wpr, wpi, u[LI - 1] + 2);
+      cmac_s<1>(y[LO - 1] + 4, wmr, wmi, u[LI - 1] + 4);
+      cmac_s<1>(y[LO - 1] + 6, wmr, wmi, u[LI - 1] + 6);
+      if constexpr (LO != LI) {
+        cmac_s<S>(y[LI - 1], wpr, wpi, u[LO - 1]);
+        cmac_s<S>(y[LI - 1] + 2, wpr, wpi, u[LO - 1] + 2);
+        cmac_s<S>(y[LI - 1] + 4, wmr, wmi, u[LO - 1] + 4);
+        cmac_s<S>(y[LI - 1] + 6, wmr, wmi, u[LO - 1] + 6);
       }
     }
   }
 }
-template <int L, int MU, int LO, typename R, typename XV, int... LII>
-__device__ __forceinline__ void ax_sym_row(const Geom<L, R>& g, XV& xp, R (&y)[L][8],
+template <int L, int MU, int LO, typename R, int... LII>
+__device__ __forceinline__ void ax_sym_row(const Hankel<L, R>& h, const R (&u)[L][8], R (&y)[L][8],
                                            std::integer_sequence<int, LII...>) {
-  (ax_sym_pair<L, MU, LO, LII + 1>(g, xp, y), ...);
+  (ax_sym_pair<L, MU, LO, LII + 1>(h, u, y), ...);
 }
-template <int L, int MU, typename R, typename XV, typename YV, int... LOI>
-__device__ __forceinline__ void ax_mu_sym(const Geom<L, R>& g, XV& xp, YV& yp, std::integer_sequence<int, LOI...>) {
-  R y[L][8];
+template <int L, int MU, int l, typename R, typename XV>
+__device__ __forceinline__ void ax_load(XV& xp, R (&u)[L][8], R (&y)[L][8]) {
+  if constexpr (l >= MU) {
+    constexpr int rc = 4 * Row<l, MU>::r, rs = 4 * Row<l, -MU>::r;
 #pragma unroll
-  for (int a = 0; a < L; ++a)
+    for (int q = 0; q < 2; ++q) {
+      const R c1 = xp(rc + q), c2 = xp(rc + 2 + q);
+      if constexpr (MU == 0) {
+        u[l - 1][q] = c1;
+        u[l - 1][2 + q] = c2;
+      } else {
+        const R s1 = xp(rs + q), s2 = xp(rs + 2 + q);
+        u[l - 1][q] = c1 + s2;
+        u[l - 1][2 + q] = c2 - s1;
+        u[l - 1][4 + q] = c1 - s2;
+        u[l - 1][6 + q] = c2 + s1;
+      }
+    }
 #pragma unroll
-    for (int q = 0; q < 8; ++q) y[a][q] = static_cast<R>(0);
-  (ax_sym_row<L, MU, LOI + 1>(g, xp, y, std::make_integer_sequence<int, L>{}), ...);
-  (ax_store<L, MU, LOI + 1>(yp, y[LOI]), ...);
-}
-
-template <int L, int MU, int LO, typename R, typename XV, int... LII>
-__device__ __forceinline__ void ax_row(const Geom<L, R>& g, XV& xp, R (&y)[8], std::integer_sequence<int, LII...>) {
-  if constexpr (LO >= MU) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) y[q] = static_cast<R>(0);
-    (ax_pair<L, MU, LO, LII + 1>(g, xp, y), ...);
+    for (int q = 0; q < 8; ++q) y[l - 1][q] = static_cast<R>(0);
   }
 }
-template <int L, int MU, int LO, typename R, typename YV>
-__device__ __forceinline__ void ax_store(YV& yp, const R (&y)[8]) {
-  constexpr int NH = L * (L + 2);
-  if constexpr (LO >= MU) {
-    constexpr int ro = Row<LO, MU>::r;
-    yp(2 * ro) = y[0];
-    yp(2 * ro + 1) = y[1];
-    yp(2 * (NH + ro)) = y[2];
-    yp(2 * (NH + ro) + 1) = y[3];
-    if constexpr (MU > 0) {
-      constexpr int rom = Row<LO, -MU>::r;
-      yp(2 * rom) = y[4];
-      yp(2 * rom + 1) = y[5];
-      yp(2 * (NH + rom)) = y[6];
-      yp(2 * (NH + rom) + 1) = y[7];
+template <int L, int MU, int l, typename R, typename XV>
+__device__ __forceinline__ void ax_store(XV& xp, const R (&y)[L][8]) {
+  if constexpr (l >= MU) {
+    constexpr int rc = 4 * Row<l, MU>::r, rs = 4 * Row<l, -MU>::r;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if constexpr (MU == 0) {
+        xp(rc + q) = y[l - 1][q];
+        xp(rc + 2 + q) = y[l - 1][2 + q];
+      } else {
+        xp(rc + q) = y[l - 1][q] + y[l - 1][4 + q];
+        xp(rc + 2 + q) = y[l - 1][2 + q] + y[l - 1][6 + q];
+        xp(rs + q) = y[l - 1][6 + q] - y[l - 1][2 + q];
+        xp(rs + 2 + q) = y[l - 1][q] - y[l - 1][4 + q];
+      }
     }
   }
 }
-template <int L, int MU, int LO, typename R, typename XV, typename YV>
-__device__ __forceinline__ void ax_row_store(const Geom<L, R>& g, XV& xp, YV& yp) {
-  R y[8];
-  ax_row<L, MU, LO>(g, xp, y, std::make_integer_sequence<int, L>{});
-  ax_store<L, MU, LO>(yp, y);
+template <int L, int MU, typename R, typename XV, int... LOI>
+__device__ __forceinline__ void ax_mu(const Hankel<L, R>& h, XV& xp, std::integer_sequence<int, LOI...>) {
+  R u[L][8], y[L][8];
+  (ax_load<L, MU, LOI + 1>(xp, u, y), ...);
+  (ax_sym_row<L, MU, LOI + 1>(h, u, y, std::make_integer_sequence<int, L>{}), ...);
+  (ax_store<L, MU, LOI + 1>(xp, y), ...);
 }
-// in place (y' overwrites x'): all rows of one |mu| are formed before any is
-// stored, since the rows of |mu| read every x'[., +-mu]; otherwise each row is
-// stored as soon as it is formed
-template <int L, int MU, bool INPLACE, typename R, typename XV, typename YV, int... LOI>
-__device__ __forceinline__ void ax_mu(const Geom<L, R>& g, XV& xp, YV& yp, std::integer_sequence<int, LOI...>) {
-  if constexpr (INPLACE) {
-    R y[L][8];
-    (ax_row<L, MU, LOI + 1>(g, xp, y[LOI], std::make_integer_sequence<int, L>{}), ...);
-    (ax_store<L, MU, LOI + 1>(yp, y[LOI]), ...);
-  } else {
-    (ax_row_store<L, MU, LOI + 1>(g, xp, yp), ...);
-  }
-}
-template <int L, bool INPLACE, bool SYM, typename R, typename XV, typename YV, int... MUS>
-__device__ __forceinline__ void axial(const Geom<L, R>& g, XV& xp, YV& yp, std::integer_sequence<int, MUS...>) {
-  if constexpr (SYM) {
-    (ax_mu_sym<L, MUS>(g, xp, yp, std::make_integer_sequence<int, L>{}), ...);
-  } else {
-    (ax_mu<L, MUS, INPLACE>(g, xp, yp, std::make_integer_sequence<int, L>{}), ...);
-  }
+template <int L, typename R, typename XV, int... MUS>
+__device__ __forceinline__ void axial(const Hankel<L, R>& h, XV& xp, std::integer_sequence<int, MUS...>) {
+  (ax_mu<L, MUS>(h, xp, std::make_integer_sequence<int, L>{}), ...);
 }
 
-// ---- step 4: y[l, M] += e^{-i M phi} sum_MU R_{MU,M} y'[l, MU] -------------
-template <int L, int l, int M, int OPT, typename R, typename YV, typename Acc, int... MUI>
-__device__ __forceinline__ void rot_bwd_col(const Geom<L, R>& g, const R* dv, YV& yp, Acc& acc,
-                                            std::integer_sequence<int, MUI...>) {
-  constexpr int NH = L * (L + 2);
-  R a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-  if constexpr (kPackedRot<L, R, OPT>) {
-    float2 a = make_float2(0.0f, 0.0f), b = a;
-    (
-        [&] {
-          constexpr int MU = MUI - l;
-          using RA = RAt<l, MU, M>;
-          const float w = RA::sign > 0 ? dv[RA::id] : -dv[RA::id];
-          const float2 ww = make_float2(w, w);
-          constexpr int r = Row<l, MU>::r;
-          a = __ffma2_rn(ww, make_float2(yp(2 * r), yp(2 * r + 1)), a);
-          b = __ffma2_rn(ww, make_float2(yp(2 * (NH + r)), yp(2 * (NH + r) + 1)), b);
-        }(),
-        ...);
-    a0 = a.x;
-    a1 = a.y;
-    b0 = b.x;
-    b1 = b.y;
-  } else {
-    (
-        [&] {
-          constexpr int MU = MUI - l;
-          using RA = RAt<l, MU, M>;
-          const R w = RA::sign > 0 ? dv[RA::id] : -dv[RA::id];
-          constexpr int r = Row<l, MU>::r;
-          a0 = fma_(w, yp(2 * r), a0);
-          a1 = fma_(w, yp(2 * r + 1), a1);
-          b0 = fma_(w, yp(2 * (NH + r)), b0);
-          b1 = fma_(w, yp(2 * (NH + r) + 1), b1);
-        }(),
-        ...);
+// ---- step 4: y += ((C, S) y') turned back by phi, degree l ------------------
+template <int L, int l, typename R, typename XV, typename Acc>
+__device__ __forceinline__ void rot_bwd_block(const Angles<L, R>& g, XV& xp, Acc& acc) {
+  C2<R> c[2][l + 1], s[2][l], oc[2][l + 1], os[2][l];
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+#pragma unroll
+    for (int m = 0; m <= l; ++m) {
+      const int rc = 4 * (l * (l + 1) - 1 + m) + 2 * t;
+      c[t][m] = C2<R>{xp(rc), xp(rc + 1)};
+    }
+#pragma unroll
+    for (int m = 0; m < l; ++m) {
+      const int rs = 4 * (l * (l + 1) - 2 - m) + 2 * t;
+      s[t][m] = C2<R>{xp(rs), xp(rs + 1)};
+    }
   }
-  constexpr int AM = M < 0 ? -M : M;
-  const R er = g.ere[AM];
-  const R ei = M < 0 ? g.eim[AM] : -g.eim[AM];  // e^{-i M phi}
-  constexpr int r = Row<l, M>::r;
-  // row r of the receiver's sums: (y+ re, y+ im, y- re, y- im)
-  R c[4];
-  acc.load(r, c);
-  c[0] = fma_(a0, er, fma_(-a1, ei, c[0]));
-  c[1] = fma_(a0, ei, fma_(a1, er, c[1]));
-  c[2] = fma_(b0, er, fma_(-b1, ei, c[2]));
-  c[3] = fma_(b0, ei, fma_(b1, er, c[3]));
-  acc.store(r, c);
-  (void)NH;
+  R vc[RotCount<l>::nc], vs[RotCount<l>::ns];
+  rot_table<L, l>(g, vc, vs, std::make_integer_sequence<int, l + 1>{});
+  rot_apply<l, 0>(vc, c[0], oc[0], std::make_integer_sequence<int, l + 1>{});
+  rot_apply<l, 0>(vc, c[1], oc[1], std::make_integer_sequence<int, l + 1>{});
+  rot_apply<l, 1>(vs, s[0], os[0], std::make_integer_sequence<int, l>{});
+  rot_apply<l, 1>(vs, s[1], os[1], std::make_integer_sequence<int, l>{});
+  C2<R> a[2];
+  acc.load(Row<l, 0>::r, a);
+  a[0] = C2<R>{a[0].x + oc[0][0].x, a[0].y + oc[0][0].y};
+  a[1] = C2<R>{a[1].x + oc[1][0].x, a[1].y + oc[1][0].y};
+  acc.store(Row<l, 0>::r, a);
+#pragma unroll
+  for (int m = 1; m <= l; ++m) {
+    const int rc = l * (l + 1) - 1 + m, rs = l * (l + 1) - 1 - m;
+    const R cf = g.cf[m], sf = g.sf[m];
+    acc.load(rc, a);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) a[t] = fma2(cf, oc[t][m], fma2(-sf, os[t][m - 1], a[t]));
+    acc.store(rc, a);
+    acc.load(rs, a);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) a[t] = fma2(cf, os[t][m - 1], fma2(sf, oc[t][m], a[t]));
+    acc.store(rs, a);
+  }
 }
-
-template <int L, int l, int OPT, typename R, typename YV, typename Acc, int... MI>
-__device__ __forceinline__ void rot_bwd_block(const Geom<L, R>& g, YV& yp, Acc& acc,
-                                              std::integer_sequence<int, MI...>) {
-  R dv[DCount<l>::ncanon];
-  dmatrix<L, l>(g, dv);
-  (rot_bwd_col<L, l, MI - l, OPT>(g, dv, yp, acc, std::make_integer_sequence<int, 2 * l + 1>{}), ...);
-}
-
-template <int L, int OPT, typename R, typename YV, typename Acc, int... LI>
-__device__ __forceinline__ void rot_bwd(const Geom<L, R>& g, YV& yp, Acc& acc, std::integer_sequence<int, LI...>) {
-  (rot_bwd_block<L, LI + 1, OPT>(g, yp, acc, std::make_integer_sequence<int, 2 * (LI + 1) + 1>{}), ...);
+template <int L, typename R, typename XV, typename Acc, int... LI>
+__device__ __forceinline__ void rot_bwd(const Angles<L, R>& g, XV& xp, Acc& acc, std::integer_sequence<int, LI...>) {
+  (rot_bwd_block<L, LI + 1>(g, xp, acc), ...);
 }
 
 // storage views: registers (compile-time index) or a per-thread column of a
@@ -632,74 +532,106 @@ struct AccSmem {
   __device__ __forceinline__ R& operator()(int q) const { return a[q * BLOCK]; }
 };
 
-// receiver sums, one 4-vector (y+ re, y+ im, y- re, y- im) per output row:
-// registers [NH][4], or shared memory [NH][BLOCK] of 4-vectors (one 16- or
-// 32-byte access per row)
+// receiver sums, one 4-vector (tau 1 re, im, tau 2 re, im) per row (l, m):
+// c_m for m >= 0, s_|m| for m < 0; registers [NH][4], or shared memory
+// [NH][BLOCK] of 4-vectors (one 16- or 32-byte access per row)
 template <typename R>
 struct RowAccReg {
   R* a;
-  __device__ __forceinline__ void load(int r, R (&c)[4]) const {
-    c[0] = a[4 * r];
-    c[1] = a[4 * r + 1];
-    c[2] = a[4 * r + 2];
-    c[3] = a[4 * r + 3];
+  __device__ __forceinline__ void load(int r, C2<R> (&c)[2]) const {
+    c[0] = C2<R>{a[4 * r], a[4 * r + 1]};
+    c[1] = C2<R>{a[4 * r + 2], a[4 * r + 3]};
   }
-  __device__ __forceinline__ void store(int r, const R (&c)[4]) const {
-    a[4 * r] = c[0];
-    a[4 * r + 1] = c[1];
-    a[4 * r + 2] = c[2];
-    a[4 * r + 3] = c[3];
+  __device__ __forceinline__ void store(int r, const C2<R> (&c)[2]) const {
+    a[4 * r] = c[0].x;
+    a[4 * r + 1] = c[0].y;
+    a[4 * r + 2] = c[1].x;
+    a[4 * r + 3] = c[1].y;
   }
 };
 template <typename R, int BLOCK>
 struct RowAccSmem {
   Quad4<R>* a;  // this thread's element of row 0
-  __device__ __forceinline__ void load(int r, R (&c)[4]) const {
+  __device__ __forceinline__ void load(int r, C2<R> (&c)[2]) const {
     const Quad4<R> v = a[r * BLOCK];
-    c[0] = v.x;
-    c[1] = v.y;
-    c[2] = v.z;
-    c[3] = v.w;
+    c[0] = C2<R>{v.x, v.y};
+    c[1] = C2<R>{v.z, v.w};
   }
-  __device__ __forceinline__ void store(int r, const R (&c)[4]) const { a[r * BLOCK] = Quad4<R>{c[0], c[1], c[2], c[3]}; }
+  __device__ __forceinline__ void store(int r, const C2<R> (&c)[2]) const {
+    a[r * BLOCK] = Quad4<R>{c[0].x, c[0].y, c[1].x, c[1].y};
+  }
 };
 
-template <int L, bool INPLACE, bool SYM, typename R, int OPT = 0, typename XV, typename YV, typename Acc>
-__device__ __forceinline__ void pair(const Geom<L, R>& g, const Pair2<R>* __restrict__ xs, XV& xp, YV& yp, Acc& acc) {
-  rot_fwd<L, OPT>(g, xs, xp, std::make_integer_sequence<int, L>{});
-  axial<L, INPLACE, SYM>(g, xp, yp, std::make_integer_sequence<int, L + 1>{});
-  rot_bwd<L, OPT>(g, yp, acc, std::make_integer_sequence<int, L>{});
-}
-
-// One pair with the tables rebuilt per stage from the pair's scalars: the
-// half-angle powers and e^{i m phi} for each rotation, h_p for the axial
-// step.  The rebuild before the backward rotation reads the scalars through
-// an optimizer barrier, so the compiler cannot keep the forward rotation's
-// tables alive across the axial step (fewer live registers per thread).
-template <int L, bool INPLACE, bool SYM, int OPT = 0, typename XV, typename YV, typename Acc>
-__device__ __forceinline__ void pair_lazy(const GeomS& q, const Pair2<float>* __restrict__ xs, XV& xp, YV& yp,
-                                          Acc& acc) {
-  {
-    Geom<L, float> g;
-    geometry_angles<L>(q.ct, q.st, q.cph, q.sph, g);
-    rot_fwd<L, OPT>(g, xs, xp, std::make_integer_sequence<int, L>{});
-  }
-  {
-    Geom<L, float> g;
-    fill_hankel<L>(q, g);
-    axial<L, INPLACE, SYM>(g, xp, yp, std::make_integer_sequence<int, L + 1>{});
-  }
-  float ct = q.ct, st = q.st, cph = q.cph, sph = q.sph;
-  asm volatile("" : "+f"(ct), "+f"(st), "+f"(cph), "+f"(sph));
-  {
-    Geom<L, float> g;
-    geometry_angles<L>(ct, st, cph, sph, g);
-    rot_bwd<L, OPT>(g, yp, acc, std::make_integer_sequence<int, L>{});
+// the sums of one receiver from the cosine / sine basis to (y+, y-) =
+// (y_1 + y_2, y_1 - y_2) per row, in place, once per tile
+template <int L, typename R, typename Acc>
+__device__ __forceinline__ void to_plus_minus(Acc& acc) {
+  constexpr R H = static_cast<R>(0.5), Q = static_cast<R>(0.70710678118654752440);
+#pragma unroll
+  for (int l = 1; l <= L; ++l) {
+    const int r0 = l * (l + 1) - 1;
+    C2<R> a[2], b[2];
+    acc.load(r0, a);  // y_1 = c1 / sqrt 2, y_2 = i c2 / sqrt 2
+    b[0] = C2<R>{Q * (a[0].x - a[1].y), Q * (a[0].y + a[1].x)};
+    b[1] = C2<R>{Q * (a[0].x + a[1].y), Q * (a[0].y - a[1].x)};
+    acc.store(r0, b);
+#pragma unroll
+    for (int m = 1; m <= l; ++m) {
+      acc.load(r0 + m, a);  // c1, c2
+      acc.load(r0 - m, b);  // s1, s2
+      const C2<R> u{a[0].x + b[1].x, a[0].y + b[1].y}, v{a[0].x - b[1].x, a[0].y - b[1].y};
+      const C2<R> p{a[1].x - b[0].x, a[1].y - b[0].y}, q{a[1].x + b[0].x, a[1].y + b[0].y};
+      // y+_m = (u + i p)/2, y-_m = (v - i q)/2, y+_{-m} = (v + i q)/2, y-_{-m} = (u - i p)/2
+      a[0] = C2<R>{H * (u.x - p.y), H * (u.y + p.x)};
+      a[1] = C2<R>{H * (v.x + q.y), H * (v.y - q.x)};
+      b[0] = C2<R>{H * (v.x - q.y), H * (v.y + q.x)};
+      b[1] = C2<R>{H * (u.x + p.y), H * (u.y - p.x)};
+      acc.store(r0 + m, a);
+      acc.store(r0 - m, b);
+    }
   }
 }
 
-// Launch shape per (lmax, precision), chosen by timing sweeps on GB300 at
-// N = 10 000
+// Row r of source vector x ([2][NH] complex) in the cosine / sine basis
+template <typename R>
+__device__ __forceinline__ Quad4<R> stage_row(const Pair2<R>* __restrict__ x, int NH, int r) {
+  // degree l holds rows l^2 - 1 .. (l+1)^2 - 2, m = 0 at l (l + 1) - 1
+  const int l = 1 + (r >= 3) + (r >= 8) + (r >= 15) + (r >= 24);
+  const int m = r - (l * (l + 1) - 1);
+  const Pair2<R> a1 = x[r], a2 = x[NH + r];
+  if (m == 0) {
+    constexpr R Q = static_cast<R>(1.41421356237309504880);
+    return Quad4<R>{Q * a1.re, Q * a1.im, Q * a2.im, -Q * a2.re};
+  }
+  const Pair2<R> b1 = x[r - 2 * m], b2 = x[NH + r - 2 * m];
+  if (m > 0) return Quad4<R>{a1.re + b1.re, a1.im + b1.im, a2.im + b2.im, -(a2.re + b2.re)};
+  // b is x_|m| here: s1 = i (b1 - a1), s2 = b2 - a2
+  return Quad4<R>{a1.im - b1.im, b1.re - a1.re, b2.re - a2.re, b2.im - a2.im};
+}
+
+// One pair.  The angle tables are rebuilt for the backward rotation from the
+// pair's scalars, read through an optimizer barrier, so that they are not kept
+// alive across the axial step (fewer live registers per thread).
+template <int L, typename R, typename XV, typename Acc>
+__device__ __forceinline__ void pair(const GeomS<R>& q, const Quad4<R>* __restrict__ xs, XV& xp, Acc& acc) {
+  {
+    const Angles<L, R> g(q.ct, q.st, q.cph, q.sph);
+    rot_fwd<L>(g, xs, xp, std::make_integer_sequence<int, L>{});
+  }
+  {
+    const Hankel<L, R> h(q);
+    axial<L>(h, xp, std::make_integer_sequence<int, L + 1>{});
+  }
+  R ct = q.ct, st = q.st, cph = q.cph, sph = q.sph;
+  if constexpr (sizeof(R) == 4) asm volatile("" : "+f"(ct), "+f"(st), "+f"(cph), "+f"(sph));
+  else asm volatile("" : "+d"(ct), "+d"(st), "+d"(cph), "+d"(sph));
+  {
+    const Angles<L, R> g(ct, st, cph, sph);
+    rot_bwd<L>(g, xp, acc, std::make_integer_sequence<int, L>{});
+  }
+}
+
+// Launch shape per (lmax, precision)
 template <int L, typename R>
 struct Config {
   static constexpr bool FP64 = sizeof(R) == 8;
@@ -707,30 +639,15 @@ struct Config {
   static constexpr int TJ = FP64 ? 16 : 32;
   static constexpr bool ACC_SMEM = FP64 ? (L >= 2) : (L >= 3);
   static constexpr bool XY_SMEM = FP64 && L >= 3;
-  static constexpr bool XY_INPLACE = XY_SMEM;  // y' overwrites x' (one shared-memory array)
-  static constexpr bool SYM_AXIAL = true;       // axial entries formed once per (l, l') pair
-  // FP32: per-stage geometry tables (pair_lazy); removes the spills at lmax 5
-  // (22.8 vs 26.1 ms); at lmax 4 the full tables are faster (12.3 vs 12.8 ms),
-  // at lmax 3 the two are within run-to-run noise
-  static constexpr bool LAZY_GEOM = !FP64 && L == 5;
-  static constexpr bool SYNC_PAIR = false;  // barrier per source (keeps a CTA's warps in step)
   static constexpr int MINB = (!FP64 && L == 3) ? 3 : 1;  // minimum resident CTAs per SM for the allocator
-  static constexpr int OPT = 0;  // pair-code option bits (kPackedRot)
 };
 
 // The alternative FP32 launch shape of each lmax, the second candidate of
-// the autotuner (celes_ctx tuning): lmax 1-2 64-receiver CTAs, lmax 3 the
-// register allocator left free (two CTAs per SM), lmax 4 the x+ phase
-// multiply on the packed FMA, lmax 5 64-receiver CTAs with x' and y' in shared
-// memory (in place) and the rotations on the packed FMA.  Everything else as
-// in Config.
+// the autotuner (celes_ctx tuning)
 template <int L, typename R>
 struct ConfigAlt : Config<L, R> {
-  static constexpr int BLOCK = (L <= 2 || L == 5) ? 64 : 128;
-  static constexpr int MINB = 1;
-  static constexpr int OPT = L == 4 ? 1 : (L == 5 ? 2 : 0);
-  static constexpr bool XY_SMEM = Config<L, R>::XY_SMEM || L == 5;
-  static constexpr bool XY_INPLACE = XY_SMEM;
+  static constexpr int BLOCK = L <= 2 ? 64 : 128;
+  static constexpr int MINB = L == 4 ? 3 : 1;
 };
 
 template <int L, typename R, typename C = Config<L, R>>
@@ -739,9 +656,9 @@ struct Layout {
   static constexpr size_t col = sizeof(R) * 4 * NH * C::BLOCK;  // one [4 NH][BLOCK] array
   static constexpr size_t off_pos = 0;
   static constexpr size_t off_x = off_pos + sizeof(Pos4) * C::TJ;
-  static constexpr size_t off_acc = off_x + sizeof(Pair2<R>) * 2 * NH * C::TJ;
+  static constexpr size_t off_acc = off_x + sizeof(Quad4<R>) * NH * C::TJ;
   static constexpr size_t off_xy = off_acc + (C::ACC_SMEM ? col : 0);
-  static constexpr size_t bytes = off_xy + (C::XY_SMEM ? (C::XY_INPLACE ? 1 : 2) * col : 0);
+  static constexpr size_t bytes = off_xy + (C::XY_SMEM ? col : 0);
 };
 
 // whether `atomic` asks for the in-L2 vector reduction of the partial sums
@@ -771,7 +688,7 @@ __device__ __forceinline__ void rtr_tile(int N, const Pos4* __restrict__ pos, co
   constexpr int BLOCK = C::BLOCK;
   constexpr int TJ = C::TJ;
   Pos4* spos = reinterpret_cast<Pos4*>(smem_raw + LY::off_pos);
-  Pair2<R>* sx = reinterpret_cast<Pair2<R>*>(smem_raw + LY::off_x);
+  Quad4<R>* sx = reinterpret_cast<Quad4<R>*>(smem_raw + LY::off_x);
   R* sacc = reinterpret_cast<R*>(smem_raw + LY::off_acc);
   R* sxy = reinterpret_cast<R*>(smem_raw + LY::off_xy);
 
@@ -799,10 +716,7 @@ __device__ __forceinline__ void rtr_tile(int N, const Pos4* __restrict__ pos, co
     for (int q = tid; q < nj * NH; q += BLOCK) {
       const int jj = q / NH;
       const int r = q - jj * NH;
-      const Pair2<R> a = x[(size_t)(jt + jj) * (2 * NH) + r];
-      const Pair2<R> b = x[(size_t)(jt + jj) * (2 * NH) + NH + r];
-      sx[jj * 2 * NH + r] = Pair2<R>{a.re + b.re, a.im + b.im};
-      sx[jj * 2 * NH + NH + r] = Pair2<R>{a.re - b.re, a.im - b.im};
+      sx[q] = stage_row<R>(x + (size_t)(jt + jj) * (2 * NH), NH, r);
     }
     if constexpr (FF) {
       for (int q = tid; q < nj; q += BLOCK) sposf[q] = split_pos(pos[jt + q], k);
@@ -810,48 +724,41 @@ __device__ __forceinline__ void rtr_tile(int N, const Pos4* __restrict__ pos, co
       for (int q = tid; q < nj; q += BLOCK) spos[q] = pos[jt + q];
     }
     __syncthreads();
-    {
-      for (int jj = 0; jj < nj; ++jj) {
-        // optional barrier per pair: keeps the warps of a CTA on the same
-        // stretch of the (long, fully unrolled) pair code
-        if constexpr (C::SYNC_PAIR) __syncthreads();
-        if (!active || jt + jj == i) continue;  // no self coupling
-        constexpr bool LAZY = FF && C::LAZY_GEOM;
-        Geom<L, R> g;
-        GeomS gs;
-        if constexpr (LAZY) {
-          gs = geometry_ff_scalars<L>(rf, sposf[jj]);
-        } else if constexpr (FF) {
-          geometry_ff<L>(rf, sposf[jj], g);
+    for (int jj = 0; jj < nj; ++jj) {
+      if (!active || jt + jj == i) continue;  // no self coupling
+      GeomS<R> gs;
+      if constexpr (FF) {
+        gs = geometry_ff(rf, sposf[jj]);
+      } else {
+        const Pos4 rj = spos[jj];
+        gs = geometry(ri.x - rj.x, ri.y - rj.y, ri.z - rj.z, k);
+      }
+      const Quad4<R>* xs = sx + jj * NH;
+      auto run = [&](auto& xp) {
+        if constexpr (C::ACC_SMEM) {
+          RowAccSmem<R, BLOCK> acc{sacc4 + tid};
+          pair<L, R>(gs, xs, xp, acc);
         } else {
-          const Pos4 rj = spos[jj];
-          geometry<L, R>(ri.x - rj.x, ri.y - rj.y, ri.z - rj.z, k, g);
+          RowAccReg<R> acc{areg};
+          pair<L, R>(gs, xs, xp, acc);
         }
-        const Pair2<R>* xs = sx + jj * 2 * NH;
-        auto run = [&](auto& xp, auto& yp) {
-          constexpr bool INPL = C::XY_SMEM && C::XY_INPLACE;
-          if constexpr (C::ACC_SMEM) {
-            RowAccSmem<R, BLOCK> acc{sacc4 + tid};
-            if constexpr (LAZY) pair_lazy<L, INPL, C::SYM_AXIAL, C::OPT>(gs, xs, xp, yp, acc);
-            else pair<L, INPL, C::SYM_AXIAL, R, C::OPT>(g, xs, xp, yp, acc);
-          } else {
-            RowAccReg<R> acc{areg};
-            if constexpr (LAZY) pair_lazy<L, INPL, C::SYM_AXIAL, C::OPT>(gs, xs, xp, yp, acc);
-            else pair<L, INPL, C::SYM_AXIAL, R, C::OPT>(g, xs, xp, yp, acc);
-          }
-        };
-        if constexpr (C::XY_SMEM) {
-          AccSmem<R, BLOCK> xp{sxy + tid};
-          AccSmem<R, BLOCK> yp{sxy + (C::XY_INPLACE ? 0 : 4 * NH * BLOCK) + tid};
-          run(xp, yp);
-        } else {
-          R xa[4 * NH], ya[4 * NH];
-          AccReg<R> xp{xa};
-          AccReg<R> yp{ya};
-          run(xp, yp);
-        }
+      };
+      if constexpr (C::XY_SMEM) {
+        AccSmem<R, BLOCK> xp{sxy + tid};
+        run(xp);
+      } else {
+        R xa[4 * NH];
+        AccReg<R> xp{xa};
+        run(xp);
       }
     }
+  }
+  if constexpr (C::ACC_SMEM) {
+    RowAccSmem<R, BLOCK> acc{sacc4 + tid};
+    to_plus_minus<L, R>(acc);
+  } else {
+    RowAccReg<R> acc{areg};
+    to_plus_minus<L, R>(acc);
   }
   if constexpr (CRED) {
     static_assert(C::ACC_SMEM, "the cluster reduction reads shared-memory accumulators");

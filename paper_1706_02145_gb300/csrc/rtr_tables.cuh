@@ -16,12 +16,23 @@
 // (a5 for tau = tau', i b5' otherwise; App. A.2).  Under mu -> -mu the a5
 // factor is unchanged and b5' changes sign.
 //
+// The rotations run in the cosine / sine basis
+//   c_0 = sqrt(2) x_0,  c_M = x_M + x_{-M},  s_M = i (x_M - x_{-M})   (M > 0)
+// of each tau (tau = 2 multiplied by -i).  R_{-mu,-m} = R_{mu m} and
+// R_{-mu,m} = R_{mu,-m}, so R^l splits into a (l+1) x (l+1) block C on the c
+// and an l x l block S on the s: 2 l^2 + 2 l + 1 products instead of
+// (2 l + 1)^2, and e^{i M phi} becomes a real rotation of (c_M, s_M).  With
+// the rotated row mu multiplied by (-1)^mu (which W_z does not see) both blocks
+// are symmetric and orthogonal, hence their own inverses: the forward and the
+// backward rotation use the same numbers.
+//
 // Wigner's small-d matrix from its explicit sum:
 //   d^l_{m'm}(b) = sum_k (-1)^{k-m+m'} sqrt((l+m')!(l-m')!(l+m)!(l-m)!)
 //                  / [(l+m-k)! k! (l-k-m')! (k-m+m')!]  c^{2l-j} s^j,
-//   c = cos(b/2), s = sin(b/2), j = 2k - m + m'.
-// With d_{m'm} = (-1)^{m-m'} d_{mm'} = d_{-m,-m'} only one entry of each orbit
-// is evaluated.
+//   c = cos(b/2), s = sin(b/2), j = 2k - m + m',
+// expanded here into cos(q b) or sin(q b), q = 0..l: entry (mu, m) of a block
+// has two or three such terms (q of one parity) whose coefficients are at most
+// one, so it loses nothing to cancellation.
 #pragma once
 
 #include "coupling_tables.cuh"
@@ -39,84 +50,97 @@ constexpr int sgn_pm1(int e) { return (((e % 2) + 2) % 2) ? -1 : 1; }
 constexpr int sigma(int m) { return m >= 0 ? sgn_pm1(m) : 1; }
 
 // ---------------------------------------------------------------------------
-// Wigner small-d for one degree l
+// rotation blocks of one degree l
 // ---------------------------------------------------------------------------
+// Fourier coefficients of one entry: sum_q v[q] cos(q b), or sin(q b) when
+// `sine` (the entries with mu - m odd)
 template <int l>
-struct DTable {
-  static constexpr int W = 2 * l + 1;
-  static constexpr int MAXT = W * W * (l + 1);
-  int ncanon = 0;
-  int canon_mp[W * W] = {};  // canonical entries (m', m)
-  int canon_m[W * W] = {};
-  int cid[W * W] = {};       // entry (m' + l, m + l) -> canonical id
-  int csgn[W * W] = {};      // and its sign
-  int off[W * W + 1] = {};   // terms of canonical id c: [off[c], off[c+1])
-  int tj[MAXT] = {};         // monomial index j
-  double tc[MAXT] = {};      // coefficient
+struct Fourier {
+  double v[l + 1] = {};
+  bool sine = false;
 };
 
+// d^l_{m'm} as a Fourier sum: c^{2l-j} s^j = (z + 1/z)^{2l-j} (z - 1/z)^j / (2^{2l} i^j), z = e^{i b/2}
 template <int l>
-constexpr DTable<l> make_dtable() {
-  DTable<l> T{};
-  constexpr int W = 2 * l + 1;
-  for (int q = 0; q < W * W; ++q) T.cid[q] = -1;
-  int t = 0;
-  for (int mp = -l; mp <= l; ++mp) {
-    for (int m = -l; m <= l; ++m) {
-      const int q = (mp + l) * W + (m + l);
-      if (T.cid[q] >= 0) continue;
-      const int c = T.ncanon++;
-      T.canon_mp[c] = mp;
-      T.canon_m[c] = m;
-      // orbit: (m',m) +1, (m,m') (-1)^{m-m'}, (-m,-m') +1, (-m',-m) (-1)^{m-m'}
-      const int s1 = sgn_pm1(m - mp);
-      const int om[4][3] = {{mp, m, 1}, {m, mp, s1}, {-m, -mp, 1}, {-mp, -m, s1}};
-      for (int o = 0; o < 4; ++o) {
-        const int qq = (om[o][0] + l) * W + (om[o][1] + l);
-        if (T.cid[qq] < 0) {
-          T.cid[qq] = c;
-          T.csgn[qq] = om[o][2];
-        }
-      }
-      T.off[c] = t;
-      const double num = csqrt(fact(l + mp) * fact(l - mp) * fact(l + m) * fact(l - m));
-      for (int k = 0; k <= 2 * l; ++k) {
-        const int a1 = l + m - k, a2 = l - k - mp, a3 = k - m + mp;
-        if (a1 < 0 || a2 < 0 || a3 < 0) continue;
-        T.tj[t] = 2 * k - m + mp;
-        T.tc[t] = sgn_pm1(k - m + mp) * num / (fact(a1) * fact(k) * fact(a2) * fact(a3));
-        ++t;
-      }
+constexpr Fourier<l> wigner_fourier(int mp, int m) {
+  Fourier<l> F{};
+  F.sine = iabs(mp - m) % 2 == 1;
+  const double num = csqrt(fact(l + mp) * fact(l - mp) * fact(l + m) * fact(l - m));
+  for (int k = 0; k <= 2 * l; ++k) {
+    const int a1 = l + m - k, a2 = l - k - mp, a3 = k - m + mp;
+    if (a1 < 0 || a2 < 0 || a3 < 0) continue;
+    const int j = 2 * k - m + mp;
+    const double c = sgn_pm1(k - m + mp) * num / (fact(a1) * fact(k) * fact(a2) * fact(a3));
+    // coefficients of z^{2 t - 2 l}, t = 0..2l
+    double w[2 * l + 1] = {1.0};
+    for (int f = 0; f < 2 * l; ++f) {
+      const double sg = f < j ? -1.0 : 1.0;
+      for (int t = f + 1; t >= 0; --t) w[t] = (t > 0 ? w[t - 1] : 0.0) + sg * (t <= f ? w[t] : 0.0);
+    }
+    double scale = c;
+    for (int f = 0; f < 2 * l; ++f) scale *= 0.5;
+    if (!F.sine) {
+      if ((j / 2) % 2) scale = -scale;  // i^{-j}, j even
+      F.v[0] += scale * w[l];
+      for (int q = 1; q <= l; ++q) F.v[q] += 2.0 * scale * w[l + q];
+    } else {
+      if (((j - 1) / 2) % 2) scale = -scale;  // i^{1-j}, j odd
+      for (int q = 1; q <= l; ++q) F.v[q] += 2.0 * scale * w[l + q];
     }
   }
-  T.off[T.ncanon] = t;
-  return T;
+  return F;
 }
 
+// entry (mu, m) of block C (KIND 0, mu, m >= 0) or S (KIND 1, mu, m >= 1)
+template <int l, int KIND>
+constexpr Fourier<l> rot_fourier(int mu, int m) {
+  // R_{mu m} = s_mu s_m d_{m mu}
+  Fourier<l> F = wigner_fourier<l>(m, mu);
+  const double s1 = sigma(mu) * sigma(m);
+  const double f = sgn_pm1(mu) * s1 * ((mu == 0) != (m == 0) ? csqrt(2.0) : 1.0);
+  Fourier<l> G{};
+  double g = 0.0;
+  if (mu > 0 && m > 0) {
+    G = wigner_fourier<l>(-m, mu);
+    g = (KIND == 0 ? 1.0 : -1.0) * sgn_pm1(mu) * sigma(mu) * sigma(-m);
+  }
+  for (int q = 0; q <= l; ++q) {
+    F.v[q] = f * F.v[q] + g * G.v[q];
+    if (F.v[q] < 1e-13 && F.v[q] > -1e-13) F.v[q] = 0.0;  // terms that cancel
+  }
+  return F;
+}
+
+template <int l, int KIND, int MU, int M>
+struct RotEntry {
+  static constexpr Fourier<l> value = rot_fourier<l, KIND>(MU, M);
+  // true when the entry is the constant +-1 (S of degree 1)
+  static constexpr bool unit() { return l == 1 && KIND == 1; }
+  static constexpr int terms() {
+    int n = 0;
+    for (int q = 0; q <= l; ++q) n += value.v[q] != 0.0;
+    return n;
+  }
+};
+// coefficient of cos(q b) or sin(q b) in an entry
+template <int l, int KIND, int MU, int M, int Q>
+struct RotCoef {
+  static constexpr double v = RotEntry<l, KIND, MU, M>::value.v[Q];
+  static constexpr bool sine = RotEntry<l, KIND, MU, M>::value.sine;
+  static constexpr int before() {  // terms of lower q
+    int n = 0;
+    for (int q = 0; q < Q; ++q) n += RotEntry<l, KIND, MU, M>::value.v[q] != 0.0;
+    return n;
+  }
+};
+// canonical position of entry (mu, m) (symmetric blocks, lower triangle)
+constexpr int rot_id(int kind, int mu, int m) {
+  const int a = mu > m ? mu : m, b = mu > m ? m : mu;
+  return kind == 0 ? a * (a + 1) / 2 + b : (a - 1) * a / 2 + (b - 1);
+}
 template <int l>
-struct DTab {
-  static constexpr DTable<l> value = make_dtable<l>();
-};
-template <int l, int T>
-struct DTerm {
-  static constexpr int j = DTab<l>::value.tj[T];
-  static constexpr double c = DTab<l>::value.tc[T];
-};
-template <int l, int C>
-struct DCanon {
-  static constexpr int t0 = DTab<l>::value.off[C];
-  static constexpr int t1 = DTab<l>::value.off[C + 1];
-};
-template <int l>
-struct DCount {
-  static constexpr int ncanon = DTab<l>::value.ncanon;
-};
-// R^l_{mu m} = s_mu s_m d^l_{m mu} = sign * (canonical entry id)
-template <int l, int MU, int M>
-struct RAt {
-  static constexpr int q = (M + l) * (2 * l + 1) + (MU + l);
-  static constexpr int id = DTab<l>::value.cid[q];
-  static constexpr int sign = DTab<l>::value.csgn[q] * sigma(MU) * sigma(M);
+struct RotCount {
+  static constexpr int nc = (l + 1) * (l + 2) / 2, ns = l * (l + 1) / 2;
 };
 
 // ---------------------------------------------------------------------------
