@@ -865,12 +865,13 @@ extern "C" int celes_precond_build(celes_ctx* c, double edge) {
   }
   boff.push_back(c->N);
   const int64_t nb = static_cast<int64_t>(boff.size()) - 1;
-  std::vector<int64_t> moff(nb + 1, 0), toff(nb + 1, 0);
+  std::vector<int64_t> moff(nb + 1, 0), toff(nb + 1, 0), dims(nb);
   int64_t max_pairs = 0, max_dim = 0, max_tiles = 0;
   for (int64_t q = 0; q < nb; ++q) {
     const int64_t ns = boff[q + 1] - boff[q];
     const int64_t n = ns * c->nmax;
     const int64_t nt = (n + 31) / 32;
+    dims[q] = n;
     moff[q + 1] = moff[q] + n * n;
     toff[q + 1] = toff[q] + nt * 2048;
     max_pairs = std::max(max_pairs, ns * ns);
@@ -891,10 +892,22 @@ extern "C" int celes_precond_build(celes_ctx* c, double edge) {
   CK(launch_precond_assemble(c->L, nb, c->block_off.as<int64_t>(), c->mat_off.as<int64_t>(), c->perm.as<int>(),
                              c->pos.p, c->tq.as<double>(), c->k, c->mats.as<double>(), max_pairs, c->stream),
      "precond assembly");
-  CK(launch_precond_lu(nb, c->block_off.as<int64_t>(), c->mat_off.as<int64_t>(), c->nmax, c->mats.as<double>(),
+  PrecondPlan plan;
+  std::vector<int> order;
+  std::vector<int64_t> counts;
+  precond_plan(dims, plan, order, counts);
+  DevBuf plan_order, plan_off;
+  CK(plan_order.ensure(sizeof(int) * order.size()), "block order");
+  CK(plan_off.ensure(sizeof(int64_t) * counts.size()), "tile counts");
+  CK(cudaMemcpyAsync(plan_order.p, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, c->stream),
+     "h2d");
+  CK(cudaMemcpyAsync(plan_off.p, counts.data(), sizeof(int64_t) * counts.size(), cudaMemcpyHostToDevice, c->stream),
+     "h2d");
+  plan.order = plan_order.as<int>();
+  plan.off = plan_off.as<int64_t>();
+  CK(launch_precond_lu(plan, c->block_off.as<int64_t>(), c->mat_off.as<int64_t>(), c->nmax, c->mats.as<double>(),
                        c->piv.as<int>(), c->info.as<int>(), c->stream),
      "precond LU");
-  CK(launch_f64_to_f32(2 * moff[nb], c->mats.as<double>(), c->mats32.as<float>(), c->stream), "FP32 factors");
   CK(c->tile_off.ensure(sizeof(int64_t) * (nb + 1)), "tile offsets");
   CK(c->tinv.ensure(sizeof(double) * 2 * toff[nb]), "tile inverses");
   CK(c->tinv32.ensure(sizeof(float) * 2 * toff[nb]), "tile inverses (FP32 copy)");
@@ -904,7 +917,6 @@ extern "C" int celes_precond_build(celes_ctx* c, double edge) {
                                  c->tile_off.as<int64_t>(), c->nmax, c->mats.as<double>(), c->tinv.as<double>(),
                                  c->stream),
      "tile inverses");
-  CK(launch_f64_to_f32(2 * toff[nb], c->tinv.as<double>(), c->tinv32.as<float>(), c->stream), "FP32 tile inverses");
   c->precond_csize = precond_cluster_size(static_cast<double>(toff[nb] / 2048) / static_cast<double>(nb));
   // the apply's operator: the explicit inverses of L and U (FP64, and their
   // FP32 rounding), in place of the LU factors, when the block vectors fit in
@@ -913,7 +925,7 @@ extern "C" int celes_precond_build(celes_ctx* c, double edge) {
   if (precond_inverse_fits(static_cast<int>(max_dim))) {
     DevBuf inv;
     CK(inv.ensure(sizeof(double) * 2 * moff[nb]), "inverse factors");
-    CK(launch_precond_tri_inverse(nb, max_tiles, c->block_off.as<int64_t>(), c->mat_off.as<int64_t>(),
+    CK(launch_precond_tri_inverse(plan, c->block_off.as<int64_t>(), c->mat_off.as<int64_t>(),
                                   c->tile_off.as<int64_t>(), c->nmax, c->mats.as<double>(), c->tinv.as<double>(),
                                   inv.as<double>(), c->stream),
        "inverse factors");
@@ -922,6 +934,10 @@ extern "C" int celes_precond_build(celes_ctx* c, double edge) {
     std::swap(c->mats.bytes, inv.bytes);
     CK(launch_f64_to_f32(2 * moff[nb], c->mats.as<double>(), c->mats32.as<float>(), c->stream), "FP32 inverses");
     c->precond_inverse = true;
+  } else {
+    // the substitution form reads the factors and their diagonal tiles' inverses
+    CK(launch_f64_to_f32(2 * moff[nb], c->mats.as<double>(), c->mats32.as<float>(), c->stream), "FP32 factors");
+    CK(launch_f64_to_f32(2 * toff[nb], c->tinv.as<double>(), c->tinv32.as<float>(), c->stream), "FP32 tile inverses");
   }
   CK(c->pivperm.ensure(sizeof(int) * c->N * c->nmax), "pivot permutation");
   CK(launch_pivot_perm(nb, c->block_off.as<int64_t>(), c->nmax, c->piv.as<int>(), c->pivperm.as<int>(), c->stream),

@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <vector>
 
 #include "../../include/celes.h"
 #include "per_device.h"
@@ -114,7 +115,26 @@ cudaError_t launch_gemm_bf16_tn(int M, int N, int K, const void* A, int lda, con
 cudaError_t launch_precond_assemble(int L, int64_t nblocks, const int64_t* block_off, const int64_t* mat_off,
                                     const int* perm, const void* pos, const double* tq, double k, double* mats,
                                     int64_t max_pairs, cudaStream_t st);
-cudaError_t launch_precond_lu(int64_t nblocks, const int64_t* block_off, const int64_t* mat_off, int nmax,
+// The steps that all blocks take together: blocks in descending order of size
+// (`order`), in step k the first `active` of them have a row tile k.  Every
+// `*_off` is the start in `off` of that step's table, which counts the CTAs of
+// the blocks before each active one; the field beside it is their total.
+struct PrecondPlan {
+  struct Step {
+    int active;
+    int64_t columns_off, columns;      // column tiles other than the panel
+    int64_t tiles_off, tiles;          // tiles of the trailing update
+    int64_t rows_off, rows;            // tiles of one row of both inverses
+    int64_t inv_tiles_off, inv_tiles;  // tiles of the inverses' update
+  };
+  std::vector<Step> steps;
+  std::vector<int64_t> dims;     // of the blocks in that order
+  const int* order = nullptr;    // device
+  const int64_t* off = nullptr;  // device
+};
+void precond_plan(const std::vector<int64_t>& dims, PrecondPlan& plan, std::vector<int>& order,
+                  std::vector<int64_t>& off);
+cudaError_t launch_precond_lu(const PrecondPlan& plan, const int64_t* block_off, const int64_t* mat_off, int nmax,
                               double* mats, int* piv, int* info, cudaStream_t st);
 // tile_off/tinv/tinv32: explicit inverses of the 32 x 32 diagonal tiles of
 // each block's L and U (launch_precond_tile_inverse; tinv = nullptr selects
@@ -127,9 +147,9 @@ cudaError_t launch_precond_apply(int64_t nblocks, const int64_t* block_off, cons
                                  const float* tinv32 = nullptr, int csize = 0, bool inverse = false);
 // FP64 explicit inverses of each block's L and U from its FP64 LU factors and
 // FP64 tile inverses (same layout as the factors)
-cudaError_t launch_precond_tri_inverse(int64_t nblocks, int64_t max_tiles, const int64_t* block_off,
-                                       const int64_t* mat_off, const int64_t* tile_off, int nmax, const double* lu,
-                                       const double* tinv, double* inv, cudaStream_t st);
+cudaError_t launch_precond_tri_inverse(const PrecondPlan& plan, const int64_t* block_off, const int64_t* mat_off,
+                                       const int64_t* tile_off, int nmax, const double* lu, const double* tinv,
+                                       double* inv, cudaStream_t st);
 bool precond_inverse_fits(int max_block_dim);
 cudaError_t launch_precond_tile_inverse(int64_t nblocks, int64_t max_tiles, const int64_t* block_off,
                                         const int64_t* mat_off, const int64_t* tile_off, int nmax, const double* mats,

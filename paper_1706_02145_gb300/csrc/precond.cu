@@ -10,7 +10,10 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
+#include <numeric>
+#include <vector>
 
 #include "cmath.cuh"
 #include "coupling_kernel.cuh"
@@ -19,32 +22,192 @@
 namespace celes {
 
 // ---------------------------------------------------------------------------
-// batched LU with partial pivoting: one CTA per block, right-looking
+// batched LU with partial pivoting, blocked by 32 columns
+//
+// FP64 arithmetic bounds the build: 8/3 n^3 flops for the factors of a block
+// and as many for their inverses, on a pipe that does 1.7 FMAs per clock and
+// SM.  Blocks differ in size by an order of magnitude, so one CTA per block
+// leaves the GPU to the largest one.  All blocks go through the same panel
+// step together instead: (1) the panel's 32 columns, one row per thread in
+// registers, a cluster of up to 8 CTAs per block; (2) the row interchanges and
+// U_12, one CTA per 32 columns; (3) the trailing update, one CTA per 32 x 32
+// tile of any block, which is nearly all of the work and spreads over the whole
+// GPU.  Tiles of 32 move 0.25 bytes per flop, far below what this FP64 rate
+// asks of L2.  Measured on GB300, 175 blocks of up to 1 248 unknowns (77
+// GFLOP): the whole build 1 090-1 260 ms with one unblocked CTA per block (859
+// ms of it the factors), 133 ms now (about 65 ms of it the factors: the FP64
+// pipe at its 1.05 TFLOP/s during the update).
 // ---------------------------------------------------------------------------
-constexpr int kLuThreads = 512;
+namespace cg = cooperative_groups;
 
-__global__ void __launch_bounds__(kLuThreads) precond_lu_kernel(const int64_t* __restrict__ block_off,
-                                                                const int64_t* __restrict__ mat_off, int nmax,
-                                                                double2* __restrict__ mats, int* __restrict__ piv,
-                                                                int* __restrict__ info) {
-  const int64_t q = blockIdx.x;
+constexpr int kTile = 32;
+constexpr int kPanelMaxCluster = 8;
+constexpr int kTileThreads = 256;
+
+// tile `t` of a step, of the block that holds it: blocks are listed in `order`
+// and `off[s]` counts the tiles of the blocks before order[s]
+__device__ __forceinline__ int tile_block(const int64_t* __restrict__ off, int nact, int64_t t) {
+  int lo = 0, hi = nact - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (off[mid] <= t) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// (1) panel of columns kb .. kb + 31 of the blocks order[0 .. grid / C - 1];
+// grid: clusters of C CTAs, one per block; the panel has at most C * THREADS
+// rows.  The owner of a candidate row also inverts its pivot, so that the rows
+// below are scaled by a product (every row dividing for itself took as long as
+// the rest of the column's work).
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
+    precond_panel_kernel(int64_t kb, const int* __restrict__ order, const int64_t* __restrict__ block_off,
+                         const int64_t* __restrict__ mat_off, int nmax, double2* __restrict__ mats,
+                         int* __restrict__ piv, int* __restrict__ info) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = static_cast<int>(cluster.num_blocks());
+  const int rank = static_cast<int>(cluster.block_rank());
+  const int q = order[blockIdx.x / C];
   const int64_t n = (block_off[q + 1] - block_off[q]) * nmax;
   double2* A = mats + mat_off[q];
   int* pv = piv + block_off[q] * nmax;
-  __shared__ double sval[kLuThreads / 32];
-  __shared__ int sidx[kLuThreads / 32];
+  __shared__ double wval[THREADS / 32];
+  __shared__ int widx[THREADS / 32];
+  // candidates of every CTA and the row at the pivot position, double buffered
+  __shared__ double cval[2][kPanelMaxCluster];
+  __shared__ int cidx[2][kPanelMaxCluster];
+  __shared__ double2 crow[2][kPanelMaxCluster][kTile];
+  __shared__ double2 cinv[2][kPanelMaxCluster];
+  __shared__ double2 krow[2][kTile];
+  const int tid = threadIdx.x;
+  const int tb = static_cast<int>(n - kb < kTile ? n - kb : kTile);
+  const int i = static_cast<int>(kb) + rank * THREADS + tid;  // this thread's row
+  const bool live = i < n;
+  double2 a[kTile];
+#pragma unroll
+  for (int t = 0; t < kTile; ++t) a[t] = live && t < tb ? A[i + (kb + t) * n] : make_double2(0.0, 0.0);
+  if (kb == 0 && rank == 0 && tid == 0) info[q] = 0;
+  if (C > 1) cluster.sync();  // every CTA has started before any writes into another's shared memory
+#pragma unroll
+  for (int c = 0; c < kTile; ++c) {
+    if (c < tb) {
+      const int kk = static_cast<int>(kb) + c, par = c & 1;
+      double best = live && i >= kk ? fabs(a[c].x) + fabs(a[c].y) : -1.0;
+      if (!(best >= 0.0)) best = -1.0;  // NaN never wins
+      int bi = i;
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ob > best || (ob == best && oi < bi)) {
+          best = ob;
+          bi = oi;
+        }
+      }
+      if ((tid & 31) == 0) {
+        wval[tid >> 5] = best;
+        widx[tid >> 5] = bi;
+      }
+      __syncthreads();
+      best = wval[0];
+      bi = widx[0];
+#pragma unroll
+      for (int w = 1; w < THREADS / 32; ++w) {
+        if (wval[w] > best) {  // rows ascend with w: ties keep the first
+          best = wval[w];
+          bi = widx[w];
+        }
+      }
+      if (i == bi || i == kk) {
+        const cd pv_c = mkc(a[c].x, a[c].y);
+        const cd rp = i == bi && abs2(pv_c) > 0.0 ? mkc(1.0) / pv_c : mkc(0.0);
+        for (int dst = 0; dst < C; ++dst) {
+          double2* cr = C > 1 ? cluster.map_shared_rank(&crow[par][rank][0], dst) : &crow[par][rank][0];
+          double2* kr = C > 1 ? cluster.map_shared_rank(&krow[par][0], dst) : &krow[par][0];
+          if (i == bi) {
+            double* cv = C > 1 ? cluster.map_shared_rank(&cval[par][rank], dst) : &cval[par][rank];
+            int* ci = C > 1 ? cluster.map_shared_rank(&cidx[par][rank], dst) : &cidx[par][rank];
+            double2* cp = C > 1 ? cluster.map_shared_rank(&cinv[par][rank], dst) : &cinv[par][rank];
+            *cv = best;
+            *ci = bi;
+            *cp = make_double2(rp.re, rp.im);
+#pragma unroll
+            for (int t = 0; t < kTile; ++t) cr[t] = a[t];
+          }
+          if (i == kk) {
+#pragma unroll
+            for (int t = 0; t < kTile; ++t) kr[t] = a[t];
+          }
+        }
+      }
+      if (C > 1) cluster.sync();
+      else __syncthreads();
+      int b = 0;
+      for (int r = 1; r < C; ++r)
+        if (cval[par][r] > cval[par][b]) b = r;
+      const bool none = !(cval[par][b] > 0.0);
+      const int p = cval[par][b] < 0.0 ? kk : cidx[par][b];
+      const double2* prow = cval[par][b] < 0.0 ? krow[par] : crow[par][b];
+      if (rank == 0 && tid == 0) {
+        pv[kk] = p;
+        if (none && info[q] == 0) info[q] = kk + 1;
+      }
+      if (p != kk) {
+        if (i == kk) {
+#pragma unroll
+          for (int t = 0; t < kTile; ++t) a[t] = prow[t];
+        } else if (i == p) {
+#pragma unroll
+          for (int t = 0; t < kTile; ++t) a[t] = krow[par][t];
+        }
+      }
+      if (live && i > kk) {
+        const double2 rp = cval[par][b] < 0.0 ? make_double2(0.0, 0.0) : cinv[par][b];
+        const cd l = mkc(a[c].x, a[c].y) * mkc(rp.x, rp.y);
+        a[c] = make_double2(l.re, l.im);
+#pragma unroll
+        for (int t = c + 1; t < kTile; ++t) {
+          const double2 u = prow[t];
+          a[t].x = fma(-l.re, u.x, fma(l.im, u.y, a[t].x));
+          a[t].y = fma(-l.re, u.y, fma(-l.im, u.x, a[t].y));
+        }
+      }
+    }
+  }
+  if (live) {
+#pragma unroll
+    for (int t = 0; t < kTile; ++t)
+      if (t < tb) A[i + (kb + t) * n] = a[t];
+  }
+  if (C > 1) cluster.sync();  // no CTA leaves while others may still read what it wrote into them
+}
+
+// (1), panels of more rows than a cluster holds: one CTA per block, in global memory
+__global__ void __launch_bounds__(1024) precond_panel_tall_kernel(int64_t kb, const int* __restrict__ order,
+                                                                  const int64_t* __restrict__ block_off,
+                                                                  const int64_t* __restrict__ mat_off, int nmax,
+                                                                  double2* __restrict__ mats, int* __restrict__ piv,
+                                                                  int* __restrict__ info) {
+  const int q = order[blockIdx.x];
+  const int64_t n = (block_off[q + 1] - block_off[q]) * nmax;
+  double2* A = mats + mat_off[q];
+  int* pv = piv + block_off[q] * nmax;
+  __shared__ double sval[32];
+  __shared__ int sidx[32];
   __shared__ int s_p;
-  __shared__ double2 s_pivot;
-  if (threadIdx.x == 0) info[q] = 0;
-  for (int64_t kk = 0; kk < n; ++kk) {
-    // pivot search in column kk
+  __shared__ double2 s_row[kTile];
+  const int tb = static_cast<int>(n - kb < kTile ? n - kb : kTile);
+  if (kb == 0 && threadIdx.x == 0) info[q] = 0;
+  for (int c = 0; c < tb; ++c) {
+    const int64_t kk = kb + c;
     double best = -1.0;
     int bi = static_cast<int>(kk);
     for (int64_t i = kk + threadIdx.x; i < n; i += blockDim.x) {
       const double2 v = A[i + kk * n];
-      const double a = fabs(v.x) + fabs(v.y);
-      if (a > best) {
-        best = a;
+      const double x = fabs(v.x) + fabs(v.y);
+      if (x > best) {
+        best = x;
         bi = static_cast<int>(i);
       }
     }
@@ -64,7 +227,7 @@ __global__ void __launch_bounds__(kLuThreads) precond_lu_kernel(const int64_t* _
     if (threadIdx.x == 0) {
       double b = -1.0;
       int ix = static_cast<int>(kk);
-      for (int w = 0; w < kLuThreads / 32; ++w) {
+      for (int w = 0; w < static_cast<int>(blockDim.x) / 32; ++w) {
         if (sval[w] > b || (sval[w] == b && sidx[w] < ix)) {
           b = sval[w];
           ix = sidx[w];
@@ -76,49 +239,304 @@ __global__ void __launch_bounds__(kLuThreads) precond_lu_kernel(const int64_t* _
     }
     __syncthreads();
     const int64_t p = s_p;
-    // swap rows kk and p over all columns
-    if (p != kk) {
-      for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-        const double2 t = A[kk + j * n];
-        A[kk + j * n] = A[p + j * n];
-        A[p + j * n] = t;
+    if (threadIdx.x < tb) {
+      const int64_t col = (kb + threadIdx.x) * n;
+      const double2 u = A[p + col];
+      s_row[threadIdx.x] = u;
+      if (p != kk) {
+        A[p + col] = A[kk + col];
+        A[kk + col] = u;
       }
     }
     __syncthreads();
-    if (threadIdx.x == 0) s_pivot = A[kk + kk * n];
-    __syncthreads();
-    const cd piv_v = mkc(s_pivot.x, s_pivot.y);
-    const bool ok = abs2(piv_v) > 0.0;
-    // scale the column below the pivot
+    const cd pvt = mkc(s_row[c].x, s_row[c].y);
+    const bool ok = abs2(pvt) > 0.0;
     for (int64_t i = kk + 1 + threadIdx.x; i < n; i += blockDim.x) {
       const double2 v = A[i + kk * n];
-      const cd l = ok ? mkc(v.x, v.y) / piv_v : mkc(0.0);
+      const cd l = ok ? mkc(v.x, v.y) / pvt : mkc(0.0);
       A[i + kk * n] = make_double2(l.re, l.im);
-    }
-    __syncthreads();
-    // rank-1 update of the trailing matrix, threads over rows (coalesced)
-    const int64_t m = n - kk - 1;
-    for (int64_t t = threadIdx.x; t < m * m; t += blockDim.x) {
-      const int64_t jj = t / m, ii = t - jj * m;
-      const int64_t i = kk + 1 + ii, j = kk + 1 + jj;
-      const double2 l = A[i + kk * n];
-      const double2 u = A[kk + j * n];
-      double2 a = A[i + j * n];
-      a.x -= l.x * u.x - l.y * u.y;
-      a.y -= l.x * u.y + l.y * u.x;
-      A[i + j * n] = a;
+      for (int t = c + 1; t < tb; ++t) {
+        double2 x = A[i + (kb + t) * n];
+        const double2 u = s_row[t];
+        x.x = fma(-l.re, u.x, fma(l.im, u.y, x.x));
+        x.y = fma(-l.re, u.y, fma(-l.im, u.x, x.y));
+        A[i + (kb + t) * n] = x;
+      }
     }
     __syncthreads();
   }
 }
 
-cudaError_t launch_precond_lu(int64_t nblocks, const int64_t* block_off, const int64_t* mat_off, int nmax,
+// (2) the panel's row interchanges on 32 other columns of a block, and, right
+// of the panel, U_12 = L_11^{-1} A_12 by forward substitution.  One CTA per
+// column tile; lanes are columns, warps take the rows in turn.
+__global__ void __launch_bounds__(kTileThreads)
+    precond_swap_solve_kernel(int64_t kb, int nact, const int* __restrict__ order, const int64_t* __restrict__ off,
+                              const int64_t* __restrict__ block_off, const int64_t* __restrict__ mat_off, int nmax,
+                              double2* __restrict__ mats, const int* __restrict__ piv) {
+  const int s = tile_block(off, nact, blockIdx.x);
+  const int q = order[s];
+  const int64_t n = (block_off[q + 1] - block_off[q]) * nmax;
+  double2* A = mats + mat_off[q];
+  int64_t ct = blockIdx.x - off[s];
+  if (ct >= kb / kTile) ++ct;  // every column tile but the panel's own
+  const int tb = static_cast<int>(n - kb < kTile ? n - kb : kTile);
+  const int cb = static_cast<int>(n - ct * kTile < kTile ? n - ct * kTile : kTile);
+  __shared__ double2 top[kTile][kTile + 1];  // [row][column] of rows kb ..
+  __shared__ double2 far[kTile][kTile + 1];  // rows below the panel's top tile that a swap touches; then L_11
+  __shared__ int prow[kTile], slot[kTile];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (wid == 0) {
+    const int p = lane < tb ? piv[block_off[q] * nmax + kb + lane] : static_cast<int>(kb) + lane;
+    prow[lane] = p;
+    slot[lane] = __ffs(__match_any_sync(0xffffffffu, p)) - 1;  // the first interchange with the same row
+  }
+  __syncthreads();
+  // rows along the lanes: coalesced
+  for (int e = tid; e < kTile * kTile; e += kTileThreads) {
+    const int c = e >> 5, r = e & 31;
+    const double2* col = A + (ct * kTile + c) * n;
+    if (c < cb && r < tb) {
+      top[r][c] = col[kb + r];
+      if (slot[r] == r && prow[r] >= kb + tb) far[r][c] = col[prow[r]];
+    }
+  }
+  __syncthreads();
+  if (wid == 0 && lane < cb) {
+    for (int k = 0; k < tb; ++k) {
+      const int p = prow[k];
+      if (p == kb + k) continue;
+      double2& x = p < kb + tb ? top[p - kb][lane] : far[slot[k]][lane];
+      const double2 t = top[k][lane];
+      top[k][lane] = x;
+      x = t;
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < kTile * kTile; e += kTileThreads) {
+    const int c = e >> 5, r = e & 31;
+    if (c < cb && r < tb && slot[r] == r && prow[r] >= kb + tb) A[prow[r] + (ct * kTile + c) * n] = far[r][c];
+  }
+  if (ct * kTile > kb) {
+    __syncthreads();
+    for (int e = tid; e < kTile * kTile; e += kTileThreads) {
+      const int c = e >> 5, r = e & 31;
+      if (r < tb && c < tb) far[r][c] = A[(kb + r) + (kb + c) * n];
+    }
+    __syncthreads();
+    for (int j = 0; j < tb; ++j) {
+      const double2 u = top[j][lane];
+      for (int r = wid; r < tb; r += kTileThreads / 32) {
+        if (r > j) {
+          const double2 l = far[r][j];
+          double2 x = top[r][lane];
+          x.x = fma(-l.x, u.x, fma(l.y, u.y, x.x));
+          x.y = fma(-l.x, u.y, fma(-l.y, u.x, x.y));
+          top[r][lane] = x;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  for (int e = tid; e < kTile * kTile; e += kTileThreads) {
+    const int c = e >> 5, r = e & 31;
+    if (c < cb && r < tb) A[kb + r + (ct * kTile + c) * n] = top[r][c];
+  }
+}
+
+// A complex 32 x 32 tile as three real ones, [col][row]: real and imaginary
+// part and their sum.  Products take three real multiplications instead of
+// four (Re = P1 - P2, Im = P3 - P1 - P2 with P1 = ar br, P2 = ai bi, P3 =
+// (ar + ai)(br + bi)): the FP64 pipe is all that these kernels wait for (the
+// two updates 119 -> 98 ms at the size above; the application's error against
+// 64 bits 1.6e-15 -> 1.5e-15; the FP64 mma runs no faster than the FMA here,
+// 1.04 against 1.00 TFLOP/s).
+struct Tile3 {
+  double re[kTile][kTile + 1], im[kTile][kTile + 1], sum[kTile][kTile + 1];
+  __device__ __forceinline__ void set(int c, int r, double2 v) {
+    re[c][r] = v.x;
+    im[c][r] = v.y;
+    sum[c][r] = v.x + v.y;
+  }
+};
+// stage tile (ti, tk) of a column-major n x n matrix, zero outside the block
+__device__ __forceinline__ void load_tile(Tile3& dst, const double2* __restrict__ M, int64_t n, int64_t ti,
+                                          int64_t tk) {
+  const int64_t r0 = ti * kTile, c0 = tk * kTile;
+  for (int e = threadIdx.x; e < kTile * kTile; e += kTileThreads) {
+    const int c = e >> 5, r = e & 31;
+    dst.set(c, r, r0 + r < n && c0 + c < n ? M[(r0 + r) + (c0 + c) * n] : make_double2(0.0, 0.0));
+  }
+}
+// the inverse of a diagonal tile (32 x 32 column-major, identity-padded)
+__device__ __forceinline__ void load_tinv(Tile3& dst, const double2* __restrict__ Ti) {
+  for (int e = threadIdx.x; e < kTile * kTile; e += kTileThreads) dst.set(e >> 5, e & 31, Ti[e]);
+}
+// acc[u] += S (as xs)[r][4 g + u], thread (r, g) = (tid & 31, tid >> 5)
+template <int S>
+__device__ __forceinline__ void tile_product(const Tile3& as, const Tile3& xs, double2 (&acc)[4]) {
+  const int r = threadIdx.x & 31, g = threadIdx.x >> 5;
+  double p1[4] = {}, p2[4] = {}, p3[4] = {};
+#pragma unroll 8
+  for (int m = 0; m < kTile; ++m) {
+    const double ar = as.re[m][r], ai = as.im[m][r], at = as.sum[m][r];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      p1[u] = fma(ar, xs.re[4 * g + u][m], p1[u]);
+      p2[u] = fma(ai, xs.im[4 * g + u][m], p2[u]);
+      p3[u] = fma(at, xs.sum[4 * g + u][m], p3[u]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const double re = p1[u] - p2[u], im = p3[u] - p1[u] - p2[u];
+    acc[u].x = S > 0 ? acc[u].x + re : acc[u].x - re;
+    acc[u].y = S > 0 ? acc[u].y + im : acc[u].y - im;
+  }
+}
+
+// (3) A_22 -= L_21 U_12, one CTA per 32 x 32 tile
+__global__ void __launch_bounds__(kTileThreads)
+    precond_update_kernel(int64_t kt, int nact, const int* __restrict__ order, const int64_t* __restrict__ off,
+                          const int64_t* __restrict__ block_off, const int64_t* __restrict__ mat_off, int nmax,
+                          double2* __restrict__ mats) {
+  const int s = tile_block(off, nact, blockIdx.x);
+  const int q = order[s];
+  const int64_t n = (block_off[q + 1] - block_off[q]) * nmax;
+  const int64_t rem = (n + kTile - 1) / kTile - kt - 1;
+  const int64_t t = blockIdx.x - off[s];
+  const int64_t ti = kt + 1 + t % rem, tj = kt + 1 + t / rem;
+  double2* A = mats + mat_off[q];
+  extern __shared__ Tile3 tiles3[];
+  Tile3& as = tiles3[0];
+  Tile3& xs = tiles3[1];
+  load_tile(as, A, n, ti, kt);
+  load_tile(xs, A, n, kt, tj);
+  const int r = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int64_t row = ti * kTile + r, col = tj * kTile + 4 * g;
+  double2 acc[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    acc[u] = row < n && col + u < n ? A[row + (col + u) * n] : make_double2(0.0, 0.0);
+  __syncthreads();
+  tile_product<-1>(as, xs, acc);
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    if (row < n && col + u < n) A[row + (col + u) * n] = acc[u];
+}
+
+// the two staged tiles are above the default limit of 48 KB
+template <typename K>
+static cudaError_t tile_smem(K* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(2 * sizeof(Tile3)));
+}
+
+// The blocks of one panel step by the rows they have left, each class with the
+// smallest cluster that holds them: a launch has one cluster size, and eight
+// CTAs for the small blocks too would be nine waves of mostly idle rows.  The
+// classes run side by side on streams of their own (with the reciprocal pivots
+// and the three-product tiles, this took the build of the 175 blocks above from
+// 173 to 133 ms).
+struct PanelClass {
+  int64_t rows;
+  int threads, cluster;
+};
+constexpr PanelClass kPanelClasses[] = {{128, 128, 1}, {256, 128, 2}, {512, 128, 4}, {1024, 128, 8}, {2048, 256, 8}};
+constexpr int kPanelStreams = 5;
+
+// side streams and events of one build, given back at its end
+struct PanelStreams {
+  cudaStream_t side[kPanelStreams] = {};
+  cudaEvent_t fork = nullptr, join[kPanelStreams] = {};
+  cudaError_t init() {
+    cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    for (int q = 0; q < kPanelStreams && e == cudaSuccess; ++q) {
+      e = cudaStreamCreateWithFlags(&side[q], cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[q], cudaEventDisableTiming);
+    }
+    return e;
+  }
+  ~PanelStreams() {
+    if (fork) cudaEventDestroy(fork);
+    for (int q = 0; q < kPanelStreams; ++q) {
+      if (side[q]) cudaStreamDestroy(side[q]);  // its work is done first
+      if (join[q]) cudaEventDestroy(join[q]);
+    }
+  }
+};
+
+template <int THREADS>
+static cudaError_t launch_panel(int64_t kb, int nblk, int C, const int* order, const int64_t* block_off,
+                                const int64_t* mat_off, int nmax, double2* M, int* piv, int* info, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(nblk * C));
+  cfg.blockDim = dim3(THREADS);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = static_cast<unsigned>(C);
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, precond_panel_kernel<THREADS>, kb, order, block_off, mat_off, nmax, M, piv, info);
+}
+
+cudaError_t launch_precond_lu(const PrecondPlan& plan, const int64_t* block_off, const int64_t* mat_off, int nmax,
                               double* mats, int* piv, int* info, cudaStream_t st) {
-  if (nblocks <= 0) return cudaSuccess;
-  precond_lu_kernel<<<static_cast<unsigned>(nblocks), kLuThreads, 0, st>>>(
-      block_off, mat_off, nmax, reinterpret_cast<double2*>(mats), piv, info);
-  note_launch();
-  return cudaGetLastError();
+  double2* M = reinterpret_cast<double2*>(mats);
+  PanelStreams ps;
+  cudaError_t e = tile_smem(precond_update_kernel);
+  if (e == cudaSuccess) e = ps.init();
+  for (size_t k = 0; k < plan.steps.size() && e == cudaSuccess; ++k) {
+    const PrecondPlan::Step& p = plan.steps[k];
+    const int64_t kb = static_cast<int64_t>(k) * kTile;
+    e = cudaEventRecord(ps.fork, st);
+    // blocks are in descending order of size: each class is a run of them
+    int side = 0;
+    for (int s = 0; s < p.active && e == cudaSuccess;) {
+      const int64_t rows = plan.dims[s] - kb;
+      const PanelClass* pc = nullptr;
+      for (const PanelClass& c : kPanelClasses)
+        if (!pc && rows <= c.rows) pc = &c;
+      int end = s + 1;
+      const int64_t least = !pc ? kPanelClasses[4].rows : (pc == kPanelClasses ? 0 : pc[-1].rows);
+      while (end < p.active && plan.dims[end] - kb > least) ++end;
+      // the last class stays on the main stream
+      const bool fork = end < p.active;
+      const cudaStream_t to = fork ? ps.side[side] : st;
+      if (fork) e = cudaStreamWaitEvent(to, ps.fork, 0);
+      if (e != cudaSuccess) break;
+      if (!pc) {
+        precond_panel_tall_kernel<<<static_cast<unsigned>(end - s), 1024, 0, to>>>(kb, plan.order + s, block_off,
+                                                                                   mat_off, nmax, M, piv, info);
+        e = cudaGetLastError();
+      } else if (pc->threads == 128) {
+        e = launch_panel<128>(kb, end - s, pc->cluster, plan.order + s, block_off, mat_off, nmax, M, piv, info, to);
+      } else {
+        e = launch_panel<256>(kb, end - s, pc->cluster, plan.order + s, block_off, mat_off, nmax, M, piv, info, to);
+      }
+      note_launch();
+      if (fork && e == cudaSuccess) e = cudaEventRecord(ps.join[side], to);
+      if (fork) ++side;
+      s = end;
+    }
+    for (int q = 0; q < side && e == cudaSuccess; ++q) e = cudaStreamWaitEvent(st, ps.join[q], 0);
+    if (e != cudaSuccess) break;
+    if (p.columns > 0) {
+      precond_swap_solve_kernel<<<static_cast<unsigned>(p.columns), kTileThreads, 0, st>>>(
+          kb, p.active, plan.order, plan.off + p.columns_off, block_off, mat_off, nmax, M, piv);
+      note_launch();
+    }
+    if (p.tiles > 0) {
+      precond_update_kernel<<<static_cast<unsigned>(p.tiles), kTileThreads, 2 * sizeof(Tile3), st>>>(
+          static_cast<int64_t>(k), p.active, plan.order, plan.off + p.tiles_off, block_off, mat_off, nmax, M);
+      note_launch();
+    }
+    e = cudaGetLastError();
+  }
+  return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -259,7 +677,6 @@ __global__ void __launch_bounds__(256) precond_apply_kernel(const int64_t* __res
 // GEMV per tile, the factor traffic is spread over C SMs, and blocks much
 // fewer than SMs still fill the GPU.
 // ---------------------------------------------------------------------------
-namespace cg = cooperative_groups;
 
 // explicit inverses of the diagonal tiles of each block's LU (unit lower L,
 // upper U), column-major 32 x 32 each, tiles beyond the block padded with the
@@ -432,110 +849,88 @@ __global__ void __launch_bounds__(kApplyThreads) precond_apply_cluster_kernel(
 // inverses in FP64 keeps the FP32 copy within FP32 rounding of the FP64 one.
 // ---------------------------------------------------------------------------
 
-// Column tile j of L^{-1} (z = 0) or U^{-1} (z = 1) of block q, by blocked
-// substitution: X_jj = (tile inverse), and for the other row tiles i (below j
-// for L, above for U) X_ij = -inv(T_ii) sum_k T_ik X_kj over the tiles k
-// between them.  One CTA of 256 threads per (column tile, block, factor);
-// thread (row r, column group g) owns X[r][4g .. 4g + 3].
-template <typename F>
-__global__ void __launch_bounds__(256) precond_tri_inverse_kernel(const int64_t* __restrict__ block_off,
-                                                                  const int64_t* __restrict__ mat_off,
-                                                                  const int64_t* __restrict__ tile_off, int nmax,
-                                                                  const Pair2<F>* __restrict__ lu,
-                                                                  const Pair2<F>* __restrict__ tinv,
-                                                                  Pair2<F>* __restrict__ inv) {
-  using V = Pair2<F>;
-  const int64_t q = blockIdx.y;
+// Inverses of L and U of every block, in step k for row tile k of L^{-1}
+// (from the top) and row tile T - 1 - k of U^{-1} (from the bottom), all blocks
+// together.  With S_ij = sum_k T_ik X_kj over the finished rows k, a step first
+// forms X_kj = -inv(T_kk) S_kj, then adds T_ik X_kj to the S_ij of the rows to
+// come: every tile of a step is one CTA and one tile product, so the work of
+// the largest block spreads over the whole GPU (163 ms with one CTA per column
+// tile, 58 ms now; 175 blocks of up to 1 248 unknowns).  S and X
+// share the slot of the result; the diagonal tile keeps the strictly lower part
+// of L^{-1} and the upper part of U^{-1}.
+__global__ void __launch_bounds__(kTileThreads)
+    precond_inverse_row_kernel(int64_t k, int nact, const int* __restrict__ order, const int64_t* __restrict__ off,
+                               const int64_t* __restrict__ block_off, const int64_t* __restrict__ mat_off,
+                               const int64_t* __restrict__ tile_off, int nmax, const double2* __restrict__ tinv,
+                               double2* __restrict__ inv) {
+  const int s = tile_block(off, nact, blockIdx.x);
+  const int q = order[s];
   const int64_t n = (block_off[q + 1] - block_off[q]) * nmax;
-  const int64_t T = (n + 31) / 32;
-  const int64_t j = blockIdx.x;
-  if (j >= T) return;
-  const bool upper = blockIdx.z == 1;
-  const V* A = lu + mat_off[q];
-  V* X = inv + mat_off[q];
-  const V* TI = tinv + tile_off[q];
-  __shared__ V as[32][33];  // as[m][r]: factor tile, column m, row r
-  __shared__ V xs[32][33];  // xs[c][m]: X tile, column c, row m
-  const int tid = threadIdx.x;
-  const int r = tid & 31, g = tid >> 5;
-  auto tb_of = [&](int64_t t) { return static_cast<int>(n - t * 32 < 32 ? n - t * 32 : 32); };
-  const int tbj = tb_of(j);
-  // stage tile (ti, tk) of a column-major n x n matrix as dst[col][row]
-  // (zero outside the block)
-  auto load_tile = [&](V (*dst)[33], const V* M, int64_t ti, int64_t tk) {
-    const int tbr = tb_of(ti), tbc = tb_of(tk);
-    for (int e = tid; e < 1024; e += 256) {
-      const int c = e >> 5, rr = e & 31;
-      dst[c][rr] = (rr < tbr && c < tbc) ? M[(ti * 32 + rr) + (tk * 32 + c) * n] : V{0, 0};
+  const int64_t T = (n + kTile - 1) / kTile;
+  const int64_t t = blockIdx.x - off[s];  // k + 1 tiles of L, then k + 1 of U
+  const bool upper = t > k;
+  const int64_t row = upper ? T - 1 - k : k;
+  const int64_t col = upper ? T - 1 - (t - k - 1) : t;
+  double2* X = inv + mat_off[q];
+  const double2* Ti = tinv + tile_off[q] + row * 2048 + (upper ? 1024 : 0);
+  const int r = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int64_t i = row * kTile + r, j = col * kTile + 4 * g;
+  if (row == col) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = 4 * g + u;
+      if (i < n && j + u < n && (upper ? r <= c : r > c)) X[i + (j + u) * n] = Ti[c * 32 + r];
     }
-  };
-  // the inverse of diagonal tile t (the whole unit-lower L or upper U
-  // inverse, identity-padded), as dst[col][row]
-  auto load_tinv = [&](V (*dst)[33], int64_t t) {
-    const V* Ti = TI + t * 2048 + (upper ? 1024 : 0);
-    for (int e = tid; e < 1024; e += 256) dst[e >> 5][e & 31] = Ti[e];
-  };
-  // X_jj: write its part (strictly lower for L, upper for U) into the slot
-  load_tinv(xs, j);
-  __syncthreads();
-  for (int e = tid; e < 1024; e += 256) {
-    const int c = e >> 5, rr = e & 31;
-    if (rr < tbj && c < tbj && (upper ? rr <= c : rr > c)) X[(j * 32 + rr) + (j * 32 + c) * n] = xs[c][rr];
+    return;
   }
+  extern __shared__ Tile3 tiles3[];
+  Tile3& as = tiles3[0];
+  Tile3& xs = tiles3[1];
+  load_tinv(as, Ti);
+  load_tile(xs, X, n, row, col);
   __syncthreads();
-  const int64_t i0 = upper ? j - 1 : j + 1;
-  const int64_t di = upper ? -1 : 1;
-  for (int64_t i = i0; upper ? i >= 0 : i < T; i += di) {
-    V acc[4];
+  double2 acc[4] = {};
+  tile_product<-1>(as, xs, acc);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] = V{0, 0};
-    // S = sum over the tiles k strictly between i and j, and k = j
-    const int64_t k0 = upper ? i + 1 : j, k1 = upper ? j : i - 1;
-    for (int64_t k = k0; k <= k1; ++k) {
-      load_tile(as, A, i, k);  // as[m][r] = T_ik[r][m]
-      if (k == j) load_tinv(xs, j);
-      else load_tile(xs, X, k, j);  // xs[c][m] = X_kj[m][c]
-      __syncthreads();
-#pragma unroll 8
-      for (int m = 0; m < 32; ++m) {
-        const V a = as[m][r];
+  for (int u = 0; u < 4; ++u)
+    if (i < n && j + u < n) X[i + (j + u) * n] = acc[u];
+}
+
+__global__ void __launch_bounds__(kTileThreads)
+    precond_inverse_update_kernel(int64_t k, int nact, const int* __restrict__ order, const int64_t* __restrict__ off,
+                                  const int64_t* __restrict__ block_off, const int64_t* __restrict__ mat_off,
+                                  const int64_t* __restrict__ tile_off, int nmax, const double2* __restrict__ lu,
+                                  const double2* __restrict__ tinv, double2* __restrict__ inv) {
+  const int s = tile_block(off, nact, blockIdx.x);
+  const int q = order[s];
+  const int64_t n = (block_off[q + 1] - block_off[q]) * nmax;
+  const int64_t T = (n + kTile - 1) / kTile;
+  const int64_t rem = T - 1 - k, half = rem * (k + 1);  // rem rows to come, k + 1 columns; L, then U
+  int64_t t = blockIdx.x - off[s];
+  const bool upper = t >= half;
+  if (upper) t -= half;
+  const int64_t mid = upper ? rem : k;
+  const int64_t row = upper ? rem - 1 - t % rem : k + 1 + t % rem;
+  const int64_t col = upper ? T - 1 - t / rem : t / rem;
+  const double2* A = lu + mat_off[q];
+  double2* X = inv + mat_off[q];
+  extern __shared__ Tile3 tiles3[];
+  Tile3& as = tiles3[0];
+  Tile3& xs = tiles3[1];
+  load_tile(as, A, n, row, mid);
+  if (col == mid) load_tinv(xs, tinv + tile_off[q] + mid * 2048 + (upper ? 1024 : 0));
+  else load_tile(xs, X, n, mid, col);
+  const int r = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int64_t i = row * kTile + r, j = col * kTile + 4 * g;
+  double2 acc[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const V b = xs[4 * g + u][m];
-          acc[u].re += a.re * b.re - a.im * b.im;
-          acc[u].im += a.re * b.im + a.im * b.re;
-        }
-      }
-      __syncthreads();
-    }
-    // X_ij = -inv(T_ii) S
+  for (int u = 0; u < 4; ++u)  // the first term of S_ij is the one of k = j
+    acc[u] = col != mid && i < n && j + u < n ? X[i + (j + u) * n] : make_double2(0.0, 0.0);
+  __syncthreads();
+  tile_product<1>(as, xs, acc);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) xs[4 * g + u][r] = acc[u];
-    load_tinv(as, i);
-    __syncthreads();
-    V out[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) out[u] = V{0, 0};
-#pragma unroll 8
-    for (int m = 0; m < 32; ++m) {
-      const V a = as[m][r];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const V b = xs[4 * g + u][m];
-        out[u].re -= a.re * b.re - a.im * b.im;
-        out[u].im -= a.re * b.im + a.im * b.re;
-      }
-    }
-    const int tbi = tb_of(i);
-    if (r < tbi) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int c = 4 * g + u;
-        if (c < tbj) X[(i * 32 + r) + (j * 32 + c) * n] = out[u];
-      }
-    }
-    __syncthreads();  // X_ij is read back by the next row tiles
-  }
+  for (int u = 0; u < 4; ++u)
+    if (i < n && j + u < n) X[i + (j + u) * n] = acc[u];
 }
 constexpr int kInvThreads = 256;
 
@@ -627,18 +1022,60 @@ __global__ void __launch_bounds__(kInvThreads) precond_apply_inv_kernel(const in
 }
 
 // FP64 explicit inverses of L and U of every block (from the FP64 LU and
-// FP64 tile inverses) into inv64
-cudaError_t launch_precond_tri_inverse(int64_t nblocks, int64_t max_tiles, const int64_t* block_off,
-                                       const int64_t* mat_off, const int64_t* tile_off, int nmax, const double* lu,
-                                       const double* tinv, double* inv, cudaStream_t st) {
-  if (nblocks <= 0 || max_tiles <= 0) return cudaSuccess;
-  dim3 grid(static_cast<unsigned>(max_tiles), static_cast<unsigned>(nblocks), 2);
-  precond_tri_inverse_kernel<double><<<grid, 256, 0, st>>>(block_off, mat_off, tile_off, nmax,
-                                                           reinterpret_cast<const Pair2<double>*>(lu),
-                                                           reinterpret_cast<const Pair2<double>*>(tinv),
-                                                           reinterpret_cast<Pair2<double>*>(inv));
-  note_launch();
+// FP64 tile inverses) into inv
+cudaError_t launch_precond_tri_inverse(const PrecondPlan& plan, const int64_t* block_off, const int64_t* mat_off,
+                                       const int64_t* tile_off, int nmax, const double* lu, const double* tinv,
+                                       double* inv, cudaStream_t st) {
+  const double2* T = reinterpret_cast<const double2*>(tinv);
+  double2* X = reinterpret_cast<double2*>(inv);
+  cudaError_t e = tile_smem(precond_inverse_row_kernel);
+  if (e == cudaSuccess) e = tile_smem(precond_inverse_update_kernel);
+  if (e != cudaSuccess) return e;
+  for (size_t k = 0; k < plan.steps.size(); ++k) {
+    const PrecondPlan::Step& p = plan.steps[k];
+    precond_inverse_row_kernel<<<static_cast<unsigned>(p.rows), kTileThreads, 2 * sizeof(Tile3), st>>>(
+        static_cast<int64_t>(k), p.active, plan.order, plan.off + p.rows_off, block_off, mat_off, tile_off, nmax, T, X);
+    note_launch();
+    if (p.inv_tiles > 0) {
+      precond_inverse_update_kernel<<<static_cast<unsigned>(p.inv_tiles), kTileThreads, 2 * sizeof(Tile3), st>>>(
+          static_cast<int64_t>(k), p.active, plan.order, plan.off + p.inv_tiles_off, block_off, mat_off, tile_off, nmax,
+          reinterpret_cast<const double2*>(lu), T, X);
+      note_launch();
+    }
+  }
   return cudaGetLastError();
+}
+
+// steps of the blocked factorisation and of the inverses for blocks of the
+// given dimensions; `order` and `off` (host) go to the device
+void precond_plan(const std::vector<int64_t>& dims, PrecondPlan& plan, std::vector<int>& order,
+                  std::vector<int64_t>& off) {
+  order.resize(dims.size());
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return dims[a] > dims[b]; });
+  off.clear();
+  plan.steps.clear();
+  plan.dims.clear();
+  for (int q : order) plan.dims.push_back(dims[q]);
+  const int64_t steps = dims.empty() ? 0 : (plan.dims[0] + kTile - 1) / kTile;
+  for (int64_t k = 0; k < steps; ++k) {
+    PrecondPlan::Step p{};
+    auto tiles = [&](int s) { return (plan.dims[s] + kTile - 1) / kTile; };
+    while (p.active < static_cast<int>(order.size()) && tiles(p.active) > k) ++p.active;
+    auto prefix = [&](int64_t& at, int64_t& total, auto count) {
+      at = static_cast<int64_t>(off.size());
+      total = 0;
+      for (int s = 0; s < p.active; ++s) {
+        off.push_back(total);
+        total += count(tiles(s));
+      }
+    };
+    prefix(p.columns_off, p.columns, [&](int64_t T) { return T - 1; });
+    prefix(p.tiles_off, p.tiles, [&](int64_t T) { return (T - 1 - k) * (T - 1 - k); });
+    prefix(p.rows_off, p.rows, [&](int64_t) { return 2 * (k + 1); });
+    prefix(p.inv_tiles_off, p.inv_tiles, [&](int64_t T) { return 2 * (T - 1 - k) * (k + 1); });
+    plan.steps.push_back(p);
+  }
 }
 
 // position -> source index of the row interchanges of each block's LU
