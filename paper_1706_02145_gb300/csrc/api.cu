@@ -35,7 +35,7 @@ namespace celes {
   int coupling_rpb_##LL(int precision);                                                                    \
   cudaError_t launch_coupling_rtr_##LL(int precision, int64_t N, const void* pos, const void* x,           \
                                        void* partial, double k, int chunks, cudaStream_t st, int maxcl,    \
-                                       int atomic);                                                        \
+                                       int atomic, int nrhs);                                              \
   int coupling_rtr_rpb_##LL(int precision);                                                                \
   int coupling_rtr_slices_##LL(int precision, int chunks, int maxcl, int atomic);                          \
   int coupling_rtr_slots_##LL(int precision);                                                              \
@@ -43,7 +43,8 @@ namespace celes {
   int coupling_terms_export_##LL(int* idx, double* val, int cap);
 #define CELES_DECLARE_ALT(LL)                                                                              \
   cudaError_t launch_coupling_rtr_alt_##LL(int64_t N, const void* pos, const void* x, void* partial,       \
-                                           double k, int chunks, cudaStream_t st, int maxcl, int atomic);  \
+                                           double k, int chunks, cudaStream_t st, int maxcl, int atomic,   \
+                                           int nrhs);                                                      \
   int coupling_rtr_alt_rpb_##LL();                                                                         \
   int coupling_rtr_alt_slices_##LL(int chunks, int maxcl, int atomic);                                     \
   int coupling_rtr_alt_slots_##LL();
@@ -72,13 +73,13 @@ cudaError_t launch_coupling_partial(int L, int precision, int64_t N, const void*
   }
 }
 cudaError_t launch_coupling_rtr(int L, int precision, int64_t N, const void* pos, const void* x, void* partial,
-                                double k, int chunks, cudaStream_t st, int maxcl = 1, int atomic = 0) {
+                                double k, int chunks, cudaStream_t st, int maxcl, int atomic, int nrhs) {
   switch (L) {
-    case 1: return launch_coupling_rtr_1(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic);
-    case 2: return launch_coupling_rtr_2(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic);
-    case 3: return launch_coupling_rtr_3(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic);
-    case 4: return launch_coupling_rtr_4(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic);
-    case 5: return launch_coupling_rtr_5(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic);
+    case 1: return launch_coupling_rtr_1(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
+    case 2: return launch_coupling_rtr_2(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
+    case 3: return launch_coupling_rtr_3(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
+    case 4: return launch_coupling_rtr_4(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
+    case 5: return launch_coupling_rtr_5(precision, N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -88,19 +89,20 @@ int coupling_rtr_slots(int L, int precision);
 // launch shape `variant`: bit 0 the compile-time shape (0: Config, 1:
 // ConfigAlt, FP32 only), bit 1 the cluster reduction of the partial sums
 // (clusters of up to 8 chunks), bit 2 the in-L2 vector reduction of all
-// chunks into one slice (FP32 only)
+// chunks into one slice (FP32 only; the slice is zero before the launch).  One
+// launch for nrhs right-hand sides.
 cudaError_t launch_coupling_rtr_v(int L, int precision, int variant, int64_t N, const void* pos, const void* x,
-                                  void* partial, double k, int chunks, cudaStream_t st) {
+                                  void* partial, double k, int chunks, cudaStream_t st, int nrhs) {
   const int maxcl = (variant & 2) ? 8 : 1;
   const int atomic = (variant & 4) && precision == CELES_FP32 ? 1 : 0;
   if ((variant & 1) == 0 || precision == CELES_FP64)
-    return launch_coupling_rtr(L, precision, N, pos, x, partial, k, chunks, st, maxcl, atomic);
+    return launch_coupling_rtr(L, precision, N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
   switch (L) {
-    case 1: return launch_coupling_rtr_alt_1(N, pos, x, partial, k, chunks, st, maxcl, atomic);
-    case 2: return launch_coupling_rtr_alt_2(N, pos, x, partial, k, chunks, st, maxcl, atomic);
-    case 3: return launch_coupling_rtr_alt_3(N, pos, x, partial, k, chunks, st, maxcl, atomic);
-    case 4: return launch_coupling_rtr_alt_4(N, pos, x, partial, k, chunks, st, maxcl, atomic);
-    case 5: return launch_coupling_rtr_alt_5(N, pos, x, partial, k, chunks, st, maxcl, atomic);
+    case 1: return launch_coupling_rtr_alt_1(N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
+    case 2: return launch_coupling_rtr_alt_2(N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
+    case 3: return launch_coupling_rtr_alt_3(N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
+    case 4: return launch_coupling_rtr_alt_4(N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
+    case 5: return launch_coupling_rtr_alt_5(N, pos, x, partial, k, chunks, st, maxcl, atomic, nrhs);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -247,6 +249,7 @@ struct celes_ctx {
   // the first product picks it (autotuner) or the default is taken
   int tune_variant[2] = {-1, -1};
   int tune_chunks[2] = {0, 0};
+  double tune_waves[2] = {8.0, 8.0};
   double tune_ms[2] = {0.0, 0.0};
   DevBuf pos, radii, nrel, tq, tq32, tdiag;
   int nrhs = 0;
@@ -254,6 +257,10 @@ struct celes_ctx {
   DevBuf ain, rhs, b, x0;
   bool has_b = false, has_x0 = false, x0_learned = false;
   DevBuf partial;
+  // the slice that the in-L2 reduction adds into: zero between products (its
+  // epilogue zeroes what it reads), and used by nothing else
+  DevBuf accum;
+  bool accum_dirty = false;
   // preconditioner
   bool has_precond = false;
   int64_t nblocks = 0;
@@ -348,11 +355,14 @@ int auto_chunks(const celes_ctx* c, int precision) {
 }
 
 // ---- autotuner of the coupling kernel's launch shape ----------------------
-// Candidates: the compile-time shape (Config, and for FP32 ConfigAlt) times
-// the number of source chunks (about 4, 8 or 16 waves of resident CTAs).
-// Each is timed with CUDA events on the context's own positions (the first
-// 20 000 spheres of larger problems) and the fastest kept, once per (device,
-// lmax, precision, log2 N) for the whole process.
+// Candidates: the compile-time shape (Config, and for FP32 ConfigAlt) and the
+// form of the partial sums (slices, or added in L2) times the number of source
+// chunks (about 2 to 32 waves of resident CTAs).  The cluster reduction is not
+// among them: it was slower at every size measured (11.4 against 10.3 ms at
+// N = 10 000, lmax 4).  Each is timed with CUDA events, with its epilogue, on
+// the context's own positions (the first 20 000 spheres of larger problems)
+// and the fastest kept, once per (device, lmax, precision, log2 N) for the
+// whole process.
 struct TuneKey {
   int dev, L, prec, bucket;
   bool operator<(const TuneKey& o) const {
@@ -367,19 +377,15 @@ struct TuneVal {
 std::mutex g_tune_mu;
 std::map<TuneKey, TuneVal> g_tune;
 
-int chunks_for(const celes_ctx* c, int64_t N, int precision, int variant, double waves) {
+// source chunks of one launch over nrhs right-hand sides
+int chunks_for(const celes_ctx* c, int64_t N, int precision, int variant, double waves, int nrhs = 1) {
   const int rpb = coupling_rtr_rpb_v(c->L, precision, variant);
-  const int64_t rb = (N + rpb - 1) / rpb;
+  const int64_t rb = (N + rpb - 1) / rpb * nrhs;
   const int slots = coupling_rtr_slots_v(c->L, precision, variant);
-  const double target = waves * (slots > 0 ? slots : 2 * device_sms());
-  int64_t ch = static_cast<int64_t>(std::ceil(target / static_cast<double>(rb)));
-  ch = std::min<int64_t>(ch, std::max<int64_t>(1, N / 64));
-  ch = std::max<int64_t>(1, std::min<int64_t>(ch, 256));
-  // a multiple of 8 (of 4 below 8): whole clusters for the partial-sum reduction
-  if (ch >= 8) ch = (ch + 7) / 8 * 8;
-  else if (ch >= 4) ch = 4;
-  return static_cast<int>(std::min<int64_t>(ch, 256));
+  return coupling_chunks(N, rb, slots > 0 ? slots : 2 * device_sms(), waves, precision);
 }
+
+bool rtr_atomic(int precision, int variant) { return (variant & 4) && precision == CELES_FP32; }
 
 int autotune(celes_ctx* c, int precision, const void* x, cudaStream_t st) {
   const int pi = precision == CELES_FP64 ? 0 : 1;
@@ -398,47 +404,60 @@ int autotune(celes_ctx* c, int precision, const void* x, cudaStream_t st) {
     }
   }
   if (!have) {
-    const size_t elem = precision == CELES_FP64 ? 16 : 8;
-    const size_t per = static_cast<size_t>(c->N) * c->nmax * elem;
-    // shapes: FP32 built-in / alternative, each with the partial sums in
-    // slices, added in clusters, added in L2, or both
-    std::vector<int> vars =
-        precision == CELES_FP64 ? std::vector<int>{0, 2} : std::vector<int>{0, 1, 2, 3, 4, 5, 6, 7};
-    // waves of CTAs per launch; the L2 reduction (bit 2) makes more chunks
-    // cost no DRAM traffic, so it also tries twice the largest count
-    const double waves[4] = {4.0, 8.0, 16.0, 32.0};
-    auto nwaves = [](int v) { return (v & 4) ? 4 : 3; };
-    int maxch = 1;
-    for (int v : vars)
-      for (int wi = 0; wi < nwaves(v); ++wi) maxch = std::max(maxch, chunks_for(c, Nt, precision, v, waves[wi]));
-    CK(c->partial.ensure(per * std::max(maxch, 1)), "coupling scratch");
+    struct Cand {
+      int variant, chunks, slices;
+      double waves;
+    };
+    std::vector<Cand> cands;
+    int maxsl = 1;
+    for (int v : {0, 1, 4, 5}) {
+      for (double w : {2.0, 4.0, 8.0, 16.0, 32.0}) {
+        if (w > 8.0 && !rtr_atomic(precision, v)) continue;  // slices cost traffic: no more than needed
+        const int ch = chunks_for(c, Nt, precision, v, w);
+        if (!cands.empty() && cands.back().variant == v && cands.back().chunks == ch) continue;
+        const int sl = coupling_rtr_slices_v(c->L, precision, v, ch);
+        cands.push_back(Cand{v, ch, sl, w});
+        maxsl = std::max(maxsl, sl);
+      }
+    }
+    const size_t per = static_cast<size_t>(Nt) * c->nmax * (precision == CELES_FP64 ? 16 : 8);
+    CK(c->partial.ensure(per * (maxsl + 1)), "coupling scratch");
+    char* part = c->partial.as<char>();
+    char* ytmp = part + per * maxsl;
     cudaEvent_t a = nullptr, b = nullptr;
     CK(cudaEventCreate(&a), "event");
     if (cudaEventCreate(&b) != cudaSuccess) {
       cudaEventDestroy(a);
       return cuda_fail(c, cudaErrorMemoryAllocation, "event");
     }
+    auto product = [&](const Cand& q) {
+      cudaError_t e = launch_coupling_rtr_v(c->L, precision, q.variant, Nt, c->pos.p, x, part, c->k, q.chunks, st, 1);
+      if (e != cudaSuccess) return e;
+      const bool zero = rtr_atomic(precision, q.variant);
+      return precision == CELES_FP64
+                 ? launch_coupling_epilogue<double>(Nt, c->L, q.slices, part, x, nullptr, ytmp, 0, st, 1, zero)
+                 : launch_coupling_epilogue<float>(Nt, c->L, q.slices, part, x, nullptr, ytmp, 0, st, 1, zero);
+    };
     best.ms = 1e300;
     cudaError_t e = cudaSuccess;
-    for (int v : vars) {
-      if (e != cudaSuccess) break;
-      for (int wi = 0; wi < nwaves(v); ++wi) {
-        const double w = waves[wi];
-        const int ch = chunks_for(c, Nt, precision, v, w);
-        // one untimed launch (first use of the shape on this device), then one timed
-        e = launch_coupling_rtr_v(c->L, precision, v, Nt, c->pos.p, x, c->partial.p, c->k, ch, st);
-        if (e == cudaSuccess) e = cudaEventRecord(a, st);
-        if (e == cudaSuccess) e = launch_coupling_rtr_v(c->L, precision, v, Nt, c->pos.p, x, c->partial.p, c->k, ch, st);
+    for (const Cand& q : cands) {
+      e = product(q);  // untimed: the first use of the shape on this device
+      float ms = 0.0f;
+      // short products are timed over several
+      for (int reps = 1; e == cudaSuccess; reps = 10) {
+        e = cudaEventRecord(a, st);
+        for (int r = 0; r < reps && e == cudaSuccess; ++r) e = product(q);
         if (e == cudaSuccess) e = cudaEventRecord(b, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(b);
-        float ms = 0.0f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
-        if (e != cudaSuccess) break;
-        if (ms < best.ms) {
-          best.ms = ms;
-          best.variant = v;
-          best.waves = w;
-        }
+        ms /= static_cast<float>(reps);
+        if (reps > 1 || ms > 0.3f) break;
+      }
+      if (e != cudaSuccess) break;
+      if (ms < best.ms) {
+        best.ms = ms;
+        best.variant = q.variant;
+        best.waves = q.waves;
       }
     }
     cudaEventDestroy(a);
@@ -448,6 +467,7 @@ int autotune(celes_ctx* c, int precision, const void* x, cudaStream_t st) {
     g_tune[key] = best;
   }
   c->tune_variant[pi] = best.variant;
+  c->tune_waves[pi] = best.waves;
   c->tune_chunks[pi] = chunks_for(c, c->N, precision, best.variant, best.waves);
   c->tune_ms[pi] = best.ms;
   return CELES_OK;
@@ -486,12 +506,31 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
     }
   }
   const int variant = c->tune_variant[pi];
-  const int chunks = c->tune_chunks[pi];
-  const int slices = use_rtr(c, precision) ? coupling_rtr_slices_v(c->L, precision, variant, chunks) : chunks;
+  const bool rtr = use_rtr(c, precision);
+  const bool atomic = rtr && rtr_atomic(precision, variant);
   const size_t elem = precision == CELES_FP64 ? 16 : 8;
   const size_t per = static_cast<size_t>(c->N) * c->nmax * elem;
-  CK(c->partial.ensure(per * chunks), "coupling scratch");
-  for (int r = 0; r < nrhs; ++r) {
+  for (int r = 0; r < nrhs;) {
+    // right-hand sides of one launch (with fewer source chunks each, so that
+    // the launch keeps its waves: N = 777, lmax 5, 8 right-hand sides 1.11 ->
+    // 0.98 ms), as many as keep the partial sums within 1 GB
+    int group = rtr ? std::min(nrhs - r, 256) : 1;
+    int chunks = 0, slices = 0;
+    for (;; group = (group + 1) / 2) {
+      chunks = group == 1 || c->chunks_opt > 0 ? c->tune_chunks[pi]
+                                               : chunks_for(c, c->N, precision, variant, std::max(c->tune_waves[pi], 6.0),
+                                                            group);
+      slices = rtr ? coupling_rtr_slices_v(c->L, precision, variant, chunks) : chunks;
+      if (group == 1 || per * slices * group <= (size_t(1) << 30)) break;
+    }
+    DevBuf& buf = atomic ? c->accum : c->partial;
+    const size_t need = per * slices * group;
+    const bool fresh = need > buf.bytes;
+    CK(buf.ensure(need), "coupling scratch");
+    if (atomic) {
+      if (fresh || c->accum_dirty) CK(cudaMemsetAsync(buf.p, 0, buf.bytes, st), "coupling scratch");
+      c->accum_dirty = true;  // until the epilogue that zeroes it is launched
+    }
     const char* xr = static_cast<const char*>(x) + per * r;
     char* yr = static_cast<char*>(y) + per * r;
     celes_ctx::Rec rec{};
@@ -499,12 +538,11 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
       int s = prof_begin(c, st, rec, precision == CELES_FP64 ? 1 : 0);
       if (s) return s;
     }
-    if (use_rtr(c, precision))
-      CK(launch_coupling_rtr_v(c->L, precision, variant, c->N, c->pos.p, xr, c->partial.p, c->k, chunks, st),
+    if (rtr)
+      CK(launch_coupling_rtr_v(c->L, precision, variant, c->N, c->pos.p, xr, buf.p, c->k, chunks, st, group),
          "coupling kernel");
     else
-      CK(launch_coupling_partial(c->L, precision, c->N, c->pos.p, xr, c->partial.p, c->k, chunks, st),
-         "coupling kernel");
+      CK(launch_coupling_partial(c->L, precision, c->N, c->pos.p, xr, buf.p, c->k, chunks, st), "coupling kernel");
     if (c->profiling) {
       CK(cudaEventRecord(rec.b, st), "event");
       c->recs.push_back(rec);
@@ -512,13 +550,16 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
       if (s) return s;
     }
     if (precision == CELES_FP64)
-      CK(launch_coupling_epilogue<double>(c->N, c->L, slices, c->partial.p, xr, c->tq.p, yr, mode, st), "epilogue");
+      CK(launch_coupling_epilogue<double>(c->N, c->L, slices, buf.p, xr, c->tq.p, yr, mode, st, group), "epilogue");
     else
-      CK(launch_coupling_epilogue<float>(c->N, c->L, slices, c->partial.p, xr, c->tq32.p, yr, mode, st), "epilogue");
+      CK(launch_coupling_epilogue<float>(c->N, c->L, slices, buf.p, xr, c->tq32.p, yr, mode, st, group, atomic),
+         "epilogue");
+    if (atomic) c->accum_dirty = false;
     if (c->profiling) {
       CK(cudaEventRecord(rec.b, st), "event");
       c->recs.push_back(rec);
     }
+    r += group;
   }
   return CELES_OK;
 }
@@ -672,6 +713,7 @@ extern "C" void celes_destroy(celes_ctx* c) {
     c->b.release();
     c->x0.release();
     c->partial.release();
+    c->accum.release();
     c->block_off.release();
     c->mat_off.release();
     c->perm.release();

@@ -844,8 +844,9 @@ extern "C" int celes_batch_create(celes_batch** out, celes_ctx* const* ctxs, int
     }
   }
   // source chunk length per lmax group: about eight waves of tiles over the
-  // group's work (FP32 launch shape), between 32 and 512 sources, so that
-  // groups of a few large-lmax ensembles do not run in less than one wave
+  // group's work, between 32 (FP64: 8, a pair takes forty times as long) and
+  // 512 sources, so that groups of a few large-lmax ensembles do not run in
+  // less than one wave
   for (int L = 1; L <= 5; ++L) {
     double work = 0.0;  // ordered pairs x RHS of the group
     for (const System& Sy : bt->sys)
@@ -853,21 +854,24 @@ extern "C" int celes_batch_create(celes_batch** out, celes_ctx* const* ctxs, int
     if (work == 0.0) continue;
     const int rpb = rtr_rpb(L, CELES_FP32);
     const double slots = static_cast<double>(celes::coupling_rtr_slots(L, CELES_FP32));
-    const double want = work / (8.0 * std::max(1.0, slots) * rpb);
-    int chunk = static_cast<int>(std::ceil(want / 32.0)) * 32;
-    chunk = std::max(32, std::min(512, chunk));
+    auto length = [&](double per_slot, int least) {
+      const int len = static_cast<int>(std::ceil(work / (8.0 * std::max(1.0, per_slot)) / least)) * least;
+      return std::max(least, std::min(512, len));
+    };
+    const int chunk = length(slots * rpb, 32);
+    const int chunk64 = length(static_cast<double>(celes::coupling_rtr_slots(L, CELES_FP64)) * rtr_rpb(L, CELES_FP64), 8);
     // FP32: chunks cost no partial-sum traffic (one slice per system), so
     // each system gets about two waves of tiles of its own, which keeps the
     // GPU busy once only a few systems remain active
     const int nrb_den = rpb > 0 ? rpb : 1;
     for (System& Sy : bt->sys)
       if (Sy.L == L) {
-        Sy.chunk = std::min(Sy.N, chunk);
+        Sy.chunk = std::min(Sy.N, chunk64);
         Sy.chunks = (Sy.N + Sy.chunk - 1) / Sy.chunk;
         const int nrb = (Sy.N + nrb_den - 1) / nrb_den;
         const double ch32 = std::ceil(2.0 * std::max(1.0, slots) / nrb);
         int c32 = static_cast<int>(std::ceil(Sy.N / ch32 / 32.0)) * 32;
-        c32 = std::max(64, std::min(chunk, c32));
+        c32 = std::max(32, std::min(chunk, c32));
         Sy.chunk32 = std::min(Sy.N, c32);
         Sy.chunks32 = (Sy.N + Sy.chunk32 - 1) / Sy.chunk32;
       }
@@ -879,7 +883,9 @@ extern "C" int celes_batch_create(celes_batch** out, celes_ctx* const* ctxs, int
     p64 += (long long)Sy.chunks * Sy.n * 16;
   }
   bt->ntot = off;
-  for (int L = 1; L <= 5; ++L) {
+  // the longest tiles first: the groups' launches share the GPU, and the short
+  // tiles of the low degrees then fill the end
+  for (int L = 5; L >= 1; --L) {
     Group g;
     g.L = L;
     for (size_t s = 0; s < bt->sys.size(); ++s) {

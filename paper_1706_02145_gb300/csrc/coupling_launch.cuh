@@ -124,9 +124,10 @@ long long rtr_flops_per_pair_t() {
 // the alternative FP32 shape (ConfigAlt), in a translation unit of its own
 #define CELES_INSTANTIATE_RTR_ALT(LL)                                                                      \
   cudaError_t launch_coupling_rtr_alt_##LL(int64_t N, const void* pos, const void* x, void* partial,       \
-                                           double k, int chunks, cudaStream_t st, int maxcl, int atomic) { \
+                                           double k, int chunks, cudaStream_t st, int maxcl, int atomic,   \
+                                           int nrhs) {                                                     \
     return rtr::launch_partial<LL, float, rtr::ConfigAlt<LL, float>>(N, pos, x, partial, k, chunks, st,    \
-                                                                     maxcl, atomic != 0);                  \
+                                                                     maxcl, atomic != 0, nrhs);            \
   }                                                                                                         \
   int coupling_rtr_alt_rpb_##LL() { return rtr::ConfigAlt<LL, float>::BLOCK; }                             \
   int coupling_rtr_alt_slices_##LL(int chunks, int maxcl, int atomic) {                                    \
@@ -147,10 +148,11 @@ long long rtr_flops_per_pair_t() {
   }                                                                                                        \
   cudaError_t launch_coupling_rtr_##LL(int precision, int64_t N, const void* pos, const void* x,           \
                                        void* partial, double k, int chunks, cudaStream_t st, int maxcl,    \
-                                       int atomic) {                                                       \
+                                       int atomic, int nrhs) {                                             \
     return precision == 0                                                                                  \
-               ? rtr::launch_partial<LL, double>(N, pos, x, partial, k, chunks, st, maxcl, false)          \
-               : rtr::launch_partial<LL, float>(N, pos, x, partial, k, chunks, st, maxcl, atomic != 0);    \
+               ? rtr::launch_partial<LL, double>(N, pos, x, partial, k, chunks, st, maxcl, false, nrhs)    \
+               : rtr::launch_partial<LL, float>(N, pos, x, partial, k, chunks, st, maxcl, atomic != 0,     \
+                                                nrhs);                                                     \
   }                                                                                                        \
   int coupling_rtr_rpb_##LL(int precision) {                                                               \
     return precision == 0 ? rtr::Config<LL, double>::BLOCK : rtr::Config<LL, float>::BLOCK;               \

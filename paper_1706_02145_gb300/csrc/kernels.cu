@@ -8,9 +8,12 @@
 //  * far-field amplitude g_j (App. D)
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdint>
 
+#include "../../include/celes.h"
 #include "cmath.cuh"
 #include "coupling_kernel.cuh"
 #include "kernels.h"
@@ -31,20 +34,27 @@ static __device__ __forceinline__ int row_l_rt(int r) {
 // ---------------------------------------------------------------------------
 // coupling epilogue
 // ---------------------------------------------------------------------------
-template <typename R>
-__global__ void coupling_epilogue_kernel(int64_t N, int L, int chunks, const Pair2<R>* __restrict__ partial,
+// grid (blocks, right-hand sides).  ZERO: one slice, zeroed again behind the
+// read (each element by the thread that read it) for the next launch that adds
+// into it
+template <typename R, bool ZERO>
+__global__ void coupling_epilogue_kernel(int64_t N, int L, int chunks, Pair2<R>* __restrict__ partial,
                                          const Pair2<R>* __restrict__ x, const Pair2<R>* __restrict__ tq,
                                          Pair2<R>* __restrict__ y, int mode) {
   const int NH = L * (L + 2);
   const int64_t total = N * NH;
+  partial += (int64_t)blockIdx.y * chunks * total * 2;
+  x += (int64_t)blockIdx.y * total * 2;
+  y += (int64_t)blockIdx.y * total * 2;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = t / NH;
     const int r = static_cast<int>(t - i * NH);
     R pr = 0, pi = 0, mr = 0, mi = 0;
     for (int c = 0; c < chunks; ++c) {
-      const Pair2<R>* pc = partial + ((int64_t)c * N + i) * (2 * NH);
+      Pair2<R>* pc = partial + ((int64_t)c * N + i) * (2 * NH);
       const Pair2<R> a = pc[r];
       const Pair2<R> b = pc[NH + r];
+      if (ZERO) pc[r] = pc[NH + r] = Pair2<R>{0, 0};
       pr += a.re;
       pi += a.im;
       mr += b.re;
@@ -67,24 +77,48 @@ __global__ void coupling_epilogue_kernel(int64_t N, int L, int chunks, const Pai
   }
 }
 
+// About `waves` waves of CTAs, in chunks of at least 16 sources (FP32) or 4
+// (FP64, whose pair takes forty times as long): a chunk pays for staging, its
+// flush and its share of the epilogue, one or two pairs' time, and fewer,
+// longer chunks leave the last wave of a mid-sized problem mostly empty (FP64
+// N = 1000, lmax 3: 3.0 ms with at least 64 sources, 2.5 ms so; FP32 N = 2000,
+// lmax 3: 224 and 196 us).  Where even that leaves resident slots empty, chunks
+// down to 2 or 1 sources fill them: the sources of a chunk are walked one after
+// another (N = 50, lmax 3, FP32: 18.5 -> 8.0 us; a refined solve at N = 120:
+// 30.4 -> 5.4 ms, most of it the FP64 products).
+int coupling_chunks(int64_t N, int64_t rb, int slots, double waves, int precision) {
+  const bool fp64 = precision == CELES_FP64;
+  int64_t ch = static_cast<int64_t>(std::ceil(waves * slots / static_cast<double>(rb)));
+  ch = std::min<int64_t>(ch, std::max<int64_t>(1, N / (fp64 ? 4 : 16)));
+  const int64_t fill = (slots + rb - 1) / rb;
+  ch = std::max(ch, std::min(fill, std::max<int64_t>(1, N / (fp64 ? 1 : 2))));
+  // a multiple of 8 (of 4 below 8): whole clusters for the cluster reduction
+  if (ch >= 8) ch = (ch + 7) / 8 * 8;
+  else if (ch >= 4) ch = 4;
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(ch, 512)));
+}
+
 template <typename R>
-cudaError_t launch_coupling_epilogue(int64_t N, int L, int chunks, const void* partial, const void* x, const void* tq,
-                                     void* y, int mode, cudaStream_t st) {
+cudaError_t launch_coupling_epilogue(int64_t N, int L, int chunks, void* partial, const void* x, const void* tq,
+                                     void* y, int mode, cudaStream_t st, int nrhs, bool zero) {
   const int64_t total = N * L * (L + 2);
   const int threads = 256;
   const int64_t blocks = (total + threads - 1) / threads;
   const int64_t cap = 32LL * device_sms();
-  const int grid = static_cast<int>(blocks < cap ? blocks : cap);
-  coupling_epilogue_kernel<R><<<grid > 0 ? grid : 1, threads, 0, st>>>(
-      N, L, chunks, static_cast<const Pair2<R>*>(partial), static_cast<const Pair2<R>*>(x),
-      static_cast<const Pair2<R>*>(tq), static_cast<Pair2<R>*>(y), mode);
+  const dim3 grid(static_cast<unsigned>(blocks < cap ? (blocks > 0 ? blocks : 1) : cap), static_cast<unsigned>(nrhs));
+  auto* p = static_cast<Pair2<R>*>(partial);
+  auto* xv = static_cast<const Pair2<R>*>(x);
+  auto* t = static_cast<const Pair2<R>*>(tq);
+  auto* yv = static_cast<Pair2<R>*>(y);
+  if (zero && chunks == 1) coupling_epilogue_kernel<R, true><<<grid, threads, 0, st>>>(N, L, 1, p, xv, t, yv, mode);
+  else coupling_epilogue_kernel<R, false><<<grid, threads, 0, st>>>(N, L, chunks, p, xv, t, yv, mode);
   note_launch();
   return cudaGetLastError();
 }
-template cudaError_t launch_coupling_epilogue<float>(int64_t, int, int, const void*, const void*, const void*, void*,
-                                                     int, cudaStream_t);
-template cudaError_t launch_coupling_epilogue<double>(int64_t, int, int, const void*, const void*, const void*, void*,
-                                                      int, cudaStream_t);
+template cudaError_t launch_coupling_epilogue<float>(int64_t, int, int, void*, const void*, const void*, void*, int,
+                                                     cudaStream_t, int, bool);
+template cudaError_t launch_coupling_epilogue<double>(int64_t, int, int, void*, const void*, const void*, void*, int,
+                                                      cudaStream_t, int, bool);
 
 // ---------------------------------------------------------------------------
 // Mie T-matrix (App. B): one thread per sphere, all l

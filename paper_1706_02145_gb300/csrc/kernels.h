@@ -65,8 +65,8 @@ int coupling_term_count(int L);
 int coupling_terms_export(int L, int* idx, double* val, int cap);
 
 template <typename R>
-cudaError_t launch_coupling_epilogue(int64_t N, int L, int chunks, const void* partial, const void* x, const void* tq,
-                                     void* y, int mode, cudaStream_t st);
+cudaError_t launch_coupling_epilogue(int64_t N, int L, int chunks, void* partial, const void* x, const void* tq,
+                                     void* y, int mode, cudaStream_t st, int nrhs = 1, bool zero = false);
 
 cudaError_t launch_mie(int64_t N, int L, double k, const double* radii, const double* n_rel, double* tq,
                        cudaStream_t st);
@@ -81,6 +81,8 @@ cudaError_t launch_gaussian_beam(int64_t N, int L, double k, const void* pos, do
 inline bool current_device(int* d) { return cudaGetDevice(d) == cudaSuccess; }
 
 int vec_dot_blocks(int64_t n);
+// source chunks of a coupling launch of rb receiver blocks on `slots` resident CTAs
+int coupling_chunks(int64_t N, int64_t rb, int slots, double waves, int precision);
 // streaming multiprocessors of the current device (queried once per device)
 int device_sms();
 template <typename R>

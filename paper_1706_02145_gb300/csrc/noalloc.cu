@@ -23,7 +23,7 @@ namespace celes {
 #define CELES_DECLARE_RTR(LL)                                                                               \
   cudaError_t launch_coupling_rtr_##LL(int precision, int64_t N, const void* pos, const void* x,           \
                                        void* partial, double k, int chunks, cudaStream_t st, int maxcl,    \
-                                       int atomic);                                                        \
+                                       int atomic, int nrhs);                                              \
   int coupling_rtr_rpb_##LL(int precision);                                                                \
   int coupling_rtr_slices_##LL(int precision, int chunks, int maxcl, int atomic);                          \
   int coupling_rtr_slots_##LL(int precision);
@@ -69,11 +69,11 @@ cudaError_t launch_rtr(int L, int precision, int64_t N, const void* pos, const v
                        int chunks, cudaStream_t st) {
   using namespace celes;
   switch (L) {
-    case 1: return launch_coupling_rtr_1(precision, N, pos, x, partial, k, chunks, st, 1, 0);
-    case 2: return launch_coupling_rtr_2(precision, N, pos, x, partial, k, chunks, st, 1, 0);
-    case 3: return launch_coupling_rtr_3(precision, N, pos, x, partial, k, chunks, st, 1, 0);
-    case 4: return launch_coupling_rtr_4(precision, N, pos, x, partial, k, chunks, st, 1, 0);
-    case 5: return launch_coupling_rtr_5(precision, N, pos, x, partial, k, chunks, st, 1, 0);
+    case 1: return launch_coupling_rtr_1(precision, N, pos, x, partial, k, chunks, st, 1, 0, 1);
+    case 2: return launch_coupling_rtr_2(precision, N, pos, x, partial, k, chunks, st, 1, 0, 1);
+    case 3: return launch_coupling_rtr_3(precision, N, pos, x, partial, k, chunks, st, 1, 0, 1);
+    case 4: return launch_coupling_rtr_4(precision, N, pos, x, partial, k, chunks, st, 1, 0, 1);
+    case 5: return launch_coupling_rtr_5(precision, N, pos, x, partial, k, chunks, st, 1, 0, 1);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -134,9 +134,7 @@ extern "C" int celes_coupling_matvec_noalloc(int64_t N, int lmax, double k, cons
   const int rpb = rtr_rpb(lmax, precision);
   const int64_t rb = (N + rpb - 1) / rpb;
   const int slots = rtr_slots(lmax, precision);
-  int64_t chunks = (8LL * (slots > 0 ? slots : 304) + rb - 1) / rb;  // about eight waves
-  chunks = std::min<int64_t>(chunks, std::max<int64_t>(1, N / 64));
-  chunks = std::min<int64_t>(chunks, 256);
+  int64_t chunks = celes::coupling_chunks(N, rb, slots > 0 ? slots : 304, 8.0, precision);  // about eight waves
   chunks = std::min<int64_t>(chunks, static_cast<int64_t>(max_chunks));
   chunks = std::max<int64_t>(chunks, 1);
   void* scratch = nullptr;

@@ -25,7 +25,7 @@
 // GB300, master product, before -> after: FP32 N = 10 000 lmax 4 9.87 -> 7.71
 // ms (error against 64 bits 6.0e-7 -> 3.2e-7), N = 777 lmax 5 with 8 right-hand
 // sides 2.27 -> 1.11 ms, N = 100 000 lmax 3 492 -> 395 ms; FP64 N = 2001 lmax 4
-// 22.9 -> 17.5 ms.
+// 22.9 -> 17.5 ms (16.9 ms with the shape below).
 #pragma once
 
 #include <cooperative_groups.h>
@@ -366,6 +366,24 @@ __device__ __forceinline__ void ax_entry(const Hankel<L, R>& h, R& ar, R& ai, R&
   (ax_b<L, MU, LO, LI, KB>(h, br, bi), ...);
 }
 
+// The axial products of mu > 0 on the packed FMA as well, both sums of one
+// factor together: at lmax 4 the scalar half of the FP32 lanes is the fuller
+// one without it (N = 10 000: 7.84 -> 7.68 ms; 1.77 -> 1.83 ms at lmax 2, 395 ->
+// 407 ms at N = 100 000 and lmax 3, 16.4 -> 16.5 ms at lmax 5)
+template <int L, typename R>
+constexpr bool kPackedAxial = sizeof(R) == 4 && L == 4;
+
+// y += w x for two complex values of one factor: y, x = (re, im, re, im)
+__device__ __forceinline__ void cmac_pair(float* y, float wr, float wi, const float* x) {
+  const C2<float> xr{x[0], x[2]}, xi{x[1], x[3]};
+  const C2<float> yr = fma2(wr, xr, fma2(-wi, xi, C2<float>{y[0], y[2]}));
+  const C2<float> yi = fma2(wr, xi, fma2(wi, xr, C2<float>{y[1], y[3]}));
+  y[0] = yr.x;
+  y[1] = yi.x;
+  y[2] = yr.y;
+  y[3] = yi.y;
+}
+
 // y += S w x for one (row, column) entry, S = +-1 at compile time
 template <int S, typename R>
 __device__ __forceinline__ void cmac_s(R* y, R wr, R wi, const R* x) {
@@ -402,6 +420,16 @@ __device__ __forceinline__ void ax_sym_pair(const Hankel<L, R>& h, const R (&u)[
     } else {
       // W+ = A + i B', W- = A - i B'
       const R wpr = ar - bi, wpi = ai + br, wmr = ar + bi, wmi = ai - br;
+      if constexpr (kPackedAxial<L, R>) {
+        cmac_pair(y[LO - 1], wpr, wpi, u[LI - 1]);
+        cmac_pair(y[LO - 1] + 4, wmr, wmi, u[LI - 1] + 4);
+        if constexpr (LO != LI) {
+          constexpr R SS = static_cast<R>(S);
+          cmac_pair(y[LI - 1], SS * wpr, SS * wpi, u[LO - 1]);
+          cmac_pair(y[LI - 1] + 4, SS * wmr, SS * wmi, u[LO - 1] + 4);
+        }
+        return;
+      }
       cmac_s<1>(y[LO - 1], wpr, wpi, u[LI - 1]);
       cmac_s<1>(y[LO - 1] + 2, wpr, wpi, u[LI - 1] + 2);
       cmac_s<1>(y[LO - 1] + 4, wmr, wmi, u[LI - 1] + 4);
@@ -519,17 +547,11 @@ __device__ __forceinline__ void rot_bwd(const Angles<L, R>& g, XV& xp, Acc& acc,
   (rot_bwd_block<L, LI + 1>(g, xp, acc), ...);
 }
 
-// storage views: registers (compile-time index) or a per-thread column of a
-// shared-memory array [4 NH][BLOCK]
+// x' and y' of one pair: compile-time indices, in registers as far as they go
 template <typename R>
 struct AccReg {
   R* a;
   __device__ __forceinline__ R& operator()(int q) const { return a[q]; }
-};
-template <typename R, int BLOCK>
-struct AccSmem {
-  R* a;
-  __device__ __forceinline__ R& operator()(int q) const { return a[q * BLOCK]; }
 };
 
 // receiver sums, one 4-vector (tau 1 re, im, tau 2 re, im) per row (l, m):
@@ -631,23 +653,36 @@ __device__ __forceinline__ void pair(const GeomS<R>& q, const Quad4<R>* __restri
   }
 }
 
-// Launch shape per (lmax, precision)
+// Launch shape per (lmax, precision).  FP64: the FP64 pipe takes a warp
+// instruction every 76 clocks, so every scheduler needs a warp and nothing else
+// matters: x' stays in thread-local memory (spilled registers) where a second
+// shared-memory array would leave schedulers without one (N = 2000, lmax 5: 56.8
+// ms with x' in shared memory and two warps per SM, 33.8 ms with four; lmax 4
+// 17.6 -> 16.8 ms with four-warp CTAs, lmax 3 9.09 -> 8.92 ms).  FP32: 64
+// receivers a CTA, which idle fewer lanes on a small or ragged number of
+// spheres than 128 and cost as little at large ones (lmax 4, N = 10 000: 7.88
+// against 7.84 ms; a batch of 12 ensembles x 4 right-hand sides of 300-1163
+// spheres 3.79 -> 3.57 ms).
 template <int L, typename R>
 struct Config {
   static constexpr bool FP64 = sizeof(R) == 8;
-  static constexpr int BLOCK = FP64 ? (L >= 5 ? 32 : 64) : 128;
-  static constexpr int TJ = FP64 ? 16 : 32;
+  static constexpr int BLOCK = FP64 && L == 4 ? 128 : 64;
+  static constexpr int TJ = FP64 ? (L >= 5 ? 8 : 16) : 32;
   static constexpr bool ACC_SMEM = FP64 ? (L >= 2) : (L >= 3);
-  static constexpr bool XY_SMEM = FP64 && L >= 3;
-  static constexpr int MINB = (!FP64 && L == 3) ? 3 : 1;  // minimum resident CTAs per SM for the allocator
+  static constexpr int MINB = (!FP64 && L == 3) ? 6 : 1;  // minimum resident CTAs per SM for the allocator
+  static constexpr bool SYNC_PAIR = false;                // barrier per source
 };
 
-// The alternative FP32 launch shape of each lmax, the second candidate of
-// the autotuner (celes_ctx tuning)
+// The alternative FP32 launch shape of each lmax, the second candidate of the
+// autotuner (celes_ctx tuning): 128 receivers per CTA; at lmax 5 one CTA of 256
+// whose warps take every source together, since the code of a pair (about
+// 3 600 instructions) is larger than the instruction cache (15.7 against 16.4
+// ms).
 template <int L, typename R>
 struct ConfigAlt : Config<L, R> {
-  static constexpr int BLOCK = L <= 2 ? 64 : 128;
-  static constexpr int MINB = L == 4 ? 3 : 1;
+  static constexpr int BLOCK = L == 5 ? 256 : 128;
+  static constexpr int MINB = L == 3 ? 3 : 1;
+  static constexpr bool SYNC_PAIR = L == 5;
 };
 
 template <int L, typename R, typename C = Config<L, R>>
@@ -657,8 +692,7 @@ struct Layout {
   static constexpr size_t off_pos = 0;
   static constexpr size_t off_x = off_pos + sizeof(Pos4) * C::TJ;
   static constexpr size_t off_acc = off_x + sizeof(Quad4<R>) * NH * C::TJ;
-  static constexpr size_t off_xy = off_acc + (C::ACC_SMEM ? col : 0);
-  static constexpr size_t bytes = off_xy + (C::XY_SMEM ? col : 0);
+  static constexpr size_t bytes = off_acc + (C::ACC_SMEM ? col : 0);
 };
 
 // whether `atomic` asks for the in-L2 vector reduction of the partial sums
@@ -676,7 +710,7 @@ constexpr bool partial_atomic(bool atomic) {
 // through distributed shared memory and write one partial per cluster, so
 // the partial-sum traffic shrinks by the cluster size.
 // ATOM (FP32): the sums are added into out with vector reductions in L2
-// (out zeroed before the launch), so all source chunks share one slice and
+// (out zero before the launch), so all source chunks share one slice and
 // only the final sums reach DRAM; the order of the additions, and so the
 // last bits of the result, vary from launch to launch.
 template <int L, typename R, typename C, bool CRED = false, bool ATOM = false>
@@ -690,7 +724,6 @@ __device__ __forceinline__ void rtr_tile(int N, const Pos4* __restrict__ pos, co
   Pos4* spos = reinterpret_cast<Pos4*>(smem_raw + LY::off_pos);
   Quad4<R>* sx = reinterpret_cast<Quad4<R>*>(smem_raw + LY::off_x);
   R* sacc = reinterpret_cast<R*>(smem_raw + LY::off_acc);
-  R* sxy = reinterpret_cast<R*>(smem_raw + LY::off_xy);
 
   const int tid = threadIdx.x;
   const int i = rb * BLOCK + tid;
@@ -725,6 +758,7 @@ __device__ __forceinline__ void rtr_tile(int N, const Pos4* __restrict__ pos, co
     }
     __syncthreads();
     for (int jj = 0; jj < nj; ++jj) {
+      if constexpr (C::SYNC_PAIR) __syncthreads();
       if (!active || jt + jj == i) continue;  // no self coupling
       GeomS<R> gs;
       if constexpr (FF) {
@@ -734,22 +768,14 @@ __device__ __forceinline__ void rtr_tile(int N, const Pos4* __restrict__ pos, co
         gs = geometry(ri.x - rj.x, ri.y - rj.y, ri.z - rj.z, k);
       }
       const Quad4<R>* xs = sx + jj * NH;
-      auto run = [&](auto& xp) {
-        if constexpr (C::ACC_SMEM) {
-          RowAccSmem<R, BLOCK> acc{sacc4 + tid};
-          pair<L, R>(gs, xs, xp, acc);
-        } else {
-          RowAccReg<R> acc{areg};
-          pair<L, R>(gs, xs, xp, acc);
-        }
-      };
-      if constexpr (C::XY_SMEM) {
-        AccSmem<R, BLOCK> xp{sxy + tid};
-        run(xp);
+      R xa[4 * NH];
+      AccReg<R> xp{xa};
+      if constexpr (C::ACC_SMEM) {
+        RowAccSmem<R, BLOCK> acc{sacc4 + tid};
+        pair<L, R>(gs, xs, xp, acc);
       } else {
-        R xa[4 * NH];
-        AccReg<R> xp{xa};
-        run(xp);
+        RowAccReg<R> acc{areg};
+        pair<L, R>(gs, xs, xp, acc);
       }
     }
   }
@@ -854,11 +880,12 @@ __device__ __forceinline__ void rtr_tile(int N, const Pos4* __restrict__ pos, co
   }
 }
 
-// grid (receiver blocks of BLOCK, source chunks); writes partial sums in the
-// +- basis, [chunks][N][2][NH] complex (same layout as the direct kernel)
+// grid (receiver blocks of BLOCK, source chunks, right-hand sides); writes
+// partial sums in the +- basis, [rhs][slices][N][2][NH] complex (per right-hand
+// side the layout of the direct kernel)
 // CRED: launched with clusters of `ncl` CTAs along y; cluster c writes
 // partial slice c (the grid's y extent is a multiple of ncl)
-// ATOM: every tile adds into slice 0 (zeroed before the launch)
+// ATOM: every tile adds into slice 0 of its right-hand side (zero before the launch)
 template <int L, typename R, typename C = Config<L, R>, bool CRED = false, bool ATOM = false>
 __global__ void __launch_bounds__(C::BLOCK, C::MINB)
     rtr_partial_kernel(int N, const Pos4* __restrict__ pos, const Pair2<R>* __restrict__ x,
@@ -867,9 +894,11 @@ __global__ void __launch_bounds__(C::BLOCK, C::MINB)
   constexpr int NH = L * (L + 2);
   const int j0 = blockIdx.y * chunk;
   const int j1 = min(N, j0 + chunk);
-  const int slice = ATOM ? 0 : (CRED ? static_cast<int>(blockIdx.y) / ncl : static_cast<int>(blockIdx.y));
-  rtr_tile<L, R, C, CRED, ATOM>(N, pos, x, partial + (size_t)slice * N * (2 * NH), k, blockIdx.x, j0, j1,
-                                smem_raw);
+  if (ATOM && !CRED && j0 >= j1) return;  // a chunk past the last source adds nothing
+  const size_t slices = ATOM ? 1 : (CRED ? gridDim.y / ncl : gridDim.y);
+  const size_t slice = blockIdx.z * slices + (ATOM ? 0 : (CRED ? blockIdx.y / ncl : blockIdx.y));
+  rtr_tile<L, R, C, CRED, ATOM>(N, pos, x + (size_t)blockIdx.z * N * (2 * NH), partial + slice * N * (2 * NH), k,
+                                blockIdx.x, j0, j1, smem_raw);
 }
 
 // ---- batched form: one persistent launch over the tiles of many systems ----
@@ -991,15 +1020,12 @@ int partial_slices(int chunks, int maxcl, bool atomic) {
 
 template <int L, typename R, typename C, bool CRED, bool ATOM>
 cudaError_t launch_partial_form(int64_t N, const void* pos, const void* x, void* partial, double k, int chunks,
-                                int ncl, cudaStream_t st) {
+                                int ncl, cudaStream_t st, int nrhs) {
   using LY = Layout<L, R, C>;
   if (partial_form_occupancy<L, R, C, CRED, ATOM>() < 1) return cudaErrorInvalidConfiguration;
   const int64_t chunk = (N + chunks - 1) / chunks;
-  dim3 grid(static_cast<unsigned>((N + C::BLOCK - 1) / C::BLOCK), static_cast<unsigned>(chunks));
-  if constexpr (ATOM) {
-    const cudaError_t e = cudaMemsetAsync(partial, 0, sizeof(Pair2<R>) * 2 * (L * (L + 2)) * N, st);
-    if (e != cudaSuccess) return e;
-  }
+  dim3 grid(static_cast<unsigned>((N + C::BLOCK - 1) / C::BLOCK), static_cast<unsigned>(chunks),
+            static_cast<unsigned>(nrhs));
   if constexpr (CRED) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -1029,11 +1055,12 @@ cudaError_t launch_partial_form(int64_t N, const void* pos, const void* x, void*
 
 // `chunks` source chunks, partial-sum clusters of at most `maxcl` CTAs (1:
 // no cluster reduction), `atomic`: all chunks added into one slice in L2
-// (FP32); writes partial_slices(chunks, maxcl, atomic) partial slices (the
+// (FP32; the caller hands that slice over zeroed); writes, for each of nrhs
+// right-hand sides, partial_slices(chunks, maxcl, atomic) partial slices (the
 // count the epilogue must add)
 template <int L, typename R, typename C = Config<L, R>>
 cudaError_t launch_partial(int64_t N, const void* pos, const void* x, void* partial, double k, int chunks,
-                           cudaStream_t st, int maxcl = 1, bool atomic = false) {
+                           cudaStream_t st, int maxcl = 1, bool atomic = false, int nrhs = 1) {
   const int occ = partial_occupancy<L, R, C>();
   if (occ < 1) return cudaErrorInvalidConfiguration;
   if (N <= 0) return cudaSuccess;
@@ -1042,12 +1069,12 @@ cudaError_t launch_partial(int64_t N, const void* pos, const void* x, void* part
   constexpr bool AT_OK = partial_atomic<R>(true);
   if (ncl > 1) {
     if constexpr (C::ACC_SMEM) {
-      if (AT_OK && atomic) return launch_partial_form<L, R, C, true, AT_OK>(N, pos, x, partial, k, chunks, ncl, st);
-      return launch_partial_form<L, R, C, true, false>(N, pos, x, partial, k, chunks, ncl, st);
+      if (AT_OK && atomic) return launch_partial_form<L, R, C, true, AT_OK>(N, pos, x, partial, k, chunks, ncl, st, nrhs);
+      return launch_partial_form<L, R, C, true, false>(N, pos, x, partial, k, chunks, ncl, st, nrhs);
     }
   }
-  if (AT_OK && atomic) return launch_partial_form<L, R, C, false, AT_OK>(N, pos, x, partial, k, chunks, 1, st);
-  return launch_partial_form<L, R, C, false, false>(N, pos, x, partial, k, chunks, 1, st);
+  if (AT_OK && atomic) return launch_partial_form<L, R, C, false, AT_OK>(N, pos, x, partial, k, chunks, 1, st, nrhs);
+  return launch_partial_form<L, R, C, false, false>(N, pos, x, partial, k, chunks, 1, st, nrhs);
 }
 
 // persistent batched launch: one CTA per resident slot, tiles from `counter`
