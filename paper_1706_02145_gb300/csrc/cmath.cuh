@@ -42,6 +42,41 @@ __device__ __forceinline__ cd cexp_i(double phase) {
   sincos(phase, &s, &c);
   return cd{c, s};
 }
+// sin and cos of a phase by a two-constant reduction mod pi/2 (each fma rounds
+// once, relative to a remainder of at most pi/4) and Taylor series to y^17 /
+// y^16 (truncation below 2e-18): 26 FP64 instructions, about half of
+// sincos(), in the kernels that need one per (sphere, direction) or (sphere,
+// point).  Larger arguments take sincos().
+__device__ __forceinline__ void sincos_phase(double x, double* sn, double* cs) {
+  if (!(fabs(x) < 1e5)) {
+    sincos(x, sn, cs);
+    return;
+  }
+  const double n = rint(x * 0.63661977236758134308);
+  double y = fma(-n, 1.5707963267948965580, x);
+  y = fma(-n, 6.1232339957367658861e-17, y);
+  const double z = y * y;
+  double s = fma(z, 1.0 / 355687428096000.0, -1.0 / 1307674368000.0);
+  s = fma(z, s, 1.0 / 6227020800.0);
+  s = fma(z, s, -1.0 / 39916800.0);
+  s = fma(z, s, 1.0 / 362880.0);
+  s = fma(z, s, -1.0 / 5040.0);
+  s = fma(z, s, 1.0 / 120.0);
+  s = fma(z, s, -1.0 / 6.0);
+  s = fma(y * z, s, y);
+  double c = fma(z, 1.0 / 20922789888000.0, -1.0 / 87178291200.0);
+  c = fma(z, c, 1.0 / 479001600.0);
+  c = fma(z, c, -1.0 / 3628800.0);
+  c = fma(z, c, 1.0 / 40320.0);
+  c = fma(z, c, -1.0 / 720.0);
+  c = fma(z, c, 1.0 / 24.0);
+  c = fma(z, c, -0.5);
+  c = fma(z, c, 1.0);
+  const int q = static_cast<int>(n);
+  const double s0 = (q & 1) ? c : s, c0 = (q & 1) ? s : c;
+  *sn = (q & 2) ? -s0 : s0;
+  *cs = ((q + 1) & 2) ? -c0 : c0;
+}
 __device__ __forceinline__ cd csin(cd z) { return cd{sin(z.re) * cosh(z.im), cos(z.re) * sinh(z.im)}; }
 __device__ __forceinline__ cd ccos(cd z) { return cd{cos(z.re) * cosh(z.im), -sin(z.re) * sinh(z.im)}; }
 
