@@ -1642,12 +1642,14 @@ extern "C" int celes_farfield(celes_ctx* c, const double* dirs, int64_t Nd, doub
   if (!c->has_b) return fail(c, CELES_ESTATE, "farfield: no solution yet");
   if (rhs < 0 || rhs >= c->nrhs) return fail(c, CELES_EINVAL, "farfield: rhs out of range");
   DeviceGuard dg(c->device);
-  DevBuf dd, dg_;
+  DevBuf dd, dg_, work;
+  CK(work.ensure(farfield_scratch_bytes(c->N, c->L, Nd)), "far-field sums");
   CK(dd.ensure(sizeof(double) * 2 * Nd), "dirs");
   CK(dg_.ensure(sizeof(double) * 4 * Nd), "g");
   CK(cudaMemcpyAsync(dd.p, dirs, sizeof(double) * 2 * Nd, cudaMemcpyHostToDevice, c->stream), "h2d");
   const double* b = reinterpret_cast<const double*>(c->b.as<char>() + sizeof(double) * 2 * c->N * c->nmax * rhs);
-  CK(launch_farfield(c->N, c->L, c->k, c->pos.p, b, Nd, dd.as<double>(), dg_.as<double>(), c->stream), "farfield");
+  CK(launch_farfield(c->N, c->L, c->k, c->pos.p, b, Nd, dd.as<double>(), dg_.as<double>(), work.p, c->stream),
+     "farfield");
   CK(cudaMemcpyAsync(g, dg_.p, sizeof(double) * 4 * Nd, cudaMemcpyDeviceToHost, c->stream), "d2h");
   CK(cudaStreamSynchronize(c->stream), "sync");
   return CELES_OK;

@@ -105,8 +105,10 @@ cudaError_t launch_tdiag_mul(int64_t n_per_rhs, int nrhs, const double* tdiag, c
 template <typename R>
 cudaError_t launch_nonfinite(int64_t n, const void* v, int* flag, cudaStream_t st);
 
+// scratch: farfield_scratch_bytes(N, L, Nd), at most about 64 MB
+size_t farfield_scratch_bytes(int64_t N, int L, int64_t Nd);
 cudaError_t launch_farfield(int64_t N, int L, double k, const void* pos, const double* b, int64_t Nd,
-                            const double* dirs, double* g, cudaStream_t st);
+                            const double* dirs, double* g, void* scratch, cudaStream_t st);
 cudaError_t launch_overlap_check(int64_t N, const void* pos, const double* radii, int* flag, cudaStream_t st);
 
 // tensor-core GEMM (tc_gemm.cu): C = alpha A B^T + beta C, BF16 in, FP32 out

@@ -112,22 +112,26 @@ extern "C" int celes_power(celes_ctx* ctx, int rhs, int n_beta, int n_alpha, dou
   const cudaStream_t st = v.stream;
   const int nblk = 304;
   double *dd = nullptr, *dw = nullptr, *dg = nullptr, *dp = nullptr;
+  void* ds = nullptr;
   auto cleanup = [&]() {
     cudaStreamSynchronize(st);
     if (dd) cudaFree(dd);
     if (dw) cudaFree(dw);
     if (dg) cudaFree(dg);
     if (dp) cudaFree(dp);
+    if (ds) cudaFree(ds);
   };
   if (cudaMalloc(&dd, sizeof(double) * 2 * Nd) != cudaSuccess || cudaMalloc(&dw, sizeof(double) * Nd) != cudaSuccess ||
-      cudaMalloc(&dg, sizeof(double) * 4 * Nd) != cudaSuccess || cudaMalloc(&dp, sizeof(double) * 2 * nblk) != cudaSuccess) {
+      cudaMalloc(&dg, sizeof(double) * 4 * Nd) != cudaSuccess || cudaMalloc(&dp, sizeof(double) * 2 * nblk) != cudaSuccess ||
+      cudaMalloc(&ds, farfield_scratch_bytes(v.N, v.L, Nd)) != cudaSuccess) {
+    cudaGetLastError();
     cleanup();
     return CELES_ENOMEM;
   }
   cudaError_t e = cudaMemcpyAsync(dd, dirs.data(), sizeof(double) * 2 * Nd, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dw, wts.data(), sizeof(double) * Nd, cudaMemcpyHostToDevice, st);
   const double* b = v.b + (size_t)rhs * v.N * v.nmax * 2;
-  if (e == cudaSuccess) e = launch_farfield(v.N, v.L, v.k, v.pos, b, Nd, dd, dg, st);
+  if (e == cudaSuccess) e = launch_farfield(v.N, v.L, v.k, v.pos, b, Nd, dd, dg, ds, st);
   if (e == cudaSuccess) {
     // forward hemisphere with the beam, backward without it
     power_sum_kernel<<<nblk, kPowThreads, 0, st>>>(nh, nh, dd, dw, dg, v.k, d.waist, d.focus[0], d.focus[1],
@@ -204,22 +208,26 @@ extern "C" int celes_s11(celes_ctx* ctx, int rhs_a, int rhs_b, const double* bet
     }
   const cudaStream_t st = v.stream;
   double *dd = nullptr, *ga = nullptr, *gb = nullptr, *ds = nullptr;
+  void* dw = nullptr;
   auto cleanup = [&]() {
     cudaStreamSynchronize(st);
     if (dd) cudaFree(dd);
     if (ga) cudaFree(ga);
     if (gb) cudaFree(gb);
     if (ds) cudaFree(ds);
+    if (dw) cudaFree(dw);
   };
   if (cudaMalloc(&dd, sizeof(double) * 2 * Nd) != cudaSuccess || cudaMalloc(&ga, sizeof(double) * 4 * Nd) != cudaSuccess ||
-      cudaMalloc(&gb, sizeof(double) * 4 * Nd) != cudaSuccess || cudaMalloc(&ds, sizeof(double) * n_beta) != cudaSuccess) {
+      cudaMalloc(&gb, sizeof(double) * 4 * Nd) != cudaSuccess || cudaMalloc(&ds, sizeof(double) * n_beta) != cudaSuccess ||
+      cudaMalloc(&dw, farfield_scratch_bytes(v.N, v.L, Nd)) != cudaSuccess) {
+    cudaGetLastError();
     cleanup();
     return CELES_ENOMEM;
   }
   const size_t per = (size_t)v.N * v.nmax * 2;
   cudaError_t e = cudaMemcpyAsync(dd, dirs.data(), sizeof(double) * 2 * Nd, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_farfield(v.N, v.L, v.k, v.pos, v.b + per * rhs_a, Nd, dd, ga, st);
-  if (e == cudaSuccess) e = launch_farfield(v.N, v.L, v.k, v.pos, v.b + per * rhs_b, Nd, dd, gb, st);
+  if (e == cudaSuccess) e = launch_farfield(v.N, v.L, v.k, v.pos, v.b + per * rhs_a, Nd, dd, ga, dw, st);
+  if (e == cudaSuccess) e = launch_farfield(v.N, v.L, v.k, v.pos, v.b + per * rhs_b, Nd, dd, gb, dw, st);
   if (e == cudaSuccess) {
     s11_kernel<<<n_beta, kPowThreads, 0, st>>>(n_alpha, ga, gb, ds);
     note_launch();
