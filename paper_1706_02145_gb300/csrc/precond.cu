@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
 #include "cmath.cuh"
@@ -934,91 +935,132 @@ __global__ void __launch_bounds__(kTileThreads)
 }
 constexpr int kInvThreads = 256;
 
-// x = U^{-1} (L^{-1} (P y)) for one (block, RHS) per cluster of C CTAs; the
-// 32-row tiles are dealt round robin (warp w of CTA s takes tiles s + C (w +
-// 8 m)), one lane per row, so each column of a tile is one coalesced 256-byte
-// read.  Every CTA gathers the whole (pivot-permuted) block vector.
+// one complex factor, read once per apply: past the caches' retention
+__device__ __forceinline__ Pair2<float> load_stream(const Pair2<float>* p) {
+  const float2 v = __ldcs(reinterpret_cast<const float2*>(p));
+  return Pair2<float>{v.x, v.y};
+}
+__device__ __forceinline__ Pair2<double> load_stream(const Pair2<double>* p) {
+  const double2 v = __ldcs(reinterpret_cast<const double2*>(p));
+  return Pair2<double>{v.x, v.y};
+}
+
+// x = U^{-1} (L^{-1} (P y)) for one (block, RHS) per cluster of C CTAs.  Bound
+// by HBM: every factor is read once.  The 32-row tiles are dealt round robin to
+// the CTAs, one lane per row, so each column of a tile is one coalesced read of
+// 256 (FP32) or 512 bytes.  A CTA's tiles are triangular, so their columns are
+// laid end to end and cut into equal runs, one per warp, sixteen columns in
+// flight each: with whole tiles per warp the longest row of a block set the time
+// and half of the bandwidth was left (245 blocks of up to 810 unknowns, FP32:
+// 237 -> 140 us).  A tile cut between warps is added up from their
+// pieces in order, so results do not depend on timing.  Every CTA gathers the
+// whole (pivot-permuted) block vector.
 template <typename R, typename F>
-__global__ void __launch_bounds__(kInvThreads) precond_apply_inv_kernel(const int64_t* __restrict__ block_off,
-                                                                        const int64_t* __restrict__ mat_off, int nmax,
-                                                                        const int* __restrict__ perm,
-                                                                        const Pair2<F>* __restrict__ inv,
-                                                                        const int* __restrict__ pivperm, int64_t N,
-                                                                        const Pair2<R>* __restrict__ x,
-                                                                        Pair2<R>* __restrict__ y) {
+__global__ void __launch_bounds__(kInvThreads, 3)
+    precond_apply_inv_kernel(const int64_t* __restrict__ block_off, const int64_t* __restrict__ mat_off, int nmax,
+                             const int* __restrict__ perm, const Pair2<F>* __restrict__ inv,
+                             const int* __restrict__ pivperm, int64_t N, const Pair2<R>* __restrict__ x,
+                             Pair2<R>* __restrict__ y) {
   using V = Pair2<F>;
+  constexpr int NW = kInvThreads / 32;
+  constexpr int U = sizeof(F) == 4 ? 16 : 8;  // columns in flight
   extern __shared__ __align__(16) unsigned char pi_smem[];
+  __shared__ V head[NW][32];
   cg::cluster_group cluster = cg::this_cluster();
   const int C = static_cast<int>(cluster.num_blocks());
   const int s = static_cast<int>(cluster.block_rank());
   const int64_t q = blockIdx.x / C;
   const int rhs = blockIdx.y;
   const int64_t s0 = block_off[q];
-  const int64_t n = (block_off[q + 1] - s0) * nmax;
-  const int64_t T = (n + 31) / 32;
+  const int n = static_cast<int>((block_off[q + 1] - s0) * nmax);
+  const int T = (n + 31) / 32;
   const V* A = inv + mat_off[q];
   const int* pp = pivperm + s0 * nmax;
   const Pair2<R>* xr = x + (int64_t)rhs * N * nmax;
   Pair2<R>* yr = y + (int64_t)rhs * N * nmax;
   V* xv = reinterpret_cast<V*>(pi_smem);  // [n] P y
   V* tv = xv + n;                         // [n] t = L^{-1} P y
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  constexpr int NW = kInvThreads / 32;
-  for (int64_t t = tid; t < n; t += blockDim.x) {
-    const int64_t src = pp[t];
-    const int64_t a = src / nmax;
-    const int r = static_cast<int>(src - a * nmax);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  for (int t = tid; t < n; t += blockDim.x) {
+    const int src = pp[t];
+    const int a = src / nmax;
+    const int r = src - a * nmax;
     const Pair2<R> e = xr[(int64_t)perm[s0 + a] * nmax + r];
     xv[t] = V{static_cast<F>(e.re), static_cast<F>(e.im)};
   }
   // every CTA of the cluster has started (and gathered) before any writes
   // into another's shared memory
   cluster.sync();
-  // row i: sum over columns [j0, j1) of A[i, j] v[j]
-  auto rowdot = [&](int64_t i, int64_t j0, int64_t j1, const V* v) {
-    F ar0 = 0, ai0 = 0, ar1 = 0, ai1 = 0;
-    const V* a = A + i;
-    int64_t jj = j0;
-    for (; jj + 8 <= j1; jj += 8) {
-      V m[8];
+  const int m = T > s ? (T - s + C - 1) / C : 0;  // own tiles: s + C k, k < m
+  // one triangular product; emit(row, sum) by the lane of the row
+  auto sweep = [&](auto lower_, const V* v, auto emit) {
+    constexpr bool LOWER = decltype(lower_)::value;
+    auto first = [&](int k) { return LOWER ? 0 : 32 * (s + C * k); };
+    auto count = [&](int k) { return LOWER ? min(32 * (s + C * k + 1), n) : n - 32 * (s + C * k); };
+    int64_t tot = 0;
+    for (int k = 0; k < m; ++k) tot += count(k);
+    const int64_t a0 = tot * w / NW, a1 = tot * (w + 1) / NW;
+    int64_t base = 0, tail_end = -1;
+    int tail_row = 0;
+    V tail{0, 0};
+    for (int k = 0; k < m && base < a1; ++k) {
+      const int64_t end = base + count(k);
+      const int64_t lo = a0 > base ? a0 : base, hi = a1 < end ? a1 : end;
+      if (lo < hi) {
+        const int i = 32 * (s + C * k) + lane;
+        const int j0 = first(k) + static_cast<int>(lo - base), j1 = first(k) + static_cast<int>(hi - base);
+        // columns of this row's triangle: j < i (unit diagonal implied) or j >= i
+        const int b0 = i >= n ? j1 : (LOWER ? 0 : i), b1 = LOWER ? i : n;
+        F re0 = 0, im0 = 0, re1 = 0, im1 = 0;
+        for (int j = j0; j < j1; j += U) {
+          V c[U];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) m[u] = a[(jj + u) * n];
+          for (int u = 0; u < U; ++u)
+            c[u] = j + u < j1 && j + u >= b0 && j + u < b1 ? load_stream(A + i + (int64_t)(j + u) * n) : V{0, 0};
 #pragma unroll
-      for (int u = 0; u < 8; u += 2) {
-        const V v0 = v[jj + u], v1 = v[jj + u + 1];
-        ar0 += m[u].re * v0.re - m[u].im * v0.im;
-        ai0 += m[u].re * v0.im + m[u].im * v0.re;
-        ar1 += m[u + 1].re * v1.re - m[u + 1].im * v1.im;
-        ai1 += m[u + 1].re * v1.im + m[u + 1].im * v1.re;
+          for (int u = 0; u < U; u += 2) {
+            const V v0 = v[min(j + u, n - 1)], v1 = v[min(j + u + 1, n - 1)];
+            re0 += c[u].re * v0.re - c[u].im * v0.im;
+            im0 += c[u].re * v0.im + c[u].im * v0.re;
+            re1 += c[u + 1].re * v1.re - c[u + 1].im * v1.im;
+            im1 += c[u + 1].re * v1.im + c[u + 1].im * v1.re;
+          }
+        }
+        const V sum{re0 + re1, im0 + im1};
+        if (lo > base) {
+          head[w][lane] = sum;  // a tile that an earlier warp began
+        } else if (hi < end) {
+          tail = sum;
+          tail_end = end;
+          tail_row = i;
+        } else if (i < n) {
+          emit(i, sum);
+        }
       }
+      base = end;
     }
-    for (; jj < j1; ++jj) {
-      const V m = a[jj * n], v0 = v[jj];
-      ar0 += m.re * v0.re - m.im * v0.im;
-      ai0 += m.re * v0.im + m.im * v0.re;
+    __syncthreads();
+    if (tail_end >= 0) {
+      for (int o = w + 1; o < NW && tot * o / NW < tail_end; ++o) {
+        if (tot * o / NW == tot * (o + 1) / NW) continue;  // an empty run
+        tail.re += head[o][lane].re;
+        tail.im += head[o][lane].im;
+      }
+      if (tail_row < n) emit(tail_row, tail);
     }
-    return V{ar0 + ar1, ai0 + ai1};
   };
-  // t = L^{-1} P y on own tiles (unit diagonal), into every CTA's copy of t
-  for (int64_t tt = s + (int64_t)C * wid; tt < T; tt += (int64_t)C * NW) {
-    const int64_t i = tt * 32 + lane;
-    if (i < n) {
-      const V d = rowdot(i, 0, i, xv);
-      const V t = V{xv[i].re + d.re, xv[i].im + d.im};
-      for (int dst = 0; dst < C; ++dst) cluster.map_shared_rank(tv, dst)[i] = t;
-    }
-  }
+  // t = L^{-1} P y on own tiles, into every CTA's copy of t
+  sweep(std::true_type{}, xv, [&](int i, V d) {
+    const V t = V{xv[i].re + d.re, xv[i].im + d.im};
+    for (int dst = 0; dst < C; ++dst) cluster.map_shared_rank(tv, dst)[i] = t;
+  });
   cluster.sync();
   // x = U^{-1} t on own tiles
-  for (int64_t tt = s + (int64_t)C * wid; tt < T; tt += (int64_t)C * NW) {
-    const int64_t i = tt * 32 + lane;
-    if (i < n) {
-      const V o = rowdot(i, i, n, tv);
-      const int64_t a = i / nmax;
-      const int r = static_cast<int>(i - a * nmax);
-      yr[(int64_t)perm[s0 + a] * nmax + r] = Pair2<R>{static_cast<R>(o.re), static_cast<R>(o.im)};
-    }
-  }
+  sweep(std::false_type{}, tv, [&](int i, V o) {
+    const int a = i / nmax;
+    const int r = i - a * nmax;
+    yr[(int64_t)perm[s0 + a] * nmax + r] = Pair2<R>{static_cast<R>(o.re), static_cast<R>(o.im)};
+  });
 }
 
 // FP64 explicit inverses of L and U of every block (from the FP64 LU and
@@ -1186,6 +1228,11 @@ template <typename R>
 cudaError_t launch_apply_inv(int64_t nblocks, const int64_t* block_off, const int64_t* mat_off, int nmax,
                              const int* perm, const R* inv, const int* pivperm, int64_t N, int nrhs, const void* x,
                              void* y, int max_block_dim, int csize, cudaStream_t st) {
+  // three CTAs per SM keep enough loads in flight; more per block only where
+  // there are fewer blocks, and for blocks with tiles to share out
+  const int most = csize >= 4 ? 8 : (csize >= 2 ? 4 : 1);
+  csize = 1;
+  while (csize < most && nblocks * nrhs * csize < 3LL * device_sms()) csize *= 2;
   static PerDevice attr;
   cudaError_t se = cudaSuccess;
   if (attr.get(current_device, [&] {
