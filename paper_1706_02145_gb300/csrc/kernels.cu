@@ -677,20 +677,21 @@ template cudaError_t launch_nonfinite<double>(int64_t, const void*, int*, cudaSt
 // (direction, sphere, n) (complex products as three real ones) plus the phase,
 // 26 instructions per (direction, sphere); one CTA per direction contracting
 // with both B_nj per sphere took 8 FMAs and a full sincos.  GB300, 10 000
-// spheres, lmax 4, 2 048 directions: 23.8 -> 6.3 ms.
+// spheres, lmax 4, 2 048 directions: 23.8 -> 6.1 ms.
 // ---------------------------------------------------------------------------
-constexpr int kFfDirs = 64;     // directions of a CTA
 constexpr int kFfTile = 8;      // spheres staged at a time
 constexpr int kFfThreads = 256;
+constexpr int kFfMaxL = 5;
 
 // grid (direction tiles, sphere chunks): F [chunk][direction][nmax] complex.
-// Thread (tx, ty) = (tid & 15, tid >> 4) holds directions 4 ty .. 4 ty + 3 and
-// rows tx + 16 u, u < NPT.
-template <int NPT>
+// Thread (tx, ty) = (tid & 15, tid >> 4) holds DT directions from DT ty and rows
+// tx + 16 u, u < NPT.
+template <int NPT, int DT>
 __global__ void __launch_bounds__(kFfThreads)
     farfield_sum_kernel(int64_t N, int64_t chunk, int nmax, double k, const Pos4* __restrict__ pos,
                         const double2* __restrict__ b, int64_t Nd, const double* __restrict__ dirs,
                         double2* __restrict__ F) {
+  constexpr int kFfDirs = 16 * DT;
   __shared__ double kv[kFfDirs][3];
   __shared__ double pc[kFfTile][kFfDirs], ps[kFfTile][kFfDirs], pt[kFfTile][kFfDirs];
   __shared__ double br[kFfTile][16 * NPT], bi[kFfTile][16 * NPT], bt[kFfTile][16 * NPT];
@@ -699,14 +700,14 @@ __global__ void __launch_bounds__(kFfThreads)
   if (tid < kFfDirs) {
     const int64_t d = d0 + tid < Nd ? d0 + tid : Nd - 1;
     double sb, cb, sa, ca;
-    sincos(dirs[2 * d], &sb, &cb);
-    sincos(dirs[2 * d + 1], &sa, &ca);
+    sincos_phase(dirs[2 * d], &sb, &cb);
+    sincos_phase(dirs[2 * d + 1], &sa, &ca);
     kv[tid][0] = k * sb * ca;
     kv[tid][1] = k * sb * sa;
     kv[tid][2] = k * cb;
   }
   // products P1 = c br, P2 = s bi, P3 = (c + s)(br + bi) of the phase c + i s
-  double p1[4][NPT] = {}, p2[4][NPT] = {}, p3[4][NPT] = {};
+  double p1[DT][NPT] = {}, p2[DT][NPT] = {}, p3[DT][NPT] = {};
   const int64_t i0 = blockIdx.y * chunk, i1 = i0 + chunk < N ? i0 + chunk : N;
   for (int64_t it = i0; it < i1; it += kFfTile) {
     const int ni = static_cast<int>(i1 - it < kFfTile ? i1 - it : kFfTile);
@@ -736,17 +737,17 @@ __global__ void __launch_bounds__(kFfThreads)
       for (int u = 0; u < NPT; ++u) {
         const double vr = br[j][tx + 16 * u], vi = bi[j][tx + 16 * u], vt = bt[j][tx + 16 * u];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          p1[a][u] = fma(pc[j][4 * ty + a], vr, p1[a][u]);
-          p2[a][u] = fma(ps[j][4 * ty + a], vi, p2[a][u]);
-          p3[a][u] = fma(pt[j][4 * ty + a], vt, p3[a][u]);
+        for (int a = 0; a < DT; ++a) {
+          p1[a][u] = fma(pc[j][DT * ty + a], vr, p1[a][u]);
+          p2[a][u] = fma(ps[j][DT * ty + a], vi, p2[a][u]);
+          p3[a][u] = fma(pt[j][DT * ty + a], vt, p3[a][u]);
         }
       }
     }
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int64_t d = d0 + 4 * ty + a;
+  for (int a = 0; a < DT; ++a) {
+    const int64_t d = d0 + DT * ty + a;
 #pragma unroll
     for (int u = 0; u < NPT; ++u) {
       const int n = tx + 16 * u;
@@ -757,105 +758,211 @@ __global__ void __launch_bounds__(kFfThreads)
   }
 }
 
-// one warp per direction: the chunks of F added in order, then the contraction
+// constants of the recursions of pi_l^m (pi_tau_m in cmath.cuh), for one m per thread
+struct PiTable {
+  double d[kFfMaxL + 1], a[kFfMaxL + 1][kFfMaxL + 1], ab[kFfMaxL + 1][kFfMaxL + 1], f[kFfMaxL + 1][kFfMaxL + 1];
+  double norm[kFfMaxL + 1], tau0[kFfMaxL + 1];
+};
+constexpr PiTable make_pi_table() {
+  PiTable t{};
+  for (int m = 0; m <= kFfMaxL; ++m) {
+    const int mm = m == 0 ? 1 : m;  // tau_l^0 comes from pi_l^1
+    t.d[m] = 0.70710678118654752440;
+    for (int q = 1; q <= mm; ++q) t.d[m] *= tab::csqrt((2.0 * q + 1.0) / (2.0 * q));
+    for (int l = mm; l <= kFfMaxL; ++l) {
+      if (l == mm + 1) t.a[m][l] = tab::csqrt(2.0 * mm + 3.0);
+      if (l > mm + 1) {
+        t.a[m][l] = tab::csqrt((4.0 * l * l - 1.0) / (1.0 * l * l - 1.0 * mm * mm));
+        t.ab[m][l] = t.a[m][l] * tab::csqrt(((l - 1.0) * (l - 1.0) - 1.0 * mm * mm) / (4.0 * (l - 1.0) * (l - 1.0) - 1.0));
+      }
+      t.f[m][l] = tab::csqrt((2.0 * l + 1.0) * (1.0 * l * l - 1.0 * m * m) / (2.0 * l - 1.0));
+    }
+  }
+  for (int l = 1; l <= kFfMaxL; ++l) {
+    t.norm[l] = 1.0 / tab::csqrt(2.0 * l * (l + 1.0));
+    t.tau0[l] = -tab::csqrt(l * (l + 1.0));
+  }
+  return t;
+}
+__constant__ PiTable kPiTable = make_pi_table();
+
+// eight lanes per direction, lane |m|: the chunks of F added in order, then the
+// contraction with B_nj e^{i m alpha} of both orders +-m
 __global__ void __launch_bounds__(128)
     farfield_contract_kernel(int64_t Nd, int chunks, int L, const double* __restrict__ dirs,
                              const double2* __restrict__ F, double* __restrict__ g) {
-  const int nmax = 2 * L * (L + 2);
-  const int lane = threadIdx.x & 31;
-  const int64_t d = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (d >= Nd) return;
-  double sb, cb;
-  sincos(dirs[2 * d], &sb, &cb);
-  const double alpha = dirs[2 * d + 1];
+  const int NH = L * (L + 2), nmax = 2 * NH;
+  const int am = threadIdx.x & 7;
+  const int64_t d = blockIdx.x * (int64_t)(blockDim.x >> 3) + (threadIdx.x >> 3);
   cd g1 = mkc(0.0), g2 = mkc(0.0);
-  for (int n = lane; n < nmax; n += 32) {
-    cd f = mkc(0.0);
-    for (int c = 0; c < chunks; ++c) {
-      const double2 v = F[((int64_t)c * Nd + d) * nmax + n];
-      f = f + cd{v.x, v.y};
+  if (d < Nd && am <= L) {
+    double sb, cb;
+    sincos_phase(dirs[2 * d], &sb, &cb);
+    cd em;
+    sincos_phase(am * dirs[2 * d + 1], &em.im, &em.re);
+    const int l0 = am == 0 ? 1 : am;
+    double pl = kPiTable.d[am], prev = 0.0;
+    for (int q = 1; q < l0; ++q) pl *= sb;
+    for (int l = l0; l <= L; ++l) {
+      if (l > l0) {
+        const double nx = kPiTable.a[am][l] * cb * pl - kPiTable.ab[am][l] * prev;
+        prev = pl;
+        pl = nx;
+      }
+      const double tau = am == 0 ? kPiTable.tau0[l] * sb * pl : l * cb * pl - kPiTable.f[am][l] * prev;
+      const double mp = am * pl;
+      // sums over the chunks of the rows (tau 1, 2) of +m and -m
+      cd f[4] = {};
+      const int r = l * (l + 1) - 1;
+      for (int c = 0; c < chunks; ++c) {
+        const double2* Fc = F + ((int64_t)c * Nd + d) * nmax;
+        const double2 v0 = Fc[r + am], v1 = Fc[NH + r + am];
+        f[0] = f[0] + cd{v0.x, v0.y};
+        f[1] = f[1] + cd{v1.x, v1.y};
+        if (am > 0) {
+          const double2 w0 = Fc[r - am], w1 = Fc[NH + r - am];
+          f[2] = f[2] + cd{w0.x, w0.y};
+          f[3] = f[3] + cd{w1.x, w1.y};
+        }
+      }
+      // B_n1 = -(1/i^{l+1}) norm i ang, B_n2 = -(1/i^{l+1}) norm ang; ang = tau for j = tau index, else m pi
+      const cd a = em * f[0], b = em * f[1], c = conj(em) * f[2], e = conj(em) * f[3];
+      const cd pre = (-kPiTable.norm[l]) * ipow(-(l + 1));
+      g1 = g1 + pre * (cd{0, 1} * (tau * (a + c) + mp * (b - e)));
+      g2 = g2 + pre * (mp * (a - c) + tau * (b + e));
     }
-    int tau, l, m;
-    row_decode(n, L, tau, l, m);
-    double pi[16], ta[16];
-    pi_tau_m(L, m < 0 ? -m : m, cb, sb, pi, ta);
-    f = f * cexp_i(m * alpha);
-    g1 = g1 + b_transform(tau, l, m, 1, pi[l], ta[l], false) * f;
-    g2 = g2 + b_transform(tau, l, m, 2, pi[l], ta[l], false) * f;
   }
   double v[4] = {g1.re, g1.im, g2.re, g2.im};
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
-    if (lane == 0) g[4 * d + q] = v[q] / (2.0 * 3.14159265358979323846);
+    for (int o = 4; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o, 8);
+    if (d < Nd && am == 0) g[4 * d + q] = v[q] / (2.0 * 3.14159265358979323846);
   }
 }
 
-// directions of one pass and sphere chunks: chunks so that few directions fill
-// the GPU too (four CTAs per SM), both within 64 MB of scratch
-static void farfield_shape(int64_t N, int L, int64_t Nd, int64_t* nd, int64_t* chunks) {
-  const int64_t row = 16LL * 2 * L * (L + 2), cap = int64_t(64) << 20;
-  *nd = std::min(Nd, cap / row / kFfDirs * kFfDirs);
-  const int64_t tiles = (*nd + kFfDirs - 1) / kFfDirs;
-  int64_t ch = (4LL * device_sms() + tiles - 1) / tiles;
-  ch = std::min(ch, (N + 2 * kFfTile - 1) / (2 * kFfTile));
-  *chunks = std::max<int64_t>(1, std::min(ch, cap / (row * *nd)));
+// Directions of a tile and of one pass, and sphere chunks.  64 directions a CTA
+// and chunks for four CTAs per SM, within 64 MB of scratch; a problem too small
+// for that takes tiles of 16 and at most 0.9 MB (a device allocation above 1 MB
+// costs a first call as much as the evaluation: 114 spheres, 399 directions).
+struct FarfieldShape {
+  int64_t tile, nd, chunks;
+};
+static FarfieldShape farfield_shape(int64_t N, int L, int64_t Nd) {
+  const int64_t row = 16LL * 2 * L * (L + 2), most = (N + kFfTile - 1) / kFfTile;
+  const bool small = (Nd + 63) / 64 * most < 4LL * device_sms();
+  const int64_t cap = small ? 900000 : int64_t(64) << 20;
+  FarfieldShape f;
+  f.tile = small ? 16 : 64;
+  f.nd = std::min(Nd, std::max<int64_t>(f.tile, (int64_t(64) << 20) / row / f.tile * f.tile));
+  const int64_t tiles = (f.nd + f.tile - 1) / f.tile;
+  const int64_t ch = std::min<int64_t>((4LL * device_sms() + tiles - 1) / tiles, most);
+  f.chunks = std::max<int64_t>(1, std::min(ch, cap / (row * f.nd)));
+  return f;
 }
 size_t farfield_scratch_bytes(int64_t N, int L, int64_t Nd) {
-  int64_t nd = 0, ch = 0;
-  farfield_shape(N, L, Nd, &nd, &ch);
-  return static_cast<size_t>(nd * ch) * 16 * 2 * L * (L + 2);
+  const FarfieldShape f = farfield_shape(N, L, Nd);
+  return static_cast<size_t>(f.nd * f.chunks) * 16 * 2 * L * (L + 2);
+}
+
+template <int DT>
+static void launch_farfield_sum(int64_t N, int nmax, double k, const Pos4* p, const double2* b, int64_t n, int64_t ch,
+                                const double* dirs, double2* F, cudaStream_t st) {
+  const dim3 grid(static_cast<unsigned>((n + 16 * DT - 1) / (16 * DT)), static_cast<unsigned>(ch));
+  const int64_t chunk = (N + ch - 1) / ch;
+  switch ((nmax + 15) / 16) {
+    case 1: farfield_sum_kernel<1, DT><<<grid, kFfThreads, 0, st>>>(N, chunk, nmax, k, p, b, n, dirs, F); break;
+    case 2: farfield_sum_kernel<2, DT><<<grid, kFfThreads, 0, st>>>(N, chunk, nmax, k, p, b, n, dirs, F); break;
+    case 3: farfield_sum_kernel<3, DT><<<grid, kFfThreads, 0, st>>>(N, chunk, nmax, k, p, b, n, dirs, F); break;
+    default: farfield_sum_kernel<5, DT><<<grid, kFfThreads, 0, st>>>(N, chunk, nmax, k, p, b, n, dirs, F); break;
+  }
 }
 
 cudaError_t launch_farfield(int64_t N, int L, double k, const void* pos, const double* b, int64_t Nd,
                             const double* dirs, double* g, void* scratch, cudaStream_t st) {
   const int nmax = 2 * L * (L + 2);
-  int64_t nd = 0, ch = 0;
-  farfield_shape(N, L, Nd, &nd, &ch);
-  const int64_t chunk = (N + ch - 1) / ch;
+  const FarfieldShape f = farfield_shape(N, L, Nd);
   double2* F = static_cast<double2*>(scratch);
   const auto* p = static_cast<const Pos4*>(pos);
   const auto* bv = reinterpret_cast<const double2*>(b);
-  for (int64_t d0 = 0; d0 < Nd; d0 += nd) {
-    const int64_t n = std::min(nd, Nd - d0);
-    const dim3 grid(static_cast<unsigned>((n + kFfDirs - 1) / kFfDirs), static_cast<unsigned>(ch));
-    const double* dd = dirs + 2 * d0;
-    switch ((nmax + 15) / 16) {
-      case 1: farfield_sum_kernel<1><<<grid, kFfThreads, 0, st>>>(N, chunk, nmax, k, p, bv, n, dd, F); break;
-      case 2: farfield_sum_kernel<2><<<grid, kFfThreads, 0, st>>>(N, chunk, nmax, k, p, bv, n, dd, F); break;
-      case 3: farfield_sum_kernel<3><<<grid, kFfThreads, 0, st>>>(N, chunk, nmax, k, p, bv, n, dd, F); break;
-      default: farfield_sum_kernel<5><<<grid, kFfThreads, 0, st>>>(N, chunk, nmax, k, p, bv, n, dd, F); break;
-    }
-    farfield_contract_kernel<<<static_cast<unsigned>((n + 3) / 4), 128, 0, st>>>(n, static_cast<int>(ch), L, dd, F,
-                                                                                 g + 4 * d0);
+  for (int64_t d0 = 0; d0 < Nd; d0 += f.nd) {
+    const int64_t n = std::min(f.nd, Nd - d0);
+    if (f.tile == 16) launch_farfield_sum<1>(N, nmax, k, p, bv, n, f.chunks, dirs + 2 * d0, F, st);
+    else launch_farfield_sum<4>(N, nmax, k, p, bv, n, f.chunks, dirs + 2 * d0, F, st);
+    farfield_contract_kernel<<<static_cast<unsigned>((n + 15) / 16), 128, 0, st>>>(n, static_cast<int>(f.chunks), L,
+                                                                                   dirs + 2 * d0, F, g + 4 * d0);
     note_launch(2);
   }
   return cudaGetLastError();
 }
 
-// overlap check: flag[0] = 1 if some pair overlaps (|r_i - r_j| < R_i + R_j)
-__global__ void overlap_kernel(int64_t N, const Pos4* __restrict__ pos, const double* __restrict__ radii,
-                               int* __restrict__ flag) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// overlap check: flag[0] = 1 if some pair overlaps (|r_i - r_j| < R_i + R_j).
+// Every pair in FP32 relative to the first sphere, widened by a bound on the
+// rounding of both coordinates; only pairs that this cannot clear (neighbours,
+// and anything not finite in FP32) are tested in FP64.  Grid (row tiles,
+// column tiles), upper triangle; one thread per row against a staged tile.
+// (10 000 spheres: 4.7 ms with one FP64 thread per sphere over all later ones,
+// 0.03 ms so.)
+constexpr int kOvTile = 256;
+
+__global__ void __launch_bounds__(kOvTile)
+    overlap_kernel(int64_t N, int64_t y0, const Pos4* __restrict__ pos, const double* __restrict__ radii,
+                   int* __restrict__ flag) {
+  const int64_t jt = y0 + blockIdx.y;  // column tile
+  if (jt < blockIdx.x) return;
+  __shared__ float4 sp[kOvTile];
+  __shared__ float se[kOvTile];
+  const Pos4 o = pos[0];
+  auto load = [&](int64_t i, float4& p, float& e) {
+    const Pos4 r = pos[i];
+    p = make_float4(static_cast<float>(r.x - o.x), static_cast<float>(r.y - o.y), static_cast<float>(r.z - o.z),
+                    static_cast<float>(radii[i]));
+    // 2^-21 of the largest coordinate and of the radius: over four times the rounding of a
+    // coordinate, of the sum of radii and of the distance formed from them
+    e = 4.8e-7f * (fmaxf(fmaxf(fabsf(p.x), fabsf(p.y)), fabsf(p.z)) + p.w);
+  };
+  const int64_t i = blockIdx.x * (int64_t)kOvTile + threadIdx.x, j0 = jt * kOvTile;
+  const int nj = static_cast<int>(N - j0 < kOvTile ? N - j0 : kOvTile);
+  load(j0 + threadIdx.x < N ? j0 + threadIdx.x : N - 1, sp[threadIdx.x], se[threadIdx.x]);
+  __syncthreads();
   if (i >= N) return;
-  const Pos4 a = pos[i];
-  const double ra = radii[i];
-  for (int64_t j = i + 1; j < N; ++j) {
-    const Pos4 b = pos[j];
-    const double dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
-    const double s = ra + radii[j];
-    if (dx * dx + dy * dy + dz * dz < s * s) {
-      *flag = 1;
-      return;
+  float4 p;
+  float e;
+  load(i, p, e);
+  bool hit = false;
+  for (int jb = 0; jb < nj; jb += 32) {
+    // candidates of 32 columns as a mask first: with the FP64 test inside this
+    // loop the compiler predicates it, and it takes the FP64 pipe for every pair
+    unsigned near = 0;
+#pragma unroll 8
+    for (int u = 0; u < 32; ++u) {
+      const float4 q = sp[jb + u];
+      const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
+      const float s = (p.w + q.w) + 2.0f * (e + se[jb + u]);
+      near |= (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > s * s ? 0u : 1u) << u;
+    }
+    if (nj - jb < 32) near &= (1u << (nj - jb)) - 1u;
+    while (near) {
+      const int64_t j = j0 + jb + __ffs(near) - 1;
+      near &= near - 1;
+      if (j <= i) continue;
+      const Pos4 a = pos[i], b = pos[j];
+      const double ax = a.x - b.x, ay = a.y - b.y, az = a.z - b.z;
+      const double t = radii[i] + radii[j];
+      if (ax * ax + ay * ay + az * az < t * t) hit = true;
     }
   }
+  if (hit) *flag = 1;
 }
 
 cudaError_t launch_overlap_check(int64_t N, const void* pos, const double* radii, int* flag, cudaStream_t st) {
-  const int threads = 128;
-  overlap_kernel<<<static_cast<unsigned>((N + threads - 1) / threads), threads, 0, st>>>(
-      N, static_cast<const Pos4*>(pos), radii, flag);
-  note_launch();
+  const int64_t tiles = (N + kOvTile - 1) / kOvTile;
+  // the grid's second extent ends at 65 535 tiles (16.7 million spheres): bands of columns
+  for (int64_t y0 = 0; y0 < tiles; y0 += 65535) {
+    const int64_t ny = tiles - y0 < 65535 ? tiles - y0 : 65535;
+    overlap_kernel<<<dim3(static_cast<unsigned>(tiles), static_cast<unsigned>(ny)), kOvTile, 0, st>>>(
+        N, y0, static_cast<const Pos4*>(pos), radii, flag);
+    note_launch();
+  }
   return cudaGetLastError();
 }
 

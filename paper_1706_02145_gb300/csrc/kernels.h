@@ -50,6 +50,10 @@ struct CtxView {
 int ctx_view(celes_ctx* c, CtxView* v);
 // store a learned first iterate for RHS `rhs` (device pointer, complex128 [N][nmax])
 int ctx_set_learned_guess(celes_ctx* c, int rhs, const double* b0_dev);
+// the context's device workspace for one call, at least `bytes` (contents
+// undefined); done: the call's stream is synchronised, a large one is given back
+cudaError_t ctx_workspace(celes_ctx* c, size_t bytes, void** p);
+void ctx_workspace_done(celes_ctx* c);
 // the solution buffer (b, [nrhs][N][nmax] complex128) now holds a solution
 int ctx_mark_solved(celes_ctx* c);
 

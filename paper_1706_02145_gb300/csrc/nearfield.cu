@@ -412,26 +412,29 @@ extern "C" int celes_nearfield(celes_ctx* ctx, const double* points, int64_t Np,
   } restore{prev};
   const cudaStream_t st = v.stream;
   // chunks of spheres so that small maps fill the GPU too (eight CTAs of two
-  // warps per SM), with slices of at most 64 MB
+  // warps per SM; a sphere takes 8 us one after another), with slices of at
+  // most 64 MB
   const int64_t tiles = (Np + kNfPoints - 1) / kNfPoints;
   int64_t chunks = (8LL * device_sms() + tiles - 1) / tiles;
-  chunks = std::min<int64_t>(chunks, (v.N + kNfTile - 1) / kNfTile);
+  chunks = std::min<int64_t>(chunks, (v.N + 1) / 2);
   chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, (int64_t(64) << 20) / (48 * Np)));
-  double *dp = nullptr, *dE = nullptr, *dS = nullptr, *dn = nullptr, *dw = nullptr;
-  auto cleanup = [&]() {
-    cudaStreamSynchronize(st);
-    if (dp) cudaFree(dp);
-    if (dE) cudaFree(dE);
-    if (dS) cudaFree(dS);
-    if (dn) cudaFree(dn);
-    if (dw) cudaFree(dw);
-  };
-  if (cudaMalloc(&dp, sizeof(double) * 3 * Np) != cudaSuccess || cudaMalloc(&dE, sizeof(double) * 6 * Np) != cudaSuccess ||
-      (what != 1 && chunks > 1 && cudaMalloc(&dS, sizeof(double) * 6 * Np * chunks) != cudaSuccess)) {
+  // points, field, the beam's nodes and weights, slices
+  const int nb_max = v.incidents[rhs].kind == CELES_PLANE_WAVE ? 0 : (v.incidents[rhs].n_beta > 0 ? v.incidents[rhs].n_beta : 128);
+  const size_t slices = what != 1 && chunks > 1 ? static_cast<size_t>(chunks) * 6 * Np : 0;
+  void* ws = nullptr;
+  if (ctx_workspace(ctx, sizeof(double) * (9 * static_cast<size_t>(Np) + 2 * nb_max + slices), &ws) != cudaSuccess) {
     cudaGetLastError();
-    cleanup();
     return CELES_ENOMEM;
   }
+  double* dp = static_cast<double*>(ws);
+  double* dE = dp + 3 * Np;
+  double* dn = dE + 6 * Np;
+  double* dw = dn + nb_max;
+  double* dS = dw + nb_max;
+  auto cleanup = [&]() {
+    cudaStreamSynchronize(st);
+    ctx_workspace_done(ctx);
+  };
   cudaError_t e = cudaMemcpyAsync(dp, points, sizeof(double) * 3 * Np, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && what == 1) e = cudaMemsetAsync(dE, 0, sizeof(double) * 6 * Np, st);
   if (e != cudaSuccess) {
@@ -468,10 +471,6 @@ extern "C" int celes_nearfield(celes_ctx* ctx, const double* points, int64_t Np,
       const double bmax = s2 >= 1.0 ? M_PI / 2 : std::asin(std::sqrt(s2));
       std::vector<double> hx, hw;
       gauss_legendre_nodes(nb, 0.0, bmax, hx, hw);
-      if (cudaMalloc(&dn, sizeof(double) * nb) != cudaSuccess || cudaMalloc(&dw, sizeof(double) * nb) != cudaSuccess) {
-        cleanup();
-        return CELES_ENOMEM;
-      }
       if (cudaMemcpyAsync(dn, hx.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, st) != cudaSuccess ||
           cudaMemcpyAsync(dw, hw.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, st) != cudaSuccess) {
         cleanup();
