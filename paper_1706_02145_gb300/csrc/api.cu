@@ -731,6 +731,7 @@ extern "C" void celes_destroy(celes_ctx* c) {
     c->x0.release();
     c->partial.release();
     c->accum.release();
+    c->work.release();
     c->block_off.release();
     c->mat_off.release();
     c->perm.release();
@@ -838,7 +839,7 @@ extern "C" int celes_set_incident(celes_ctx* c, const celes_incident* inc, int n
   c->incidents.assign(inc, inc + nrhs);
   c->has_b = false;
   c->has_x0 = false;
-  DevBuf nodes, weights;
+  DevBuf beam;
   for (int r = 0; r < nrhs; ++r) {
     const celes_incident& d = inc[r];
     double* a = reinterpret_cast<double*>(c->ain.as<char>() + per * r);
@@ -854,14 +855,16 @@ extern "C" int celes_set_incident(celes_ctx* c, const celes_incident* inc, int n
       const double bmax = s2 >= 1.0 ? M_PI / 2 : std::asin(std::sqrt(s2));
       std::vector<double> hx, hw;
       gauss_legendre(nb, 0.0, bmax, hx, hw);
-      CK(nodes.ensure(sizeof(double) * nb), "nodes");
-      CK(weights.ensure(sizeof(double) * nb), "weights");
-      CK(cudaMemcpyAsync(nodes.p, hx.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, c->stream), "h2d");
-      CK(cudaMemcpyAsync(weights.p, hw.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, c->stream), "h2d");
+      // one allocation: nodes, weights, table
+      CK(beam.ensure(sizeof(double) * (2 * nb + gaussian_table_entries(c->L, nb))), "beam table");
+      double* nodes = beam.as<double>();
+      double* weights = nodes + nb;
+      CK(cudaMemcpyAsync(nodes, hx.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, c->stream), "h2d");
+      CK(cudaMemcpyAsync(weights, hw.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, c->stream), "h2d");
       CK(launch_gaussian_beam(c->N, c->L, c->k, c->pos.p, d.waist, d.focus, d.alpha_G, d.E0_re, d.E0_im, nb,
-                              nodes.as<double>(), weights.as<double>(), a, c->stream),
+                              nodes, weights, weights + nb, a, c->stream),
          "gaussian beam");
-      CK(cudaStreamSynchronize(c->stream), "sync");  // nodes/weights are freed at scope end
+      CK(cudaStreamSynchronize(c->stream), "sync");  // the host nodes go out of scope, the table is overwritten by the next beam
     }
   }
   CK(launch_tdiag_mul(c->N * c->nmax, nrhs, c->tdiag.as<double>(), c->ain.as<double>(), c->rhs.as<double>(),

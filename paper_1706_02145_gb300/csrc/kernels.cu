@@ -6,6 +6,7 @@
 //  * incident-field coefficients: plane wave (App. A.2) and Gaussian beam (App. C)
 //  * GMRES vector operations (Sec. 3.2): multi-dot, multi-axpy, norms, casts
 //  * far-field amplitude g_j (App. D)
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -16,6 +17,7 @@
 #include "../../include/celes.h"
 #include "cmath.cuh"
 #include "coupling_kernel.cuh"
+#include "coupling_tables.cuh"
 #include "kernels.h"
 
 namespace celes {
@@ -246,96 +248,285 @@ cudaError_t launch_plane_wave(int64_t N, int L, double k, const void* pos, doubl
 //        + 2 pi e^{+i aG} i^{|m+1|} e^{-i(m+1) phi_G} J_{|m+1|}(k rho_G sin) (d_j1 + i d_j2)/2
 // (rho_G, phi_G, z_G) cylindrical coordinates of r_i - r_G.  beta integral by
 // the Gauss-Legendre nodes/weights given in (nodes, weights).
-// One CTA per sphere; its threads take the beta nodes.  Per node a thread
-// forms what all rows of the sphere share (the Gaussian weight, e^{i k z_G
-// cos}, J_mu(k rho_G sin) for mu = 0..L+1 and pi/tau for every |m|), then adds
-// each row's term; the terms of a row are summed over the warp by shuffles and
-// over the warps in shared memory.
-constexpr int kGbThreads = 128;
+// The sums over beta that rows share: for every degree and |m| and the two
+// Bessel orders |m| - 1 and |m| + 1, Z = sum w e^{i k z cos} {tau_l^m, m pi_l^m}
+// J; the rows of both tau and of +-m combine them with factors that do not depend
+// on beta.  A CTA holds 32 spheres (lanes); per step of 8 nodes its warps first
+// form weight e^{i k z cos} and J_0 .. J_{L+1} of one node each, then add the
+// products of their (l, |m|) (12 FP64 instructions per node, where a row of the
+// per-row form took about 40, of 48 rows at lmax 4).  Bound by FP64 issue: about
+// 310 instructions per (sphere, node).  GB300, 10 000 spheres, lmax 4, 128
+// nodes: 13.9 -> 1.7 ms.  Few spheres: a cluster of up to 8 CTAs shares the
+// nodes of 32 spheres and adds the sums through distributed shared memory, in
+// rank order.
 constexpr int kGbMaxL = 5;
-constexpr int kGbMaxRows = 2 * kGbMaxL * (kGbMaxL + 2);
+constexpr int kGbSpheres = 32;
+constexpr int kGbNodes = 8;  // nodes of a step, and warps of the CTA
+constexpr int kGbThreads = kGbSpheres * kGbNodes;
+constexpr int gb_combos(int L) { return L * (L + 3) / 2; }  // (l, |m|), l = 1..L
 
-__global__ void __launch_bounds__(kGbThreads)
-    gaussian_beam_kernel(int64_t N, int L, double k, const Pos4* __restrict__ pos, double w, double fx, double fy,
-                         double fz, double alphaG, double e0r, double e0i, int nb, const double* __restrict__ nodes,
-                         const double* __restrict__ weights, double* __restrict__ a) {
-  __shared__ cd sU[2 * kGbMaxL + 1], sV[2 * kGbMaxL + 1];
-  __shared__ double red[kGbThreads / 32][kGbMaxRows][2];
-  const int nmax = 2 * L * (L + 2);
-  const int64_t i = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const Pos4 r = pos[i];
-  const double dx = r.x - fx, dy = r.y - fy, dz = r.z - fz;
-  const double rho = sqrt(dx * dx + dy * dy);
-  const double phiG = atan2(dy, dx);
-  if (tid <= 2 * L) {
-    const int m = tid - L;
-    sU[tid] = cexp_i(-alphaG - (m - 1) * phiG) * ipow(abs(m - 1));
-    sV[tid] = cexp_i(alphaG - (m + 1) * phiG) * ipow(abs(m + 1));
+// index of (l, |m|): orders ascend, then degrees
+__host__ __device__ __forceinline__ int gb_combo(int L, int l, int am) {
+  return am == 0 ? l - 1 : L + (am - 1) * (2 * L - am + 2) / 2 + (l - am);
+}
+
+// per node: weight sin cos exp(-(w k sin)^2 / 4), sin, cos, then (tau_l^m, m pi_l^m) per (l, |m|)
+__global__ void gaussian_table_kernel(int nb, int L, double k, double w, const double* __restrict__ nodes,
+                                      const double* __restrict__ weights, double* __restrict__ table) {
+  const int id = blockIdx.x * blockDim.x + threadIdx.x;  // (node, |m|)
+  const int q = id / (L + 1), am = id - q * (L + 1);
+  if (q >= nb) return;
+  const int nc = gb_combos(L);
+  double* t = table + (int64_t)q * (3 + 2 * nc);
+  double sb, cb;
+  sincos(nodes[q], &sb, &cb);
+  if (am == 0) {
+    t[0] = weights[q] * sb * cb * exp(-0.25 * (w * k * sb) * (w * k * sb));
+    t[1] = sb;
+    t[2] = cb;
   }
-  for (int q = tid; q < (kGbThreads / 32) * kGbMaxRows * 2; q += blockDim.x) (&red[0][0][0])[q] = 0.0;
-  __syncthreads();
-  for (int q0 = 0; q0 < nb; q0 += blockDim.x) {
-    const int q = q0 + tid;
-    double gw = 0.0, sb = 0.0, cb = 1.0;
-    if (q < nb) {
-      sincos(nodes[q], &sb, &cb);
-      gw = weights[q] * sb * cb * exp(-0.25 * (w * k * sb) * (w * k * sb));
-    }
-    const bool live = gw != 0.0;
-    double J[kGbMaxL + 2];
-    double pi_all[kGbMaxL + 1][kGbMaxL + 1], ta_all[kGbMaxL + 1][kGbMaxL + 1];
-    cd ez = mkc(0.0);
-    if (live) {
-      const double xr = k * rho * sb;
-      for (int mu = 0; mu <= L + 1; ++mu) J[mu] = jn(mu, xr);
-      for (int am = 0; am <= L; ++am) pi_tau_m(L, am, cb, sb, pi_all[am], ta_all[am]);
-      ez = gw * cexp_i(k * dz * cb);
-    }
-    for (int n = 0; n < nmax; ++n) {
-      cd c = mkc(0.0);
-      if (live) {
-        int tau, l, m;
-        row_decode(n, L, tau, l, m);
-        const int am = m < 0 ? -m : m;
-        // I_1 = pi (U + V), I_2 = pi (-i U + i V), U = Um J_|m-1|, V = Vm J_|m+1| (2 pi * 1/2 = pi)
-        const cd U = J[abs(m - 1)] * sU[m + L], V = J[abs(m + 1)] * sV[m + L];
-        const cd I1 = 3.14159265358979323846 * (U + V);
-        const cd I2 = 3.14159265358979323846 * (cd{0, -1} * U + cd{0, 1} * V);
-        const cd B1 = b_transform(tau, l, m, 1, pi_all[am][l], ta_all[am][l], true);
-        const cd B2 = b_transform(tau, l, m, 2, pi_all[am][l], ta_all[am][l], true);
-        c = ez * (B1 * I1 + B2 * I2);
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        c.re += __shfl_down_sync(0xffffffffu, c.re, o);
-        c.im += __shfl_down_sync(0xffffffffu, c.im, o);
-      }
-      if (lane == 0) {
-        red[wid][n][0] += c.re;
-        red[wid][n][1] += c.im;
-      }
-    }
-  }
-  __syncthreads();
-  for (int n = tid; n < nmax; n += blockDim.x) {
-    cd acc = mkc(0.0);
-    for (int q = 0; q < (int)(blockDim.x / 32); ++q) acc = acc + cd{red[q][n][0], red[q][n][1]};
-    const cd v = (k * k * w * w / 3.14159265358979323846) * (mkc(e0r, e0i) * acc);
-    a[2 * (i * nmax + n)] = v.re;
-    a[2 * (i * nmax + n) + 1] = v.im;
+  double pi[16], ta[16];
+  pi_tau_m(L, am, cb, sb, pi, ta);
+  for (int l = am > 1 ? am : 1; l <= L; ++l) {
+    t[3 + 2 * gb_combo(L, l, am)] = ta[l];
+    t[4 + 2 * gb_combo(L, l, am)] = am * pi[l];
   }
 }
 
+// J_0 .. J_M at x >= 0: Miller's downward recurrence with sum J_0 + 2 J_2 + 2
+// J_4 + .. = 1 below 8 (from order 34, or 16 below 1: what is left out is under
+// 1e-17 of J_M), the leading term below 1e-6, else j0, j1 and the upward
+// recurrence, which is stable for orders below x
+template <int M>
+__device__ __forceinline__ void bessel_orders(double x, double (&J)[M + 1]) {
+  if (x < 1e-6) {
+    J[0] = 1.0;
+#pragma unroll
+    for (int n = 1; n <= M; ++n) J[n] = J[n - 1] * (0.5 * x / n);
+    return;
+  }
+  if (x < 8.0) {
+    const double f = 2.0 / x;
+    double up = 0.0, cur = 1e-200, sum = 0.0;
+    const int top = x < 1.0 ? 16 : 34;  // even
+    double g = top * f;                  // 2 n / x
+    for (int n = top; n > M + 1; --n) {  // cur holds order n
+      if ((n & 1) == 0) sum += cur;
+      const double dn = fma(g, cur, -up);
+      g -= f;
+      up = cur;
+      cur = dn;
+    }
+#pragma unroll
+    for (int o = M + 1; o >= 0; --o) {
+      if (o <= M) J[o <= M ? o : 0] = cur;
+      if (o > 0) {
+        if ((o & 1) == 0) sum += cur;
+        const double dn = fma(o * f, cur, -up);
+        up = cur;
+        cur = dn;
+      }
+    }
+    const double r = 1.0 / fma(2.0, sum, J[0]);
+#pragma unroll
+    for (int o = 0; o <= M; ++o) J[o] *= r;
+    return;
+  }
+  J[0] = j0(x);
+  J[1] = j1(x);
+  const double f = 2.0 / x;
+#pragma unroll
+  for (int n = 1; n < M; ++n) J[n + 1] = fma(n * f, J[n], -J[n - 1]);
+}
+
+template <int L>
+struct GbSmem {
+  static constexpr int NC = gb_combos(L);
+  union {
+    struct {
+      double ezr[kGbNodes][kGbSpheres], ezi[kGbNodes][kGbSpheres];
+      double J[kGbNodes][L + 2][kGbSpheres];
+    } step;
+    double Z[NC][8][kGbSpheres];  // (tau, J_-), (tau, J_+), (m pi, J_-), (m pi, J_+), re and im each
+  };
+  cd U[2 * L + 1][kGbSpheres], V[2 * L + 1][kGbSpheres];
+};
+
+template <int L>
+__global__ void __launch_bounds__(kGbThreads)
+    gaussian_beam_kernel(int64_t N, double k, const Pos4* __restrict__ pos, double w, double fx, double fy, double fz,
+                         double alphaG, double e0r, double e0i, int nb, const double* __restrict__ table,
+                         double* __restrict__ a) {
+  extern __shared__ __align__(16) unsigned char gb_smem[];
+  GbSmem<L>& sm = *reinterpret_cast<GbSmem<L>*>(gb_smem);
+  constexpr int NC = gb_combos(L), PER = (NC + kGbNodes - 1) / kGbNodes, TS = 3 + 2 * NC;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int C = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t i0 = blockIdx.x / C * (int64_t)kGbSpheres;
+  const Pos4 r = pos[i0 + lane < N ? i0 + lane : N - 1];
+  const double dx = r.x - fx, dy = r.y - fy, kz = k * (r.z - fz);
+  const double krho = k * sqrt(dx * dx + dy * dy);
+  const double phiG = atan2(dy, dx);
+  for (int q = wid; q <= 2 * L; q += kGbNodes) {
+    const int m = q - L;
+    sm.U[q][lane] = cexp_i(-alphaG - (m - 1) * phiG) * ipow(abs(m - 1));
+    sm.V[q][lane] = cexp_i(alphaG - (m + 1) * phiG) * ipow(abs(m + 1));
+  }
+  // this warp's (l, |m|): the Bessel orders they take
+  int jm[PER], jp[PER];
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    int c = wid + u * kGbNodes, am = 0;
+    if (c >= L) {
+      c -= L;
+      am = 1;
+      while (am < L && c >= L - am + 1) {  // past the last one: not used
+        c -= L - am + 1;
+        ++am;
+      }
+    }
+    jm[u] = am == 0 ? 1 : am - 1;
+    jp[u] = am + 1;
+  }
+  double acc[PER][8] = {};
+  for (int q0 = rank * kGbNodes; q0 < nb; q0 += C * kGbNodes) {
+    __syncthreads();
+    {
+      const int q = q0 + wid;
+      double J[L + 2], g = 0.0, sn = 0.0, cs = 0.0;
+#pragma unroll
+      for (int o = 0; o <= L + 1; ++o) J[o] = 0.0;
+      if (q < nb) g = table[(int64_t)q * TS];
+      if (g != 0.0) {
+        const double* t = table + (int64_t)q * TS;
+        bessel_orders<L + 1>(krho * t[1], J);
+        sincos_phase(kz * t[2], &sn, &cs);
+      }
+      sm.step.ezr[wid][lane] = g * cs;
+      sm.step.ezi[wid][lane] = g * sn;
+#pragma unroll
+      for (int o = 0; o <= L + 1; ++o) sm.step.J[wid][o][lane] = J[o];
+    }
+    __syncthreads();
+    for (int v = 0; v < kGbNodes; ++v) {
+      if (q0 + v >= nb) break;
+      const double er = sm.step.ezr[v][lane], ei = sm.step.ezi[v][lane];
+      const double* t = table + (int64_t)(q0 + v) * TS + 3;
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        const int c = wid + u * kGbNodes;
+        if (c < NC) {
+          const double ta = t[2 * c], mp = t[2 * c + 1];
+          const double Jm = sm.step.J[v][jm[u]][lane], Jp = sm.step.J[v][jp[u]][lane];
+          const double tr = ta * er, ti = ta * ei, pr = mp * er, pi = mp * ei;
+          acc[u][0] = fma(tr, Jm, acc[u][0]);
+          acc[u][1] = fma(ti, Jm, acc[u][1]);
+          acc[u][2] = fma(tr, Jp, acc[u][2]);
+          acc[u][3] = fma(ti, Jp, acc[u][3]);
+          acc[u][4] = fma(pr, Jm, acc[u][4]);
+          acc[u][5] = fma(pi, Jm, acc[u][5]);
+          acc[u][6] = fma(pr, Jp, acc[u][6]);
+          acc[u][7] = fma(pi, Jp, acc[u][7]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const int c = wid + u * kGbNodes;
+    if (c < NC) {
+#pragma unroll
+      for (int z = 0; z < 8; ++z) sm.Z[c][z][lane] = acc[u][z];
+    }
+  }
+  cluster.sync();
+  constexpr int nmax = 2 * L * (L + 2);
+  const cd scale = (k * k * w * w / 3.14159265358979323846) * mkc(e0r, e0i);
+  // rows along the lanes: coalesced
+  for (int q = rank * kGbThreads + threadIdx.x; q < kGbSpheres * nmax; q += C * kGbThreads) {
+    const int sph = q / nmax, n = q - sph * nmax;
+    if (i0 + sph >= N) continue;
+    int tau, l, m;
+    row_decode(n, L, tau, l, m);
+    const int am = m < 0 ? -m : m, c = gb_combo(L, l, am);
+    // J_{|m-1|} and J_{|m+1|}: J_- and J_+ of |m|, the other way round for m < 0
+    const int zu = m >= 0 ? 0 : 2, zv = 2 - zu;
+    auto Z = [&](int kind, int off) {
+      cd z = mkc(0.0);
+      for (int o = 0; o < C; ++o) {
+        const GbSmem<L>& other = *cluster.map_shared_rank(&sm, o);
+        z = z + cd{other.Z[c][4 * kind + off][sph], other.Z[c][4 * kind + off + 1][sph]};
+      }
+      return z;
+    };
+    // B_nj takes tau_l^|m| for j = tau, m pi_l^|m| otherwise
+    const double sg1 = tau == 1 ? 1.0 : (m < 0 ? -1.0 : 1.0), sg2 = tau == 2 ? 1.0 : (m < 0 ? -1.0 : 1.0);
+    const int k1 = tau == 1 ? 0 : 1, k2 = tau == 2 ? 0 : 1;
+    const cd U = sm.U[m + L][sph], V = sm.V[m + L][sph];
+    // I_1 = pi (U + V), I_2 = pi (-i U + i V)
+    const cd I1 = 3.14159265358979323846 * (U * Z(k1, zu) + V * Z(k1, zv));
+    const cd I2 = 3.14159265358979323846 * (cd{0, -1} * (U * Z(k2, zu)) + cd{0, 1} * (V * Z(k2, zv)));
+    const cd B1 = b_transform(1, l, m, 1, 0.0, sg1, true), B2 = b_transform(2, l, m, 2, 0.0, sg2, true);
+    const cd v = scale * (B1 * I1 + B2 * I2);
+    a[2 * ((i0 + sph) * nmax + n)] = v.re;
+    a[2 * ((i0 + sph) * nmax + n) + 1] = v.im;
+  }
+  cluster.sync();  // no CTA leaves while others read its sums
+}
+
+int64_t gaussian_table_entries(int L, int nb) { return (int64_t)nb * (3 + 2 * gb_combos(L)); }
+
+template <int L>
+static cudaError_t launch_gaussian_t(int64_t N, double k, const void* pos, double w, const double* focus,
+                                     double alphaG, double e0r, double e0i, int nb, const double* table, double* a,
+                                     cudaStream_t st) {
+  static PerDevice attr;
+  if (attr.get(current_device, [] {
+        return cudaFuncSetAttribute(gaussian_beam_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    static_cast<int>(sizeof(GbSmem<L>))) == cudaSuccess
+                   ? 1
+                   : 0;
+      }) == 0)
+    return cudaErrorInvalidConfiguration;
+  // two CTAs per SM before the nodes are shared out
+  const int64_t tiles = (N + kGbSpheres - 1) / kGbSpheres;
+  int C = 1;
+  while (C < 8 && tiles * C * 2 <= 2 * device_sms() && C * kGbNodes < nb) C *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(tiles * C));
+  cfg.blockDim = dim3(kGbThreads);
+  cfg.dynamicSmemBytes = sizeof(GbSmem<L>);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = static_cast<unsigned>(C);
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, gaussian_beam_kernel<L>, N, k, static_cast<const Pos4*>(pos), w,
+                                           focus[0], focus[1], focus[2], alphaG, e0r, e0i, nb, table, a);
+  note_launch();
+  return e;
+}
+
+// table: device scratch of gaussian_table_entries(L, nb) doubles
 cudaError_t launch_gaussian_beam(int64_t N, int L, double k, const void* pos, double w, const double* focus,
                                  double alphaG, double e0r, double e0i, int nb, const double* nodes,
-                                 const double* weights, double* a, cudaStream_t st) {
+                                 const double* weights, double* table, double* a, cudaStream_t st) {
   if (L < 1 || L > kGbMaxL) return cudaErrorInvalidValue;
   if (N <= 0) return cudaSuccess;
-  gaussian_beam_kernel<<<static_cast<unsigned>(N), kGbThreads, 0, st>>>(
-      N, L, k, static_cast<const Pos4*>(pos), w, focus[0], focus[1], focus[2], alphaG, e0r, e0i, nb, nodes, weights,
-      a);
+  gaussian_table_kernel<<<(nb * (L + 1) + 63) / 64, 64, 0, st>>>(nb, L, k, w, nodes, weights, table);
   note_launch();
-  return cudaGetLastError();
+  switch (L) {
+    case 1: return launch_gaussian_t<1>(N, k, pos, w, focus, alphaG, e0r, e0i, nb, table, a, st);
+    case 2: return launch_gaussian_t<2>(N, k, pos, w, focus, alphaG, e0r, e0i, nb, table, a, st);
+    case 3: return launch_gaussian_t<3>(N, k, pos, w, focus, alphaG, e0r, e0i, nb, table, a, st);
+    case 4: return launch_gaussian_t<4>(N, k, pos, w, focus, alphaG, e0r, e0i, nb, table, a, st);
+    default: return launch_gaussian_t<5>(N, k, pos, w, focus, alphaG, e0r, e0i, nb, table, a, st);
+  }
 }
 
 // ---------------------------------------------------------------------------

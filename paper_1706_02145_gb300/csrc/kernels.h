@@ -77,9 +77,10 @@ cudaError_t launch_mie(int64_t N, int L, double k, const double* radii, const do
 cudaError_t launch_tq_expand(int64_t N, int L, const double* tq, double* tdiag, float* tq32, cudaStream_t st);
 cudaError_t launch_plane_wave(int64_t N, int L, double k, const void* pos, double beta, double alpha, int pol,
                               double e0r, double e0i, double* a, cudaStream_t st);
+int64_t gaussian_table_entries(int L, int nb);
 cudaError_t launch_gaussian_beam(int64_t N, int L, double k, const void* pos, double w, const double* focus,
                                  double alphaG, double e0r, double e0i, int nb, const double* nodes,
-                                 const double* weights, double* a, cudaStream_t st);
+                                 const double* weights, double* table, double* a, cudaStream_t st);
 
 // the current device's ordinal (PerDevice's device query)
 inline bool current_device(int* d) { return cudaGetDevice(d) == cudaSuccess; }
