@@ -272,6 +272,10 @@ struct celes_ctx {
   bool precond_inverse = false;  // mats / mats32 hold the inverses of L and U (two-product apply)
   // small device scratch
   DevBuf dots, dot_partial, flag;
+  void* pinned = nullptr;  // results of an Arnoldi step (host)
+  // buffers of one solve, kept for the next (at most kKeepSolve bytes in all):
+  // Krylov vectors, two work vectors, Arnoldi step, residual and correction
+  DevBuf krylov, kw, kz, kstep, kres, kcor;
   // buffers of one field evaluation, kept for the next (at most kKeepWorkspace bytes)
   DevBuf work;
   std::string err;
@@ -732,6 +736,12 @@ extern "C" void celes_destroy(celes_ctx* c) {
     c->partial.release();
     c->accum.release();
     c->work.release();
+    c->krylov.release();
+    c->kw.release();
+    c->kz.release();
+    c->kstep.release();
+    c->kres.release();
+    c->kcor.release();
     c->block_off.release();
     c->mat_off.release();
     c->perm.release();
@@ -747,6 +757,7 @@ extern "C" void celes_destroy(celes_ctx* c) {
     c->dots.release();
     c->dot_partial.release();
     c->flag.release();
+    if (c->pinned) cudaFreeHost(c->pinned);
   }
   delete c;
 }
@@ -1075,7 +1086,10 @@ struct Gmres {
   int64_t n;        // unknowns of one RHS
   int m;            // restart
   bool precond;
-  DevBuf V, w, z;   // basis (m+1 vectors), work vectors
+  DevBuf& V = c->krylov;    // basis (m+1 vectors)
+  DevBuf &w = c->kw, &z = c->kz;  // work vectors
+  DevBuf& step = c->kstep;  // scratch and result of the one-launch Arnoldi step (short vectors)
+  int step_blocks = 0;
   std::vector<std::complex<double>> H, cs_s, g;
   std::vector<double> cs_c;
   int prec() const { return sizeof(R) == 8 ? CELES_FP64 : CELES_FP32; }
@@ -1088,6 +1102,23 @@ struct Gmres {
     CK(z.ensure(vbytes()), "work");
     CK(c->dots.ensure(sizeof(double) * 2 * (m + 2)), "dots");
     CK(c->dot_partial.ensure(sizeof(double) * 2 * (m + 2) * vec_dot_blocks(n)), "dot partials");
+    step_blocks = arnoldi_blocks(n, m);
+    if (step_blocks > 0) {
+      CK(step.ensure(arnoldi_scratch_bytes(step_blocks) + sizeof(double) * 2 * (m + 1)), "Arnoldi step");
+      if (!c->pinned) CK(cudaMallocHost(&c->pinned, sizeof(double) * 2 * (kArnoldiMaxVectors + 1)), "pinned results");
+    }
+    return CELES_OK;
+  }
+  // w against V_0 .. V_kk and the next vector; h: the coefficients, hn: the norm
+  int arnoldi(int kk, std::vector<std::complex<double>>& h, double& hn) {
+    double* out = reinterpret_cast<double*>(step.as<char>() + arnoldi_scratch_bytes(step_blocks));
+    CK(launch_arnoldi<R>(n, kk + 1, V.p, n, w.p, step.p, out, c->stream), "Arnoldi step");
+    CK(cudaMemcpyAsync(c->pinned, out, sizeof(double) * (2 * (kk + 1) + 1), cudaMemcpyDeviceToHost, c->stream), "d2h");
+    CK(cudaStreamSynchronize(c->stream), "sync");
+    const double* r = static_cast<const double*>(c->pinned);
+    h.resize(kk + 1);
+    for (int j = 0; j <= kk; ++j) h[j] = std::complex<double>(r[2 * j], r[2 * j + 1]);
+    hn = norm_from_dot(r[2 * (kk + 1)]);
     return CELES_OK;
   }
   // h[0..nv) = V[0..nv)^H v, on the host
@@ -1163,23 +1194,29 @@ struct Gmres {
         s = apply_op(Vp(kk), w.p, nmv);
         if (s) return s;
         // classical Gram-Schmidt, twice
-        s = dots(V.p, kk + 1, w.p, h1);
-        if (s) return s;
-        CK(cudaMemcpyAsync(c->dots.p, h1.data(), sizeof(double) * 2 * (kk + 1), cudaMemcpyHostToDevice, c->stream),
-           "h2d");
-        CK(launch_multi_axpy<R>(n, kk + 1, V.p, n, c->dots.as<double>(), 1.0, w.p, c->stream), "axpy");
-        s = dots(V.p, kk + 1, w.p, h2);
-        if (s) return s;
-        CK(cudaMemcpyAsync(c->dots.p, h2.data(), sizeof(double) * 2 * (kk + 1), cudaMemcpyHostToDevice, c->stream),
-           "h2d");
-        CK(launch_multi_axpy<R>(n, kk + 1, V.p, n, c->dots.as<double>(), 1.0, w.p, c->stream), "axpy");
-        for (int j = 0; j <= kk; ++j) H[(size_t)j * m + kk] = h1[j] + h2[j];
         double hn = 0.0;
-        s = norm(w.p, hn);
-        if (s) return s;
+        if (step_blocks > 0) {
+          s = arnoldi(kk, h1, hn);
+          if (s) return s;
+          for (int j = 0; j <= kk; ++j) H[(size_t)j * m + kk] = h1[j];
+        } else {
+          s = dots(V.p, kk + 1, w.p, h1);
+          if (s) return s;
+          CK(cudaMemcpyAsync(c->dots.p, h1.data(), sizeof(double) * 2 * (kk + 1), cudaMemcpyHostToDevice, c->stream),
+             "h2d");
+          CK(launch_multi_axpy<R>(n, kk + 1, V.p, n, c->dots.as<double>(), 1.0, w.p, c->stream), "axpy");
+          s = dots(V.p, kk + 1, w.p, h2);
+          if (s) return s;
+          CK(cudaMemcpyAsync(c->dots.p, h2.data(), sizeof(double) * 2 * (kk + 1), cudaMemcpyHostToDevice, c->stream),
+             "h2d");
+          CK(launch_multi_axpy<R>(n, kk + 1, V.p, n, c->dots.as<double>(), 1.0, w.p, c->stream), "axpy");
+          for (int j = 0; j <= kk; ++j) H[(size_t)j * m + kk] = h1[j] + h2[j];
+          s = norm(w.p, hn);
+          if (s) return s;
+          if (hn > 0.0) CK(launch_axpby<R, R>(n, 1.0 / hn, w.p, 0.0, Vp(kk + 1), c->stream), "normalise");
+        }
         if (!std::isfinite(hn)) return fail(c, CELES_ENUMERIC, "GMRES: non-finite Krylov vector");
         H[(size_t)(kk + 1) * m + kk] = hn;
-        if (hn > 0.0) CK(launch_axpby<R, R>(n, 1.0 / hn, w.p, 0.0, Vp(kk + 1), c->stream), "normalise");
         for (int j = 0; j < kk; ++j) {
           const std::complex<double> a = H[(size_t)j * m + kk], b = H[(size_t)(j + 1) * m + kk];
           H[(size_t)j * m + kk] = cs_c[j] * a + cs_s[j] * b;
@@ -1248,7 +1285,7 @@ struct Bicgstab {
   celes_ctx* c;
   int64_t n;
   bool precond;
-  DevBuf W, z;  // W: 7 vectors [r^ | r | t | s | p | v | u], z: preconditioned work vector
+  DevBuf &W = c->krylov, &z = c->kz;  // W: 7 vectors [r^ | r | t | s | p | v | u], z: preconditioned work vector
   enum { RH = 0, RR = 1, TT = 2, SS = 3, PP = 4, VV = 5, UU = 6 };
   int prec() const { return sizeof(R) == 8 ? CELES_FP64 : CELES_FP32; }
   size_t vbytes() const { return sizeof(R) * 2 * n; }
@@ -1470,7 +1507,23 @@ extern "C" int celes_solve(celes_ctx* c, double tol, const celes_solve_opts* o, 
   int total_its = 0, outer = 0, mv64 = 0, mv32 = 0, guess_used = 0;
   double worst = 0.0;
   int status = CELES_OK;
-  DevBuf r64, d64, r32, d32;
+  // the buffers stay with the context for its next solve up to this size (a solve
+  // of 120 spheres spent 0.15 ms on allocating them)
+  constexpr size_t kKeepSolve = size_t(32) << 20;
+  struct Trim {
+    celes_ctx* c;
+    ~Trim() {
+      DevBuf* all[] = {&c->krylov, &c->kw, &c->kz, &c->kstep, &c->kres, &c->kcor};
+      size_t sum = 0;
+      for (DevBuf* b : all) sum += b->bytes;
+      if (sum > kKeepSolve)
+        for (DevBuf* b : all) b->release();
+    }
+  } trim{c};
+  DevBuf &r64 = c->kres, &d64 = c->kcor;
+  struct {
+    void* p = nullptr;
+  } r32, d32;  // MIXED: the halves of the correction's buffer
   CK(r64.ensure(per64), "residual");
   Inner<double> g64(c, n, opt.restart, use_pc, bicg);
   Inner<float> g32(c, n, opt.restart, use_pc, bicg);
@@ -1481,8 +1534,9 @@ extern "C" int celes_solve(celes_ctx* c, double tol, const celes_solve_opts* o, 
   } else {
     int s = g32.init();
     if (s) return s;
-    CK(r32.ensure(per64 / 2), "residual32");
-    CK(d32.ensure(per64 / 2), "correction32");
+    CK(d64.ensure(per64), "residual32, correction32");
+    d32.p = d64.p;
+    r32.p = d64.as<char>() + per64 / 2;
   }
   for (int rr = 0; rr < c->nrhs; ++rr) {
     double* rhs = reinterpret_cast<double*>(c->rhs.as<char>() + per64 * rr);

@@ -26,33 +26,43 @@ static std::atomic<int64_t> g_launch_count{0};
 void note_launch(int n) { g_launch_count += n; }
 int64_t kernel_launch_count() { return g_launch_count.load(); }
 
+// degree of row r (l^2 - 1 <= r < (l+1)^2 - 1), in integers: a square root would
+// go through the FP64 pipe
 static __device__ __forceinline__ int row_l_rt(int r) {
-  int l = static_cast<int>(sqrt(static_cast<double>(r + 1)));
+  int l = 1;
   while ((l + 1) * (l + 1) - 1 <= r) ++l;
-  while (l * l - 1 > r) --l;
   return l;
 }
 
 // ---------------------------------------------------------------------------
 // coupling epilogue
 // ---------------------------------------------------------------------------
-// grid (blocks, right-hand sides).  ZERO: one slice, zeroed again behind the
+// grid (blocks, right-hand sides).  SPLIT > 1 (many slices on few spheres): that
+// many threads share an element, each adds a run of the slices, and the runs
+// are added in order (FP64, N = 120, 120 slices: 67 -> 15 us).  ZERO: one slice, zeroed again behind the
 // read (each element by the thread that read it) for the next launch that adds
 // into it
-template <typename R, bool ZERO>
-__global__ void coupling_epilogue_kernel(int64_t N, int L, int chunks, Pair2<R>* __restrict__ partial,
-                                         const Pair2<R>* __restrict__ x, const Pair2<R>* __restrict__ tq,
-                                         Pair2<R>* __restrict__ y, int mode) {
+template <typename R, bool ZERO, int SPLIT>
+__global__ void __launch_bounds__(256)
+    coupling_epilogue_kernel(int64_t N, int L, int chunks, Pair2<R>* __restrict__ partial,
+                             const Pair2<R>* __restrict__ x, const Pair2<R>* __restrict__ tq, Pair2<R>* __restrict__ y,
+                             int mode) {
   const int NH = L * (L + 2);
   const int64_t total = N * NH;
   partial += (int64_t)blockIdx.y * chunks * total * 2;
   x += (int64_t)blockIdx.y * total * 2;
   y += (int64_t)blockIdx.y * total * 2;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+  constexpr int PER = 256 / SPLIT;  // elements of a block at a time
+  __shared__ R runs[SPLIT > 1 ? SPLIT : 1][4][PER];
+  const int el = threadIdx.x % PER, part = threadIdx.x / PER;
+  const int c0 = chunks * part / SPLIT, c1 = chunks * (part + 1) / SPLIT;
+  for (int64_t tb = blockIdx.x * (int64_t)PER; tb < total; tb += (int64_t)gridDim.x * PER) {
+    const int64_t t = tb + el;
+    if (SPLIT == 1 && t >= total) break;
     const int64_t i = t / NH;
     const int r = static_cast<int>(t - i * NH);
     R pr = 0, pi = 0, mr = 0, mi = 0;
-    for (int c = 0; c < chunks; ++c) {
+    for (int c = c0; c < (t < total ? c1 : c0); ++c) {
       Pair2<R>* pc = partial + ((int64_t)c * N + i) * (2 * NH);
       const Pair2<R> a = pc[r];
       const Pair2<R> b = pc[NH + r];
@@ -61,6 +71,21 @@ __global__ void coupling_epilogue_kernel(int64_t N, int L, int chunks, Pair2<R>*
       pi += a.im;
       mr += b.re;
       mi += b.im;
+    }
+    if constexpr (SPLIT > 1) {
+      __syncthreads();
+      runs[part][0][el] = pr;
+      runs[part][1][el] = pi;
+      runs[part][2][el] = mr;
+      runs[part][3][el] = mi;
+      __syncthreads();
+      if (part > 0 || t >= total) continue;
+      for (int q = 1; q < SPLIT; ++q) {
+        pr += runs[q][0][el];
+        pi += runs[q][1][el];
+        mr += runs[q][2][el];
+        mi += runs[q][3][el];
+      }
     }
     // y_1 = (y+ + y-)/2, y_2 = (y+ - y-)/2
     Pair2<R> y1{static_cast<R>(0.5) * (pr + mr), static_cast<R>(0.5) * (pi + mi)};
@@ -104,16 +129,18 @@ template <typename R>
 cudaError_t launch_coupling_epilogue(int64_t N, int L, int chunks, void* partial, const void* x, const void* tq,
                                      void* y, int mode, cudaStream_t st, int nrhs, bool zero) {
   const int64_t total = N * L * (L + 2);
-  const int threads = 256;
-  const int64_t blocks = (total + threads - 1) / threads;
+  const bool split = chunks >= 16 && total < 64LL * device_sms() * 32;
+  const int per = split ? 32 : 256;
+  const int64_t blocks = (total + per - 1) / per;
   const int64_t cap = 32LL * device_sms();
   const dim3 grid(static_cast<unsigned>(blocks < cap ? (blocks > 0 ? blocks : 1) : cap), static_cast<unsigned>(nrhs));
   auto* p = static_cast<Pair2<R>*>(partial);
   auto* xv = static_cast<const Pair2<R>*>(x);
   auto* t = static_cast<const Pair2<R>*>(tq);
   auto* yv = static_cast<Pair2<R>*>(y);
-  if (zero && chunks == 1) coupling_epilogue_kernel<R, true><<<grid, threads, 0, st>>>(N, L, 1, p, xv, t, yv, mode);
-  else coupling_epilogue_kernel<R, false><<<grid, threads, 0, st>>>(N, L, chunks, p, xv, t, yv, mode);
+  if (zero && chunks == 1) coupling_epilogue_kernel<R, true, 1><<<grid, 256, 0, st>>>(N, L, 1, p, xv, t, yv, mode);
+  else if (split) coupling_epilogue_kernel<R, false, 8><<<grid, 256, 0, st>>>(N, L, chunks, p, xv, t, yv, mode);
+  else coupling_epilogue_kernel<R, false, 1><<<grid, 256, 0, st>>>(N, L, chunks, p, xv, t, yv, mode);
   note_launch();
   return cudaGetLastError();
 }
@@ -717,6 +744,208 @@ __global__ void __launch_bounds__(kVecThreads) multi_axpy_kernel(int64_t n, int 
     if (two) w[t1] = Pair2<R>{ar1, ai1};
   }
 }
+
+// One Arnoldi step of a short Krylov vector in one cooperative launch: classical
+// Gram-Schmidt of w against V_0 .. V_{nv-1}, twice, the norm and the normalised
+// next vector.  w stays in registers (up to four elements a thread); the dots
+// sum per thread and warp in the vector's precision and per block in FP64, like
+// multi_dotc_kernel, and the blocks' sums are added in order.  Vectors this short
+// (basis in L2) are bound by latency: five barriers here against eight launches,
+// three copies and three host synchronisations (N = 120, lmax 3, refined solve:
+// 5.4 -> 2.8 ms).  CL: up to eight blocks form one cluster and meet at its
+// hardware barrier (23 us a step at n = 3 600, as with fifteen blocks and grid
+// barriers), otherwise a cooperative launch.
+// out: nv coefficients (the sum of both passes), then the squared norm.
+constexpr int kArnoldiElems = 4;
+
+template <typename R, bool CL>
+__global__ void __launch_bounds__(kVecThreads)
+    arnoldi_kernel(int64_t n, int nv, Pair2<R>* __restrict__ V, int64_t ldv, const Pair2<R>* __restrict__ w,
+                   double* __restrict__ partial, double* __restrict__ hbuf, double* __restrict__ out) {
+  constexpr int JT = 16, NW = kVecThreads / 32;
+  namespace cg = cooperative_groups;
+  auto sync = [] {
+    if constexpr (CL) cg::this_cluster().sync();
+    else cg::this_grid().sync();
+  };
+  __shared__ double red[2 * JT][NW];
+  __shared__ R hs[2 * kArnoldiMaxVectors];
+  __shared__ double hd[2 * kArnoldiMaxVectors];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int nb = gridDim.x;
+  const int64_t stride = (int64_t)nb * kVecThreads, t0 = blockIdx.x * (int64_t)kVecThreads + tid;
+  Pair2<R> x[kArnoldiElems];
+#pragma unroll
+  for (int e = 0; e < kArnoldiElems; ++e) x[e] = t0 + e * stride < n ? w[t0 + e * stride] : Pair2<R>{0, 0};
+  // block b's dots conj(U_j) x, j < cnt, into partial[b][j]
+  auto dots = [&](const Pair2<R>* U, int cnt, bool self) {
+    for (int j0 = 0; j0 < cnt; j0 += JT) {
+      const int nj = cnt - j0 < JT ? cnt - j0 : JT;
+      R sr[JT], si[JT];
+#pragma unroll
+      for (int q = 0; q < JT; ++q) sr[q] = si[q] = static_cast<R>(0);
+#pragma unroll
+      for (int e = 0; e < kArnoldiElems; ++e) {
+        const int64_t t = t0 + e * stride;
+        if (t < n) {
+#pragma unroll
+          for (int q = 0; q < JT; ++q) {
+            if (q < nj) {
+              const Pair2<R> a = self ? x[e] : U[(j0 + q) * ldv + t];
+              sr[q] = fma_(a.re, x[e].re, fma_(a.im, x[e].im, sr[q]));
+              si[q] = fma_(a.re, x[e].im, fma_(-a.im, x[e].re, si[q]));
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < JT; ++q) {
+        if (q < nj) {
+          R a = sr[q], b = si[q];
+          for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_down_sync(0xffffffffu, a, o);
+            b += __shfl_down_sync(0xffffffffu, b, o);
+          }
+          if (lane == 0) {
+            red[2 * q][wid] = static_cast<double>(a);
+            red[2 * q + 1][wid] = static_cast<double>(b);
+          }
+        }
+      }
+      __syncthreads();
+      if (tid < 2 * nj) {
+        double s = 0.0;
+        for (int q = 0; q < NW; ++q) s += red[tid][q];
+        partial[((int64_t)blockIdx.x * kArnoldiMaxVectors + j0) * 2 + tid] = s;
+      }
+      __syncthreads();
+    }
+  };
+  // the blocks' sums of dot j, by one warp
+  auto total = [&](int j, double& re, double& im) {
+    re = im = 0.0;
+    for (int b = lane; b < nb; b += 32) {
+      re += __ldcg(partial + ((int64_t)b * kArnoldiMaxVectors + j) * 2);
+      im += __ldcg(partial + ((int64_t)b * kArnoldiMaxVectors + j) * 2 + 1);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      re += __shfl_xor_sync(0xffffffffu, re, o);
+      im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+  };
+  for (int pass = 0; pass < 2; ++pass) {
+    dots(V, nv, false);
+    sync();
+    if (nb <= 16) {
+      // few blocks: every block adds up all dots, one part per thread (a warp per
+      // dot would wait for its loads and FP64 shuffles dot after dot)
+      for (int q = tid; q < 2 * nv; q += kVecThreads) {
+        double sum = 0.0;
+#pragma unroll 8
+        for (int b = 0; b < nb; ++b) sum += __ldcg(partial + (int64_t)b * kArnoldiMaxVectors * 2 + q);
+        hd[q] = sum;
+      }
+    } else {
+      // the dots are dealt to the blocks, one more barrier
+      for (int j = blockIdx.x + nb * wid; j < nv; j += nb * NW) {
+        double re, im;
+        total(j, re, im);
+        if (lane == 0) {
+          hbuf[(pass * kArnoldiMaxVectors + j) * 2] = re;
+          hbuf[(pass * kArnoldiMaxVectors + j) * 2 + 1] = im;
+        }
+      }
+      sync();
+      for (int q = tid; q < 2 * nv; q += kVecThreads) hd[q] = __ldcg(hbuf + pass * kArnoldiMaxVectors * 2 + q);
+    }
+    __syncthreads();
+    for (int q = tid; q < 2 * nv; q += kVecThreads) {
+      hs[q] = static_cast<R>(hd[q]);
+      if (blockIdx.x == 0) out[q] = pass == 0 ? hd[q] : out[q] + hd[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < kArnoldiElems; ++e) {
+      const int64_t t = t0 + e * stride;
+      if (t < n) {
+        R ar = x[e].re, ai = x[e].im;
+#pragma unroll 8
+        for (int j = 0; j < nv; ++j) {
+          const Pair2<R> v = V[j * ldv + t];
+          ar = fma_(-hs[2 * j], v.re, fma_(hs[2 * j + 1], v.im, ar));
+          ai = fma_(-hs[2 * j], v.im, fma_(-hs[2 * j + 1], v.re, ai));
+        }
+        x[e] = Pair2<R>{ar, ai};
+      }
+    }
+    if (nb <= 16) sync();  // every block has read the sums that the next dots overwrite
+  }
+  dots(V, 1, true);
+  sync();
+  double n2, unused;
+  total(0, n2, unused);
+  if (blockIdx.x == 0 && tid == 0) out[2 * nv] = n2;
+  if (n2 > 0.0) {
+    const double a = 1.0 / sqrt(n2);
+    Pair2<R>* next = V + (int64_t)nv * ldv;
+#pragma unroll
+    for (int e = 0; e < kArnoldiElems; ++e) {
+      const int64_t t = t0 + e * stride;
+      if (t < n)
+        next[t] = Pair2<R>{static_cast<R>(a * static_cast<double>(x[e].re)), static_cast<R>(a * static_cast<double>(x[e].im))};
+    }
+  }
+}
+
+// blocks of the one-launch step for vectors of n elements and nv basis vectors; 0: not for these
+int arnoldi_blocks(int64_t n, int max_vectors) {
+  const int64_t b = (n + kVecThreads - 1) / kVecThreads;
+  const int64_t cap = std::min(64, device_sms());
+  if (max_vectors > kArnoldiMaxVectors || n > cap * kVecThreads * kArnoldiElems) return 0;
+  if (n <= 8 * kVecThreads * kArnoldiElems) {  // one cluster: 1, 2, 4 or 8 blocks
+    int c = 1;
+    while (c < 8 && c < b) c *= 2;
+    return c;
+  }
+  return static_cast<int>(std::max<int64_t>(1, std::min(b, cap)));
+}
+size_t arnoldi_scratch_bytes(int blocks) { return sizeof(double) * 2 * kArnoldiMaxVectors * (blocks + 2); }
+
+// V_nv = w orthogonalised against V_0 .. V_{nv-1} and normalised; out (device):
+// 2 nv + 1 doubles.  scratch: arnoldi_scratch_bytes(arnoldi_blocks(n, ..))
+template <typename R>
+cudaError_t launch_arnoldi(int64_t n, int nv, void* V, int64_t ldv, const void* w, void* scratch, double* out,
+                           cudaStream_t st) {
+  const int nb = arnoldi_blocks(n, nv);
+  if (nb < 1) return cudaErrorInvalidValue;
+  auto* Vp = static_cast<Pair2<R>*>(V);
+  auto* wp = static_cast<const Pair2<R>*>(w);
+  double* partial = static_cast<double*>(scratch);
+  double* hbuf = partial + (int64_t)2 * kArnoldiMaxVectors * nb;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(nb));
+  cfg.blockDim = dim3(kVecThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaError_t e;
+  if (nb <= 8) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = static_cast<unsigned>(nb);
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    e = cudaLaunchKernelEx(&cfg, arnoldi_kernel<R, true>, n, nv, Vp, ldv, wp, partial, hbuf, out);
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    e = cudaLaunchKernelEx(&cfg, arnoldi_kernel<R, false>, n, nv, Vp, ldv, wp, partial, hbuf, out);
+  }
+  note_launch();
+  return e;
+}
+template cudaError_t launch_arnoldi<float>(int64_t, int, void*, int64_t, const void*, void*, double*, cudaStream_t);
+template cudaError_t launch_arnoldi<double>(int64_t, int, void*, int64_t, const void*, void*, double*, cudaStream_t);
 
 // y <- beta * y + sum_j c_j V_j    (c given on the device)
 template <typename R>

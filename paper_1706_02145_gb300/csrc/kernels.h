@@ -99,6 +99,13 @@ cudaError_t launch_multi_axpy(int64_t n, int nv, const void* V, int64_t ldv, con
 template <typename R>
 cudaError_t launch_multi_combine(int64_t n, int nv, const void* V, int64_t ldv, const double* c, double beta, void* y,
                                  cudaStream_t st);
+// one Arnoldi step of a short vector in one launch (up to 128 basis vectors)
+constexpr int kArnoldiMaxVectors = 128;
+int arnoldi_blocks(int64_t n, int max_vectors);
+size_t arnoldi_scratch_bytes(int blocks);
+template <typename R>
+cudaError_t launch_arnoldi(int64_t n, int nv, void* V, int64_t ldv, const void* w, void* scratch, double* out,
+                           cudaStream_t st);
 template <typename RX, typename RY>
 cudaError_t launch_axpby(int64_t n, double a, const void* x, double b, void* y, cudaStream_t st);
 // z = a x + b y, complex a = ar + i ai, b = br + i bi (z may alias x or y)
