@@ -71,7 +71,10 @@ typedef struct {
                            shapes and source-chunk counts of the coupling kernel on this problem
                            (cached per device, lmax and size class) and keeps the fastest; it
                            synchronises, so make that first product before any stream capture.
-                           0 (and FP64 always): the built-in shape, about eight waves of chunks */
+                           0 (and FP64 always): the built-in shape, about eight waves of chunks.
+                           The first product of each precision allocates the scratch of all later
+                           ones, whatever their number of right-hand sides; it stays where it is
+                           until celes_destroy, so that captured products stay valid */
   int variant;          /* -1 (default): as autotune decides; 0..7 force the launch shape: bit 0 the
                            FP32 compile-time shape (0 = built-in, 1 = the alternative; FP64 always
                            uses the built-in one), bit 1 the cluster reduction of the partial sums
@@ -178,8 +181,8 @@ int celes_precond_build(celes_ctx* ctx, double cuboid_edge);
 /* Launch shape the context's coupling kernel uses in `precision`: variant
  * (bit 0: alternative FP32 shape; bit 1: cluster reduction of the partial
  * sums; bit 2: reduction in L2, see celes_options.variant), source chunks
- * per product and, if
- * the autotuner chose it, the timed duration of the winning candidate (ms; 0
+ * of a product of one right-hand side (several share launches of fewer chunks
+ * each) and, if the autotuner chose it, the timed duration of the winning candidate (ms; 0
  * otherwise).  CELES_ESTATE before the first coupling product in that
  * precision.  Measurement support; the paper has no counterpart. */
 int celes_coupling_shape(const celes_ctx* ctx, int precision, int* variant, int* chunks, double* ms);

@@ -256,11 +256,13 @@ struct celes_ctx {
   std::vector<celes_incident> incidents;  // descriptors of the current RHS
   DevBuf ain, rhs, b, x0;
   bool has_b = false, has_x0 = false, x0_learned = false;
-  DevBuf partial;
-  // the slice that the in-L2 reduction adds into: zero between products (its
-  // epilogue zeroes what it reads), and used by nothing else
-  DevBuf accum;
-  bool accum_dirty = false;
+  // partial sums of the products per precision (FP64, FP32).  Allocated by the
+  // first product, for any number of right-hand sides, and kept where it is until
+  // the context is destroyed: captured products hold its address.  With the
+  // in-L2 reduction it holds one slice per right-hand side of a launch, zero
+  // between products (the epilogue zeroes what it reads)
+  DevBuf scratch[2];
+  bool accum_dirty = true;
   // preconditioner
   bool has_precond = false;
   int64_t nblocks = 0;
@@ -442,8 +444,9 @@ int autotune(celes_ctx* c, int precision, const void* x, cudaStream_t st) {
       }
     }
     const size_t per = static_cast<size_t>(Nt) * c->nmax * (precision == CELES_FP64 ? 16 : 8);
-    CK(c->partial.ensure(per * (maxsl + 1)), "coupling scratch");
-    char* part = c->partial.as<char>();
+    DevBuf tmp;
+    CK(tmp.ensure(per * (maxsl + 1)), "coupling scratch");
+    char* part = tmp.as<char>();
     char* ytmp = part + per * maxsl;
     cudaEvent_t a = nullptr, b = nullptr;
     CK(cudaEventCreate(&a), "event");
@@ -510,6 +513,59 @@ int prof_begin(celes_ctx* c, cudaStream_t st, celes_ctx::Rec& r, int which) {
   return CELES_OK;
 }
 
+// One launch of the tuned shape over `group` right-hand sides: its source chunks
+// (fewer for each than for one alone, so that the launch keeps its waves) and
+// the slices of partial sums that each leaves.  At least six waves: the tuner
+// times one right-hand side, and two waves of its longer chunks leave the last
+// one half empty (N = 1500, lmax 4, 8 right-hand sides: 1542 us at two or four
+// waves, 1487 at six and more; within 2 % of each other at N = 30 to 2900 else)
+struct GroupPlan {
+  int group, chunks, slices;
+};
+GroupPlan group_plan(const celes_ctx* c, int precision, int group) {
+  const int pi = precision == CELES_FP64 ? 0 : 1, variant = c->tune_variant[pi];
+  const bool rtr = use_rtr(c, precision);
+  GroupPlan g{group, c->tune_chunks[pi], 0};
+  if (group > 1 && c->chunks_opt == 0)
+    g.chunks = chunks_for(c, c->N, precision, variant, std::max(c->tune_waves[pi], 6.0), group);
+  g.slices = rtr ? coupling_rtr_slices_v(c->L, precision, variant, g.chunks) : g.chunks;
+  return g;
+}
+size_t sums_bytes(const celes_ctx* c, int precision) {  // of one slice of one right-hand side
+  return static_cast<size_t>(c->N) * c->nmax * (precision == CELES_FP64 ? 16 : 8);
+}
+// Size of a context's scratch, the same for every number of right-hand sides: what
+// one needs, or, within 64 MB, what a launch over up to eight needs (more spheres
+// than that fill the GPU one right-hand side at a time); 256 KB hold a launch over
+// hundreds for a few spheres
+size_t coupling_scratch_bytes(const celes_ctx* c, int precision) {
+  const size_t per = sums_bytes(c, precision);
+  size_t bytes = std::max(per * group_plan(c, precision, 1).slices, size_t(256) << 10);
+  for (int group = use_rtr(c, precision) ? 8 : 1; group > 1; group /= 2) {
+    const size_t need = per * group_plan(c, precision, group).slices * group;
+    if (need > (size_t(64) << 20)) continue;
+    bytes = std::max(bytes, need);
+    break;
+  }
+  return bytes;
+}
+// the launch over at most `most` right-hand sides that `bytes` of scratch hold,
+// with down to half of the slices that it would like
+GroupPlan fitting_group(const celes_ctx* c, int precision, int most, size_t bytes) {
+  const size_t per = sums_bytes(c, precision);
+  int group = use_rtr(c, precision) ? std::min(most, 256) : 1;
+  for (;; group = (group + 1) / 2) {
+    GroupPlan g = group_plan(c, precision, group);
+    if (group == 1 || per * g.slices * group <= bytes) return g;
+    const size_t fit = bytes / (per * group);
+    const bool clustered = (c->tune_variant[precision == CELES_FP64 ? 0 : 1] & 2) != 0;
+    if (!clustered && c->chunks_opt == 0 && 2 * fit >= static_cast<size_t>(g.slices)) {
+      g.chunks = g.slices = static_cast<int>(fit);
+      return g;
+    }
+  }
+}
+
 int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision, int mode, cudaStream_t st) {
   const int pi = precision == CELES_FP64 ? 0 : 1;
   if (c->tune_chunks[pi] == 0) {
@@ -529,29 +585,31 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
   const int variant = c->tune_variant[pi];
   const bool rtr = use_rtr(c, precision);
   const bool atomic = rtr && rtr_atomic(precision, variant);
-  const size_t elem = precision == CELES_FP64 ? 16 : 8;
-  const size_t per = static_cast<size_t>(c->N) * c->nmax * elem;
+  const size_t per = sums_bytes(c, precision);
+  DevBuf& buf = c->scratch[pi];
+  void* sums = buf.p;
+  size_t bytes = buf.bytes;
+  bool graph_owned = false;
+  if (!sums) {
+    bytes = coupling_scratch_bytes(c, precision);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &capture), "capture status");
+    graph_owned = capture == cudaStreamCaptureStatusActive;
+    if (graph_owned) {
+      // the first product of a precision under capture: scratch of the graph's own
+      CK(cudaMallocAsync(&sums, bytes, st), "coupling scratch");
+    } else {
+      CK(buf.ensure(bytes), "coupling scratch");
+      sums = buf.p;
+    }
+  }
   for (int r = 0; r < nrhs;) {
-    // right-hand sides of one launch (with fewer source chunks each, so that
-    // the launch keeps its waves: N = 777, lmax 5, 8 right-hand sides 1.11 ->
-    // 0.98 ms), as many as keep the partial sums within 1 GB
-    int group = rtr ? std::min(nrhs - r, 256) : 1;
-    int chunks = 0, slices = 0;
-    for (;; group = (group + 1) / 2) {
-      chunks = group == 1 || c->chunks_opt > 0 ? c->tune_chunks[pi]
-                                               : chunks_for(c, c->N, precision, variant, std::max(c->tune_waves[pi], 6.0),
-                                                            group);
-      slices = rtr ? coupling_rtr_slices_v(c->L, precision, variant, chunks) : chunks;
-      if (group == 1 || per * slices * group <= (size_t(1) << 30)) break;
-    }
-    DevBuf& buf = atomic ? c->accum : c->partial;
-    const size_t need = per * slices * group;
-    const bool fresh = need > buf.bytes;
-    CK(buf.ensure(need), "coupling scratch");
-    if (atomic) {
-      if (fresh || c->accum_dirty) CK(cudaMemsetAsync(buf.p, 0, buf.bytes, st), "coupling scratch");
-      c->accum_dirty = true;  // until the epilogue that zeroes it is launched
-    }
+    // right-hand sides of one launch (N = 777, lmax 5, 8 right-hand sides together
+    // 1.11 -> 0.98 ms), as many as the scratch holds the partial sums of
+    const GroupPlan g = fitting_group(c, precision, nrhs - r, bytes);
+    const int group = g.group, chunks = g.chunks, slices = g.slices;
+    if (atomic && (graph_owned || c->accum_dirty)) CK(cudaMemsetAsync(sums, 0, bytes, st), "coupling scratch");
+    if (atomic && !graph_owned) c->accum_dirty = true;  // until the epilogue that zeroes it is launched
     const char* xr = static_cast<const char*>(x) + per * r;
     char* yr = static_cast<char*>(y) + per * r;
     celes_ctx::Rec rec{};
@@ -560,10 +618,10 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
       if (s) return s;
     }
     if (rtr)
-      CK(launch_coupling_rtr_v(c->L, precision, variant, c->N, c->pos.p, xr, buf.p, c->k, chunks, st, group),
+      CK(launch_coupling_rtr_v(c->L, precision, variant, c->N, c->pos.p, xr, sums, c->k, chunks, st, group),
          "coupling kernel");
     else
-      CK(launch_coupling_partial(c->L, precision, c->N, c->pos.p, xr, buf.p, c->k, chunks, st), "coupling kernel");
+      CK(launch_coupling_partial(c->L, precision, c->N, c->pos.p, xr, sums, c->k, chunks, st), "coupling kernel");
     if (c->profiling) {
       CK(cudaEventRecord(rec.b, st), "event");
       c->recs.push_back(rec);
@@ -571,17 +629,18 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
       if (s) return s;
     }
     if (precision == CELES_FP64)
-      CK(launch_coupling_epilogue<double>(c->N, c->L, slices, buf.p, xr, c->tq.p, yr, mode, st, group), "epilogue");
+      CK(launch_coupling_epilogue<double>(c->N, c->L, slices, sums, xr, c->tq.p, yr, mode, st, group), "epilogue");
     else
-      CK(launch_coupling_epilogue<float>(c->N, c->L, slices, buf.p, xr, c->tq32.p, yr, mode, st, group, atomic),
+      CK(launch_coupling_epilogue<float>(c->N, c->L, slices, sums, xr, c->tq32.p, yr, mode, st, group, atomic),
          "epilogue");
-    if (atomic) c->accum_dirty = false;
+    if (atomic && !graph_owned) c->accum_dirty = false;
     if (c->profiling) {
       CK(cudaEventRecord(rec.b, st), "event");
       c->recs.push_back(rec);
     }
     r += group;
   }
+  if (graph_owned) CK(cudaFreeAsync(sums, st), "coupling scratch");
   return CELES_OK;
 }
 
@@ -733,8 +792,7 @@ extern "C" void celes_destroy(celes_ctx* c) {
     c->rhs.release();
     c->b.release();
     c->x0.release();
-    c->partial.release();
-    c->accum.release();
+    for (DevBuf& b : c->scratch) b.release();
     c->work.release();
     c->krylov.release();
     c->kw.release();
