@@ -72,9 +72,9 @@ typedef struct {
                            (cached per device, lmax and size class) and keeps the fastest; it
                            synchronises, so make that first product before any stream capture.
                            0 (and FP64 always): the built-in shape, about eight waves of chunks.
-                           The first product of each precision allocates the scratch of all later
-                           ones, whatever their number of right-hand sides; it stays where it is
-                           until celes_destroy, so that captured products stay valid */
+                           The scratch of the products is allocated by the first one of each
+                           precision, and again by one of more right-hand sides; what a captured
+                           product holds stays valid until celes_destroy */
   int variant;          /* -1 (default): as autotune decides; 0..7 force the launch shape: bit 0 the
                            FP32 compile-time shape (0 = built-in, 1 = the alternative; FP64 always
                            uses the built-in one), bit 1 the cluster reduction of the partial sums

@@ -256,12 +256,15 @@ struct celes_ctx {
   std::vector<celes_incident> incidents;  // descriptors of the current RHS
   DevBuf ain, rhs, b, x0;
   bool has_b = false, has_x0 = false, x0_learned = false;
-  // partial sums of the products per precision (FP64, FP32).  Allocated by the
-  // first product, for any number of right-hand sides, and kept where it is until
-  // the context is destroyed: captured products hold its address.  With the
-  // in-L2 reduction it holds one slice per right-hand side of a launch, zero
-  // between products (the epilogue zeroes what it reads)
+  // partial sums of the products per precision (FP64, FP32).  A product of more
+  // right-hand sides than any before it may take a larger one; the old one is kept
+  // until the context is destroyed (captured products hold its address, and
+  // freeing it would wait for the device).  With the in-L2 reduction it holds one
+  // slice per right-hand side of a launch, zero between products (the epilogue
+  // zeroes what it reads)
   DevBuf scratch[2];
+  std::vector<void*> old_scratch;
+  int scratch_nrhs[2] = {0, 0};  // right-hand sides that it was sized for
   bool accum_dirty = true;
   // preconditioner
   bool has_precond = false;
@@ -534,20 +537,17 @@ GroupPlan group_plan(const celes_ctx* c, int precision, int group) {
 size_t sums_bytes(const celes_ctx* c, int precision) {  // of one slice of one right-hand side
   return static_cast<size_t>(c->N) * c->nmax * (precision == CELES_FP64 ? 16 : 8);
 }
-// Size of a context's scratch, the same for every number of right-hand sides: what
-// one needs, or, within 64 MB, what a launch over up to eight needs (more spheres
-// than that fill the GPU one right-hand side at a time); 256 KB hold a launch over
-// hundreds for a few spheres
-size_t coupling_scratch_bytes(const celes_ctx* c, int precision) {
+// Scratch that a product of nrhs right-hand sides asks for: what one needs, or,
+// within 64 MB, what a launch over as many as possible needs (more spheres than
+// that fill the GPU one right-hand side at a time)
+size_t coupling_scratch_bytes(const celes_ctx* c, int precision, int nrhs) {
   const size_t per = sums_bytes(c, precision);
-  size_t bytes = std::max(per * group_plan(c, precision, 1).slices, size_t(256) << 10);
-  for (int group = use_rtr(c, precision) ? 8 : 1; group > 1; group /= 2) {
+  const size_t one = per * group_plan(c, precision, 1).slices, most = std::max(one, size_t(64) << 20);
+  for (int group = use_rtr(c, precision) ? std::min(nrhs, 256) : 1; group > 1; group = (group + 1) / 2) {
     const size_t need = per * group_plan(c, precision, group).slices * group;
-    if (need > (size_t(64) << 20)) continue;
-    bytes = std::max(bytes, need);
-    break;
+    if (need <= most) return std::max(one, need);
   }
-  return bytes;
+  return one;
 }
 // the launch over at most `most` right-hand sides that `bytes` of scratch hold,
 // with down to half of the slices that it would like
@@ -590,17 +590,32 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
   void* sums = buf.p;
   size_t bytes = buf.bytes;
   bool graph_owned = false;
-  if (!sums) {
-    bytes = coupling_scratch_bytes(c, precision);
+  if (nrhs > c->scratch_nrhs[pi]) {
+    const size_t want = coupling_scratch_bytes(c, precision, nrhs);
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(st, &capture), "capture status");
-    graph_owned = capture == cudaStreamCaptureStatusActive;
+    const bool capturing = capture == cudaStreamCaptureStatusActive;
+    graph_owned = capturing && !sums;
     if (graph_owned) {
       // the first product of a precision under capture: scratch of the graph's own
-      CK(cudaMallocAsync(&sums, bytes, st), "coupling scratch");
-    } else {
-      CK(buf.ensure(bytes), "coupling scratch");
-      sums = buf.p;
+      CK(cudaMallocAsync(&sums, want, st), "coupling scratch");
+      bytes = want;
+    } else if (!capturing && bytes >= want) {
+      c->scratch_nrhs[pi] = nrhs;
+    } else if (!capturing) {  // under capture the launches take what there is
+      const size_t size = std::max(want, 2 * bytes);
+      const cudaError_t e = cudaMalloc(&sums, size);
+      if (e != cudaSuccess && !buf.p) return cuda_fail(c, e, "coupling scratch");
+      if (e != cudaSuccess) {
+        cudaGetLastError();  // narrower launches in the one that is there
+        sums = buf.p;
+      } else {
+        if (buf.p) c->old_scratch.push_back(buf.p);
+        buf.p = sums;
+        bytes = buf.bytes = size;
+        c->scratch_nrhs[pi] = nrhs;
+        if (atomic) c->accum_dirty = true;
+      }
     }
   }
   for (int r = 0; r < nrhs;) {
@@ -793,6 +808,7 @@ extern "C" void celes_destroy(celes_ctx* c) {
     c->b.release();
     c->x0.release();
     for (DevBuf& b : c->scratch) b.release();
+    for (void* p : c->old_scratch) cudaFree(p);
     c->work.release();
     c->krylov.release();
     c->kw.release();
