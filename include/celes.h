@@ -164,7 +164,11 @@ int celes_set_incident(celes_ctx* ctx, const celes_incident* inc, int nrhs);
 /* y = W x (Sec. 2.2, Sec. 3.2.2): y_i = sum_{j != i} W^{ij} x_j for nrhs
  * vectors, blocks evaluated on the fly.  x, y: device pointers to
  * [nrhs][N][nmax] complex128 (CELES_FP64) or complex64 (CELES_FP32); x and y
- * must not overlap. */
+ * must not overlap.  Products of one context (on any stream, replays of captured
+ * ones included) share its scratch: those that overlap on the GPU make each
+ * other's results wrong, though not those of later products; order them.  FP32
+ * products of a context that has been used on one stream only save the launch
+ * that clears the scratch. */
 int celes_coupling_matvec(celes_ctx* ctx, const void* x, void* y, int nrhs, int precision, void* stream);
 
 /* y = M x = x - T (W x) (Sec. 2.2, Eq. for M): the coupling matvec with the

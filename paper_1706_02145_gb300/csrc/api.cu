@@ -260,12 +260,17 @@ struct celes_ctx {
   // right-hand sides than any before it may take a larger one; the old one is kept
   // until the context is destroyed (captured products hold its address, and
   // freeing it would wait for the device).  With the in-L2 reduction it holds one
-  // slice per right-hand side of a launch, zero between products (the epilogue
-  // zeroes what it reads)
+  // slice per right-hand side of a launch, zero between products: the epilogue
+  // zeroes what it reads.  Products that overlap (several streams, replays of
+  // captured ones) could leave something there; a context that has seen a second
+  // stream or a capture zeroes it before every product instead, so that no later
+  // product is wrong
   DevBuf scratch[2];
   std::vector<void*> old_scratch;
   int scratch_nrhs[2] = {0, 0};  // right-hand sides that it was sized for
   bool accum_dirty = true;
+  bool one_stream = true;                 // no second stream, no capture so far
+  unsigned long long product_stream = 0;  // id of the first product's stream
   // preconditioner
   bool has_precond = false;
   int64_t nblocks = 0;
@@ -589,12 +594,22 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
   DevBuf& buf = c->scratch[pi];
   void* sums = buf.p;
   size_t bytes = buf.bytes;
-  bool graph_owned = false;
+  bool graph_owned = false, capturing = false;
+  if (nrhs > c->scratch_nrhs[pi] || atomic) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &status), "capture status");
+    capturing = status == cudaStreamCaptureStatusActive;
+  }
+  if (capturing) {
+    c->one_stream = false;
+  } else if (atomic && c->one_stream) {
+    unsigned long long id = 0;
+    CK(cudaStreamGetId(st, &id), "stream id");  // not to be asked for under capture
+    if (c->product_stream == 0) c->product_stream = id;
+    c->one_stream = id == c->product_stream;
+  }
   if (nrhs > c->scratch_nrhs[pi]) {
     const size_t want = coupling_scratch_bytes(c, precision, nrhs);
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    CK(cudaStreamIsCapturing(st, &capture), "capture status");
-    const bool capturing = capture == cudaStreamCaptureStatusActive;
     graph_owned = capturing && !sums;
     if (graph_owned) {
       // the first product of a precision under capture: scratch of the graph's own
@@ -623,8 +638,9 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
     // 1.11 -> 0.98 ms), as many as the scratch holds the partial sums of
     const GroupPlan g = fitting_group(c, precision, nrhs - r, bytes);
     const int group = g.group, chunks = g.chunks, slices = g.slices;
-    if (atomic && (graph_owned || c->accum_dirty)) CK(cudaMemsetAsync(sums, 0, bytes, st), "coupling scratch");
-    if (atomic && !graph_owned) c->accum_dirty = true;  // until the epilogue that zeroes it is launched
+    if (atomic && (c->one_stream ? c->accum_dirty : r == 0))
+      CK(cudaMemsetAsync(sums, 0, c->one_stream ? bytes : per * group, st), "coupling scratch");
+    if (atomic && !capturing) c->accum_dirty = true;  // until the epilogue that zeroes it is launched
     const char* xr = static_cast<const char*>(x) + per * r;
     char* yr = static_cast<char*>(y) + per * r;
     celes_ctx::Rec rec{};
@@ -648,7 +664,7 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
     else
       CK(launch_coupling_epilogue<float>(c->N, c->L, slices, sums, xr, c->tq32.p, yr, mode, st, group, atomic),
          "epilogue");
-    if (atomic && !graph_owned) c->accum_dirty = false;
+    if (atomic && !capturing) c->accum_dirty = false;
     if (c->profiling) {
       CK(cudaEventRecord(rec.b, st), "event");
       c->recs.push_back(rec);

@@ -109,3 +109,32 @@ def test_products_of_several_launches(N, L, nrhs, variant):
                 s.product(n, precision, dtype, tol)
     finally:
         B.celes_destroy(s.ctx)
+
+
+@pytest.mark.parametrize("variant", [-1, 0, 4, 5])
+def test_products_and_replays_on_several_streams(variant):
+    # ordered by events; the scratch is cleared by the epilogues, by the products or by the graph
+    s = Scene(300, 3, 8, variant=variant)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    try:
+        for precision, dtype, tol in PRECISIONS:
+            s.product(1, precision, dtype, tol)
+            graph, yg = captured(s, 3, precision, dtype)
+            work = [(streams[q % 3], nrhs, *s.vectors(nrhs, dtype)) for q, nrhs in enumerate((1, 8, 1, 8, 8, 1, 1, 3))]
+            torch.cuda.synchronize()
+            last = None
+            for q in range(40):
+                stream, nrhs, x, y = work[q % len(work)]
+                if last is not None:
+                    stream.wait_stream(last)
+                if q % 5 == 4:
+                    with torch.cuda.stream(stream):
+                        graph.replay()
+                B.celes_master_matvec(s.ctx, x, y, nrhs, precision, stream=stream)
+                last = stream
+            for y in [w[3] for w in work] + [yg]:
+                s.check(y, tol)
+            s.product(8, precision, dtype, tol)
+    finally:
+        torch.cuda.synchronize()
+        B.celes_destroy(s.ctx)
