@@ -1098,6 +1098,12 @@ template cudaError_t launch_nonfinite<double>(int64_t, const void*, int*, cudaSt
 // 26 instructions per (direction, sphere); one CTA per direction contracting
 // with both B_nj per sphere took 8 FMAs and a full sincos.  GB300, 10 000
 // spheres, lmax 4, 2 048 directions: 23.8 -> 6.1 ms.
+// Its error is that of k.r, as long as that is summed like x and y first, then z
+// (packings are centred in x and y: 1.2 times the error with z first), and no
+// running sum is long: one takes every eighth or fourth sphere of a chunk (256
+// spheres where there are many directions), then 16 chunks.  653 spheres, lmax 5, 221
+// directions, against 64 bits: 1.05e-15 with one running sum per chunk and z
+// first, 8.0e-16 so, 7.8e-16 with one CTA per direction (10 000 spheres: 7.3e-15).
 // ---------------------------------------------------------------------------
 constexpr int kFfTile = 8;      // spheres staged at a time
 constexpr int kFfThreads = 256;
@@ -1126,8 +1132,42 @@ __global__ void __launch_bounds__(kFfThreads)
     kv[tid][1] = k * sb * sa;
     kv[tid][2] = k * cb;
   }
-  // products P1 = c br, P2 = s bi, P3 = (c + s)(br + bi) of the phase c + i s
-  double p1[DT][NPT] = {}, p2[DT][NPT] = {}, p3[DT][NPT] = {};
+  // products P1 = c br, P2 = s bi, P3 = (c + s)(br + bi) of the phase c + i s, in NC
+  // running sums that take the spheres in turn; with 64 directions, whose registers
+  // are full, in one of at most 256 spheres, added up in F
+  constexpr int NC = DT > 1 ? 1 : (NPT == 2 || NPT == 3 ? 8 : 4), kRun = 256;
+  double p1[NC][DT][NPT] = {}, p2[NC][DT][NPT] = {}, p3[NC][DT][NPT] = {};
+  bool stored = false;
+  auto store = [&] {
+#pragma unroll
+    for (int a = 0; a < DT; ++a) {
+      const int64_t d = d0 + DT * ty + a;
+#pragma unroll
+      for (int u = 0; u < NPT; ++u) {
+#pragma unroll
+        for (int w = NC / 2; w > 0; w /= 2) {
+#pragma unroll
+          for (int q = 0; q < w; ++q) {
+            p1[q][a][u] += p1[q + w][a][u];
+            p2[q][a][u] += p2[q + w][a][u];
+            p3[q][a][u] += p3[q + w][a][u];
+          }
+        }
+        const int n = tx + 16 * u;
+        if (d < Nd && n < nmax) {
+          double2& f = F[((int64_t)blockIdx.y * Nd + d) * nmax + n];
+          double2 v = make_double2(p1[0][a][u] - p2[0][a][u], p3[0][a][u] - p1[0][a][u] - p2[0][a][u]);
+          if (stored) {
+            v.x += f.x;
+            v.y += f.y;
+          }
+          f = v;
+        }
+        p1[0][a][u] = p2[0][a][u] = p3[0][a][u] = 0.0;
+      }
+    }
+    stored = true;
+  };
   const int64_t i0 = blockIdx.y * chunk, i1 = i0 + chunk < N ? i0 + chunk : N;
   for (int64_t it = i0; it < i1; it += kFfTile) {
     const int ni = static_cast<int>(i1 - it < kFfTile ? i1 - it : kFfTile);
@@ -1137,7 +1177,7 @@ __global__ void __launch_bounds__(kFfThreads)
       double s = 0.0, c = 0.0;
       if (j < ni) {
         const Pos4 r = pos[it + j];
-        sincos_phase(-fma(kv[d][0], r.x, fma(kv[d][1], r.y, kv[d][2] * r.z)), &s, &c);
+        sincos_phase(-fma(kv[d][2], r.z, fma(kv[d][0], r.x, kv[d][1] * r.y)), &s, &c);
       }
       pc[j][d] = c;
       ps[j][d] = s;
@@ -1151,31 +1191,23 @@ __global__ void __launch_bounds__(kFfThreads)
       bt[j][n] = v.x + v.y;
     }
     __syncthreads();
-#pragma unroll 2
+#pragma unroll(NC > 1 ? kFfTile : 2)
     for (int j = 0; j < kFfTile; ++j) {
+      const int q = j % NC;
 #pragma unroll
       for (int u = 0; u < NPT; ++u) {
         const double vr = br[j][tx + 16 * u], vi = bi[j][tx + 16 * u], vt = bt[j][tx + 16 * u];
 #pragma unroll
         for (int a = 0; a < DT; ++a) {
-          p1[a][u] = fma(pc[j][DT * ty + a], vr, p1[a][u]);
-          p2[a][u] = fma(ps[j][DT * ty + a], vi, p2[a][u]);
-          p3[a][u] = fma(pt[j][DT * ty + a], vt, p3[a][u]);
+          p1[q][a][u] = fma(pc[j][DT * ty + a], vr, p1[q][a][u]);
+          p2[q][a][u] = fma(ps[j][DT * ty + a], vi, p2[q][a][u]);
+          p3[q][a][u] = fma(pt[j][DT * ty + a], vt, p3[q][a][u]);
         }
       }
     }
+    if (DT > 1 && (it + kFfTile - i0) % kRun == 0 && it + kFfTile < i1) store();
   }
-#pragma unroll
-  for (int a = 0; a < DT; ++a) {
-    const int64_t d = d0 + DT * ty + a;
-#pragma unroll
-    for (int u = 0; u < NPT; ++u) {
-      const int n = tx + 16 * u;
-      if (d < Nd && n < nmax)
-        F[((int64_t)blockIdx.y * Nd + d) * nmax + n] =
-            make_double2(p1[a][u] - p2[a][u], p3[a][u] - p1[a][u] - p2[a][u]);
-    }
-  }
+  store();
 }
 
 // constants of the recursions of pi_l^m (pi_tau_m in cmath.cuh), for one m per thread
@@ -1234,16 +1266,22 @@ __global__ void __launch_bounds__(128)
       // sums over the chunks of the rows (tau 1, 2) of +m and -m
       cd f[4] = {};
       const int r = l * (l + 1) - 1;
-      for (int c = 0; c < chunks; ++c) {
-        const double2* Fc = F + ((int64_t)c * Nd + d) * nmax;
-        const double2 v0 = Fc[r + am], v1 = Fc[NH + r + am];
-        f[0] = f[0] + cd{v0.x, v0.y};
-        f[1] = f[1] + cd{v1.x, v1.y};
-        if (am > 0) {
-          const double2 w0 = Fc[r - am], w1 = Fc[NH + r - am];
-          f[2] = f[2] + cd{w0.x, w0.y};
-          f[3] = f[3] + cd{w1.x, w1.y};
+      for (int c0 = 0; c0 < chunks; c0 += 16) {
+        cd h[4] = {};
+        const int c1 = chunks < c0 + 16 ? chunks : c0 + 16;
+        for (int c = c0; c < c1; ++c) {
+          const double2* Fc = F + ((int64_t)c * Nd + d) * nmax;
+          const double2 v0 = Fc[r + am], v1 = Fc[NH + r + am];
+          h[0] = h[0] + cd{v0.x, v0.y};
+          h[1] = h[1] + cd{v1.x, v1.y};
+          if (am > 0) {
+            const double2 w0 = Fc[r - am], w1 = Fc[NH + r - am];
+            h[2] = h[2] + cd{w0.x, w0.y};
+            h[3] = h[3] + cd{w1.x, w1.y};
+          }
         }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) f[q] = f[q] + h[q];
       }
       // B_n1 = -(1/i^{l+1}) norm i ang, B_n2 = -(1/i^{l+1}) norm ang; ang = tau for j = tau index, else m pi
       const cd a = em * f[0], b = em * f[1], c = conj(em) * f[2], e = conj(em) * f[3];
