@@ -322,11 +322,11 @@ __global__ void gaussian_table_kernel(int nb, int L, double k, double w, const d
 
 // J_0 .. J_M at x >= 0: Miller's downward recurrence with sum J_0 + 2 J_2 + 2
 // J_4 + .. = 1 below 8 (from order 34, or 16 below 1: what is left out is under
-// 1e-17 of J_M), the leading term below 1e-6, else j0, j1 and the upward
-// recurrence, which is stable for orders below x
+// 1e-17 of J_M), the leading terms below 1e-8 (the next one of J_0 is x^2 / 4),
+// else j0, j1 and the upward recurrence, which is stable for orders below x
 template <int M>
 __device__ __forceinline__ void bessel_orders(double x, double (&J)[M + 1]) {
-  if (x < 1e-6) {
+  if (x < 1e-8) {
     J[0] = 1.0;
 #pragma unroll
     for (int n = 1; n <= M; ++n) J[n] = J[n - 1] * (0.5 * x / n);
