@@ -1356,11 +1356,13 @@ cudaError_t launch_farfield(int64_t N, int L, double k, const void* pos, const d
 // overlap check: flag[0] = 1 if some pair overlaps (|r_i - r_j| < R_i + R_j).
 // Every pair in FP32 relative to the first sphere, widened by a bound on the
 // rounding of both coordinates; only pairs that this cannot clear (neighbours,
-// and anything not finite in FP32) are tested in FP64.  Grid (row tiles,
+// lengths whose squares leave FP32's range) are tested in FP64.  Grid (row tiles,
 // column tiles), upper triangle; one thread per row against a staged tile.
 // (10 000 spheres: 4.7 ms with one FP64 thread per sphere over all later ones,
 // 0.03 ms so.)
 constexpr int kOvTile = 256;
+// squares below this lose digits to FP32's least exponent (the test in FP64 takes those pairs)
+constexpr float kOvTiny = 1e-32f;
 
 __global__ void __launch_bounds__(kOvTile)
     overlap_kernel(int64_t N, int64_t y0, const Pos4* __restrict__ pos, const double* __restrict__ radii,
@@ -1396,7 +1398,7 @@ __global__ void __launch_bounds__(kOvTile)
       const float4 q = sp[jb + u];
       const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
       const float s = (p.w + q.w) + 2.0f * (e + se[jb + u]);
-      near |= (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > s * s ? 0u : 1u) << u;
+      near |= (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > fmaf(s, s, kOvTiny) ? 0u : 1u) << u;
     }
     if (nj - jb < 32) near &= (1u << (nj - jb)) - 1u;
     while (near) {
