@@ -286,8 +286,9 @@ struct celes_ctx {
   // buffers of one solve, kept for the next (at most kKeepSolve bytes in all):
   // Krylov vectors, two work vectors, Arnoldi step, residual and correction
   DevBuf krylov, kw, kz, kstep, kres, kcor;
-  // buffers of one field evaluation, kept for the next (at most kKeepWorkspace bytes)
+  // buffers of one field evaluation, kept for the next (FieldWorkspace)
   DevBuf work;
+  std::mutex work_mutex;
   std::string err;
   // kernel timing (celes_profile)
   bool profiling = false;
@@ -325,21 +326,6 @@ int cuda_fail(celes_ctx* c, cudaError_t e, const char* what) {
 }
 
 int ck_status(celes_ctx* c, cudaError_t e, const char* what) { return e == cudaSuccess ? CELES_OK : cuda_fail(c, e, what); }
-
-// A context's field workspace for one call: an allocation of some MB costs
-// more than a small field evaluation (far field of 114 spheres in 399 directions:
-// 226 -> 88 us), so what a call needed is kept up to this size.  Calls
-// end with their stream synchronised.
-constexpr size_t kKeepWorkspace = size_t(80) << 20;
-struct Workspace {
-  celes_ctx* c;
-  explicit Workspace(celes_ctx* ctx) : c(ctx) {}
-  ~Workspace() {
-    if (c->work.bytes > kKeepWorkspace) c->work.release();
-  }
-  cudaError_t ensure(size_t bytes) { return c->work.ensure(bytes); }
-  char* at(size_t offset) const { return c->work.as<char>() + offset; }
-};
 
 // CK(expression returning cudaError_t, "what"): return a celes_status on error
 #define CK(...)                                   \
@@ -1526,14 +1512,14 @@ int ctx_view(celes_ctx* c, CtxView* v) {
   return CELES_OK;
 }
 
-cudaError_t ctx_workspace(celes_ctx* c, size_t bytes, void** p) {
-  const cudaError_t e = c->work.ensure(bytes);
-  *p = c->work.p;
-  return e;
+constexpr size_t kKeepWorkspace = size_t(80) << 20;
+FieldWorkspace::FieldWorkspace(celes_ctx* ctx) : c_(ctx) { c_->work_mutex.lock(); }
+FieldWorkspace::~FieldWorkspace() {
+  if (c_->work.bytes > kKeepWorkspace) c_->work.release();
+  c_->work_mutex.unlock();
 }
-void ctx_workspace_done(celes_ctx* c) {
-  if (c->work.bytes > kKeepWorkspace) c->work.release();
-}
+cudaError_t FieldWorkspace::ensure(size_t bytes) { return c_->work.ensure(bytes); }
+char* FieldWorkspace::at(size_t offset) const { return c_->work.as<char>() + offset; }
 
 int ctx_mark_solved(celes_ctx* c) {
   if (!c || c->nrhs < 1) return CELES_EINVAL;
@@ -1817,7 +1803,7 @@ extern "C" int celes_farfield(celes_ctx* c, const double* dirs, int64_t Nd, doub
   DeviceGuard dg(c->device);
   // directions, amplitudes, sums
   const size_t dir_bytes = (sizeof(double) * 2 * Nd + 255) / 256 * 256, g_bytes = (sizeof(double) * 4 * Nd + 255) / 256 * 256;
-  Workspace ws(c);
+  FieldWorkspace ws(c);
   CK(ws.ensure(dir_bytes + g_bytes + farfield_scratch_bytes(c->N, c->L, Nd)), "far field");
   double* dd = reinterpret_cast<double*>(ws.at(0));
   double* gd = reinterpret_cast<double*>(ws.at(dir_bytes));

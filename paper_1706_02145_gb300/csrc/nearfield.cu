@@ -529,20 +529,17 @@ extern "C" int celes_nearfield(celes_ctx* ctx, const double* points, int64_t Np,
   // points, field, the beam's nodes and weights, slices
   const int nb_max = v.incidents[rhs].kind == CELES_PLANE_WAVE ? 0 : (v.incidents[rhs].n_beta > 0 ? v.incidents[rhs].n_beta : 128);
   const size_t slices = what != 1 && chunks > 1 ? static_cast<size_t>(chunks) * 6 * Np : 0;
-  void* ws = nullptr;
-  if (ctx_workspace(ctx, sizeof(double) * (9 * static_cast<size_t>(Np) + 2 * nb_max + slices), &ws) != cudaSuccess) {
+  FieldWorkspace ws(ctx);
+  if (ws.ensure(sizeof(double) * (9 * static_cast<size_t>(Np) + 2 * nb_max + slices)) != cudaSuccess) {
     cudaGetLastError();
     return CELES_ENOMEM;
   }
-  double* dp = static_cast<double*>(ws);
+  double* dp = reinterpret_cast<double*>(ws.at(0));
   double* dE = dp + 3 * Np;
   double* dn = dE + 6 * Np;
   double* dw = dn + nb_max;
   double* dS = dw + nb_max;
-  auto cleanup = [&]() {
-    cudaStreamSynchronize(st);
-    ctx_workspace_done(ctx);
-  };
+  auto cleanup = [&]() { cudaStreamSynchronize(st); };
   cudaError_t e = cudaMemcpyAsync(dp, points, sizeof(double) * 3 * Np, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && what == 1) e = cudaMemsetAsync(dE, 0, sizeof(double) * 6 * Np, st);
   if (e != cudaSuccess) {
