@@ -754,9 +754,11 @@ __global__ void __launch_bounds__(kVecThreads) multi_axpy_kernel(int64_t n, int 
 // three copies and three host synchronisations (N = 120, lmax 3, refined solve:
 // 5.4 -> 2.8 ms).  CL: up to eight blocks form one cluster and meet at its
 // hardware barrier (23 us a step at n = 3 600, as with fifteen blocks and grid
-// barriers), otherwise a cooperative launch.
+// barriers); otherwise a cooperative launch of 33 to 64 blocks, which deals the
+// dots out.
 // out: nv coefficients (the sum of both passes), then the squared norm.
 constexpr int kArnoldiElems = 4;
+constexpr int kArnoldiCluster = 8;
 
 template <typename R, bool CL>
 __global__ void __launch_bounds__(kVecThreads)
@@ -836,7 +838,10 @@ __global__ void __launch_bounds__(kVecThreads)
   for (int pass = 0; pass < 2; ++pass) {
     dots(V, nv, false);
     sync();
-    if (nb <= 16) {
+    // (a cluster never has more than 16 blocks; asked all the same, since with CL alone
+    // the compiler takes 76 registers instead of 64, and a refined solve of 120
+    // spheres 2.80 instead of 2.71 ms)
+    if (CL && nb <= 16) {
       // few blocks: every block adds up all dots, one part per thread (a warp per
       // dot would wait for its loads and FP64 shuffles dot after dot)
       for (int q = tid; q < 2 * nv; q += kVecThreads) {
@@ -846,7 +851,8 @@ __global__ void __launch_bounds__(kVecThreads)
         hd[q] = sum;
       }
     } else {
-      // the dots are dealt to the blocks, one more barrier
+      // the dots are dealt to the blocks; the barrier after them also lets the next
+      // ones overwrite the sums
       for (int j = blockIdx.x + nb * wid; j < nv; j += nb * NW) {
         double re, im;
         total(j, re, im);
@@ -878,7 +884,7 @@ __global__ void __launch_bounds__(kVecThreads)
         x[e] = Pair2<R>{ar, ai};
       }
     }
-    if (nb <= 16) sync();  // every block has read the sums that the next dots overwrite
+    if (CL && nb <= 16) sync();  // every block has read the sums that the next dots overwrite
   }
   dots(V, 1, true);
   sync();
@@ -902,9 +908,9 @@ int arnoldi_blocks(int64_t n, int max_vectors) {
   const int64_t b = (n + kVecThreads - 1) / kVecThreads;
   const int64_t cap = std::min(64, device_sms());
   if (max_vectors > kArnoldiMaxVectors || n > cap * kVecThreads * kArnoldiElems) return 0;
-  if (n <= 8 * kVecThreads * kArnoldiElems) {  // one cluster: 1, 2, 4 or 8 blocks
+  if (n <= kArnoldiCluster * kVecThreads * kArnoldiElems) {  // one cluster: 1, 2, 4 or 8 blocks
     int c = 1;
-    while (c < 8 && c < b) c *= 2;
+    while (c < kArnoldiCluster && c < b) c *= 2;
     return c;
   }
   return static_cast<int>(std::max<int64_t>(1, std::min(b, cap)));
@@ -930,7 +936,7 @@ cudaError_t launch_arnoldi(int64_t n, int nv, void* V, int64_t ldv, const void* 
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cudaError_t e;
-  if (nb <= 8) {
+  if (nb <= kArnoldiCluster) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = static_cast<unsigned>(nb);
     at[0].val.clusterDim.y = 1;
