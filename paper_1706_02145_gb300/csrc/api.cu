@@ -270,7 +270,7 @@ struct celes_ctx {
   int scratch_nrhs[2] = {0, 0};  // right-hand sides that it was sized for
   bool accum_dirty = true;
   bool one_stream = true;                 // no second stream, no capture so far
-  unsigned long long product_stream = 0;  // id of the first product's stream
+  unsigned long long product_stream = ~0ull;  // id of the first product's stream
   // preconditioner
   bool has_precond = false;
   int64_t nblocks = 0;
@@ -591,7 +591,7 @@ int coupling_apply(celes_ctx* c, const void* x, void* y, int nrhs, int precision
   } else if (atomic && c->one_stream) {
     unsigned long long id = 0;
     CK(cudaStreamGetId(st, &id), "stream id");  // not to be asked for under capture
-    if (c->product_stream == 0) c->product_stream = id;
+    if (c->product_stream == ~0ull) c->product_stream = id;
     c->one_stream = id == c->product_stream;
   }
   if (nrhs > c->scratch_nrhs[pi]) {
