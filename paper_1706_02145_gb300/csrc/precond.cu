@@ -952,7 +952,7 @@ __device__ __forceinline__ Pair2<double> load_stream(const Pair2<double>* p) {
 // laid end to end and cut into equal runs, one per warp, sixteen columns in
 // flight each: with whole tiles per warp the longest row of a block set the time
 // and half of the bandwidth was left (245 blocks of up to 810 unknowns, FP32:
-// 237 -> 140 us).  A tile cut between warps is added up from their
+// 237 -> 144 us).  A tile cut between warps is added up from their
 // pieces in order, so results do not depend on timing.  Every CTA gathers the
 // whole (pivot-permuted) block vector.
 template <typename R, typename F>

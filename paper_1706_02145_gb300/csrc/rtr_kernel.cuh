@@ -24,7 +24,7 @@
 // entries of the rotation blocks need no half-angle powers.  Measured on
 // GB300, master product, before -> after: FP32 N = 10 000 lmax 4 9.87 -> 7.71
 // ms (error against 64 bits 6.0e-7 -> 3.2e-7), N = 777 lmax 5 with 8 right-hand
-// sides 2.27 -> 1.11 ms, N = 100 000 lmax 3 492 -> 395 ms; FP64 N = 2001 lmax 4
+// sides 2.27 -> 1.11 ms, N = 100 000 lmax 3 492 -> 404 ms; FP64 N = 2001 lmax 4
 // 22.9 -> 17.5 ms (16.9 ms with the shape below).
 #pragma once
 
@@ -368,7 +368,7 @@ __device__ __forceinline__ void ax_entry(const Hankel<L, R>& h, R& ar, R& ai, R&
 
 // The axial products of mu > 0 on the packed FMA as well, both sums of one
 // factor together: at lmax 4 the scalar half of the FP32 lanes is the fuller
-// one without it (N = 10 000: 7.84 -> 7.68 ms; 1.77 -> 1.83 ms at lmax 2, 395 ->
+// one without it (N = 10 000: 7.84 -> 7.68 ms; 1.77 -> 1.83 ms at lmax 2, 403 ->
 // 407 ms at N = 100 000 and lmax 3, 16.4 -> 16.5 ms at lmax 5)
 template <int L, typename R>
 constexpr bool kPackedAxial = sizeof(R) == 4 && L == 4;
